@@ -21,7 +21,13 @@
 //   warp 16     loads the binary16 activation tile with the tensor-memory
 //               accelerator (TMA; one box of 64 features x 128 tokens in the
 //               128-byte swizzled layout, zero fill outside the matrix);
-//   warp 17     owns the TMEM allocation; its lane 0 issues the MMAs;
+//   warp 17     owns the TMEM allocation; one elected lane issues the MMAs.
+//               The lane is chosen by elect.sync: behind `lane == 0` each
+//               tcgen05.mma took ~100 ns to issue whatever its N, longer than
+//               the 62 ns the tensor pipe needs for one of 128 x 256 x 16, so
+//               the issuing thread bounded the main loop (a layer of d 5120,
+//               inter 17408 at 512 tokens: 327 us, with elect.sync 282 us; of
+//               d 2560, inter 9728 at 3001 tokens: 512 us, now 454 us);
 //   warp 18     loads the packed codes and scales/zeros of the CTA's 8 row
 //               tiles (TMA, one box each per projection and block) into their
 //               own ring.
@@ -454,14 +460,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
     if (*sm.abort_s) return false;
     if (mbar_wait_sleep(bar, parity)) return true;
     *sm.abort_s = 1;
-    if (lane == 0) gemm_timeout();
+    gemm_timeout();
     return false;
   };
 
   if (warp == kRawWarp) {
     // ---- packed codes and scales/zeros (TMA) into their ring; row tiles
     // past the matrix read as zeros ----
-    if (lane == 0)
+    if (elect_one())
       for (int it = 0; it < KB; ++it) {
         const int q = it % R;
         if (it >= R && !wait(&sm.raw_empty[q], (it / R - 1) & 1)) break;
@@ -492,7 +498,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
     }
   } else if (warp == kMmaWarp) {
     // ---- MMA issue ----
-    if (lane == 0) {
+    if (elect_one()) {
       for (int it = 0; it < nit; ++it) {
         const int sa = it % SA, sb = it % SB;
         if (!wait(&sm.a_full[sa], (it / SA) & 1) || !wait(&sm.b_full[sb], (it / SB) & 1)) break;
@@ -690,7 +696,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
     if (*sm.abort_s) return false;
     if (mbar_wait_sleep(bar, parity)) return true;
     *sm.abort_s = 1;
-    if (lane == 0) gemm_timeout();
+    gemm_timeout();
     return false;
   };
   // The parts of tiles in this CTA's range, in order: tile, units [ub, ue),
@@ -706,7 +712,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
   auto halves = [&](int m0) { return min(a.mt, (a.M - m0 + kBM - 1) / kBM); };
 
   if (warp == kRawWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       int gr = 0;  // blocks loaded so far
       bool ok = true;
       WQ_FOR_EACH_PART {
@@ -753,7 +759,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
       }
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       int gs = 0;
       bool ok = true;
       WQ_FOR_EACH_PART {
@@ -1169,12 +1175,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_swap_kernel(const GemmA
     if (*sm.abort_s) return false;
     if (mbar_wait_sleep(bar, parity)) return true;
     *sm.abort_s = 1;
-    if (lane == 0) gemm_timeout();
+    gemm_timeout();
     return false;
   };
 
   if (warp == kRawWarp) {
-    if (lane == 0)
+    if (elect_one())
       for (int it = 0; it < kb1 - kb0; ++it) {
         const int q = it % R;
         if (it >= R && !wait(&sm.raw_empty[q], (it / R - 1) & 1)) break;
@@ -1202,7 +1208,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_swap_kernel(const GemmA
       }
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       for (int it = 0; it < nit; ++it) {
         const int sa = it % SA, sb = it % SB;
         if (!wait(&sm.a_full[sa], (it / SA) & 1) || !wait(&sm.b_full[sb], (it / SB) & 1)) break;

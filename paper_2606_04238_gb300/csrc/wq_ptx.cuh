@@ -164,6 +164,15 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_
                : "memory");
 }
 
+// True in one lane of a converged warp (the same one every time).  Used where
+// one thread issues tcgen05.mma or TMA instructions: elect.sync tells the
+// compiler that a single lane is active, which `lane == 0` does not.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ uint32_t lds32(const void *p) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_addr(p)));
