@@ -22,16 +22,15 @@
  *   - Supported: group in {32, 64, 128}; in-features a multiple of the group
  *     (WQ_ERR_SHAPE otherwise); 1 <= m <= 16384 tokens (m == 0 is a no-op);
  *     LoRA rank r a multiple of 8, r <= 64 (r == 0: no adapter).
- *   - Two paths behind the same calls: up to 16 tokens (8 for layers of
- *     hidden size d >= 4096) the dequant-GEMV kernels (exact products of the
- *     codes and binary16 activations on the mma.sync tensor-core path, fp32
- *     sums); above that, and for a layer
- *     shape the GEMV kernels have no launch configuration for at the given
- *     token count, the batched dequant-GEMM on the tcgen05 tensor cores
- *     (activations and each dequantized weight s (q - z) rounded once to
- *     binary16, fp32 accumulation; with fp32 output of wq_down_w4 the weights
- *     enter as two exact binary16 parts).  The workspace size covers the path
- *     a call takes.
+ *   - Three paths behind the same calls: up to 8 tokens the dequant-GEMV
+ *     kernels, up to 64 tokens (and below, for a layer shape the GEMV kernels
+ *     have no launch configuration for) the batched-decode kernels -- both
+ *     form exact products of the codes and binary16 activations on the
+ *     mma.sync tensor-core path and sum in fp32 -- and above 64 tokens the
+ *     batched dequant-GEMM on the tcgen05 tensor cores (activations and each
+ *     dequantized weight s (q - z) rounded once to binary16, fp32
+ *     accumulation; with fp32 output of wq_down_w4 the weights enter as two
+ *     exact binary16 parts).  The workspace size covers the path a call takes.
  *   - On error the call returns a negative wq_status and wq_last_error()
  *     describes it (per host thread).  Kernel-side waits are bounded; a wait
  *     that runs out records WQ_ERR_TIMEOUT, read back by wq_device_status().
@@ -216,10 +215,9 @@ wq_status wq_gateup_w2_lora(const void *x, int m, const wq_qweight *gate, const 
  * WQ_NOALLOC_SCRATCH_BYTES bytes inside the library, which every GPU that
  * loads the library keeps until the process exits.  It returns
  * WQ_ERR_UNSUPPORTED and launches nothing when
- *   - m above the dequant-GEMV path's limit (wq_gateup_w2_lora takes the
- *     dequant-GEMM path there),
+ *   - m above that limit (use wq_gateup_w2_lora there),
  *   - the layer shape has no dequant-GEMV launch configuration at this m
- *     (wq_gateup_w2_lora takes the dequant-GEMM path for it), or
+ *     (wq_gateup_w2_lora takes the batched-decode path for it), or
  *   - the layer needs more scratch than the array holds.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress, which may load the library's device code); make
@@ -242,9 +240,8 @@ wq_status wq_gateup_w2_lora_noalloc(const void *x, int m, const wq_qweight *gate
 
 /*
  * App. B's W3-GateUp variant: wq_gateup_w2_lora with 3-bit gate/up codes
- * (bits 3, two bit planes; same arguments, same arithmetic).  Runs on the
- * dequant-GEMV kernels at every token count up to 64 (WQ_ERR_UNSUPPORTED
- * above: the dequant-GEMM path takes 2- and 4-bit codes).
+ * (bits 3, two bit planes; same arguments, same arithmetic), up to 64 tokens
+ * (WQ_ERR_UNSUPPORTED above: the dequant-GEMM path takes 2- and 4-bit codes).
  */
 wq_status wq_gateup_w3_lora(const void *x, int m, const wq_qweight *gate, const wq_qweight *up,
                             const void *lora_a, const void *lora_b_gate, const void *lora_b_up,
@@ -295,7 +292,10 @@ wq_status wq_down_bf16(const void *h, int m, const void *wd, int d, int inter, c
  *   - the launch chain: 2 kernels per layer (plus one for the first layer's
  *     input statistics) with programmatic dependent launch, each down launch
  *     also producing the next layer's RMSNorm and LoRA-A partial sums;
- *   - the dequant-GEMM chain above 16 tokens (8 for d >= 4096).
+ *   - the batched chain above 16 tokens (8 for d >= 4096): the dequant-GEMM
+ *     above 64 tokens.  From 9 to 64 tokens both chains run the batched-decode
+ *     kernels: per layer the activation panel of x with its RMSNorm scales and
+ *     LoRA-A products, gate/up (which leaves the panel of h), down.
  * Every route can be captured into a CUDA graph.
  */
 wq_status wq_mlp_forward(const void *x, int m, const wq_mlp_layer *layers, int n_layers,
@@ -417,10 +417,10 @@ wq_status wq_mlp_forward_states(const void *x, int m, const wq_mlp_layer *layers
 /*
  * How wq_mlp_forward runs this stack on the current device (for tests and
  * tuning; validates like wq_mlp_forward and launches nothing).  info[16]:
- *   [0]      route: 0 = per-layer dequant-GEMV launch chain,
- *                   1 = per-layer dequant-GEMM launch chain,
+ *   [0]      route: 0 = per-layer launch chain of the decode kernels,
+ *                   1 = per-layer batched launch chain,
  *                   2 = single-launch stack kernel
- *   [1..6]   route 0: layer 0's gate/up launch: row tiles per CTA, blocks per
+ *   [1..6]   route 0, up to 8 tokens: layer 0's gate/up launch: row tiles per CTA, blocks per
  *            panel, warps along k, row tiles per warp, panels, CTAs
  *   [7..12]  route 0: layer 0's down launch (writing layer 1's partial sums
  *            when there is a layer 1): the same fields

@@ -11,6 +11,7 @@
 #include <string>
 
 #include "wq.h"
+#include "wq_batch.h"
 #include "wq_internal.h"
 #include "wq_launch.h"
 #include "wq_stack.h"
@@ -85,9 +86,13 @@ struct WsLayout {
   // at zero -- or, for the stack kernel's, at a multiple of its grid -- by the calls)
   size_t cnt1, cnt2, sctr, sk_cnt;
   size_t tp, xa, xb, h, hq, hsc, hxs, part1, part2;
-  // dequant-GEMM path (m > kMaxTokens, or a shape the GEMV path has no plan for)
+  // dequant-GEMM path (m > kMaxTokens)
   size_t x16, rs, ta, h16, hsx, sk_part;
   bool gemm;  // the GEMM buffers are laid out
+  // batched-decode path (m <= kMaxTokens): panels of x and h, RMSNorm scales,
+  // LoRA-A products, fp32 parts of split row blocks
+  size_t bpx, bph, brs, btf, bpart;
+  bool batch;
   // single-launch stack (1..8 tokens)
   size_t sxw, stp, shg, spart, sxc;
   bool stack;
@@ -96,12 +101,18 @@ struct WsLayout {
 
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Token count above which the calls take the dequant-GEMM path: 16, or 8 for
-// layers of hidden size 4096 and more (measured on GB300: at 16 tokens the
-// launch chain of the d 4096 and d 5120 stacks took 157 and 266 us a layer,
-// the GEMM chain at 64 tokens 119 and 147 us; up to 8 tokens the single-launch
-// stack kernel serves those shapes).
+// Token count above which wq_mlp_forward_info reports the batched chain and
+// the call without a workspace refuses: 16, or 8 for hidden sizes of 4096 and
+// more (where one token's share of the GEMV kernels' work is largest).
 int gemv_prefer_tokens(int d) { return d >= 4096 ? 8 : kGemvPreferTokens; }
+
+// Above this many tokens (to kBatchMaxTokens) the launches are the
+// batched-decode ones.  Measured at the line (us a layer, W2 g128, kernels
+// before vs batched): d 2560 at 9 tokens 35.3 (GEMV) vs 26.7, d 4096 102.7
+// (tcgen05) vs 41.1, d 5120 135.8 vs 51.7; 64 tokens 75.7, 110.8 and 145.4
+// (tcgen05) vs 52.0, 89.8 and 121.3.  Above 64 tokens each weight's expansion
+// for tcgen05 is shared by 128 and more tokens.
+constexpr int kBatchAbove = 8;
 
 size_t partial_bytes(const GemvPlan &p, int nproj) {
   return p.P > 1 ? (size_t)p.RT * p.P * nproj * 16 * p.M * 4 : 0;
@@ -208,31 +219,39 @@ bool ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only = false) {
   L->part2 = off; off = up256(off + p2);
   L->total = off;
   if (gemv_only) return true;
-  // above gemv_prefer_tokens, or for a shape that lacks a GEMV plan for some
-  // group or rank at this token count, the calls take the dequant-GEMM path
-  if (m > gemv_prefer_tokens(d) || !all_fit) {
-    if (!gemm_layout(m, d, inter, off, L)) return false;
-    off = L->total;
+  // above kBatchAbove, or for a shape that lacks a GEMV plan for some group or
+  // rank at this token count, the calls take the batched-decode path
+  if (m > kBatchAbove || !all_fit) {
+    const int sms = num_sms(), nt = batch_nt(m);
+    if (sms <= 0) return false;
+    L->bpx = off;   off = up256(off + (size_t)((std::max(d, inter) + 127) / 128) * batch_rec_bytes(nt, 32));
+    L->bph = off;   off = up256(off + (size_t)((inter + 127) / 128) * batch_rec_bytes(nt, 32));
+    L->brs = off;   off = up256(off + (size_t)m * 4);
+    L->btf = off;   off = up256(off + batch_tfrag_bytes(m, kMaxRank));
+    L->bpart = off; off = up256(off + batch_scratch_floats(m, 2, sms) * 4);
+    L->batch = true;
+    L->total = off;
   }
   stack_layout(m, d, inter, off, L);
   return true;
 }
 
 
-// Whether a call takes the dequant-GEMM path: above gemv_prefer_tokens (where
-// it is the faster path on every measured layer shape; the GEMV kernels'
-// work grows faster than linearly with the token count), or where the GEMV
-// path has no launch plan.  The workspace holds the GEMM buffers then.
-bool gateup_uses_gemm(GemvKind kind, int m, const wq_qweight *gate, int r) {
-  if (kind == kGateUpW3) return false;  // the dequant-GEMM path takes 2- and 4-bit codes only
-  if (m > gemv_prefer_tokens(gate->k)) return true;
+// Which kernels a call takes by its token count: the dequant-GEMM path above
+// kMaxTokens; the batched-decode launches above kBatchAbove, and below where
+// the GEMV kernels have no launch plan; the GEMV kernels otherwise.
+enum class Path { kGemv, kBatch, kGemm };
+Path gateup_path(GemvKind kind, int m, const wq_qweight *gate, int r) {
+  if (m > kMaxTokens) return Path::kGemm;
   GemvPlan pl;
-  return !plan_gemv(kind, gate->n, gate->k, m, gate->group, r, num_sms(), &pl);
+  return m > kBatchAbove || !plan_gemv(kind, gate->n, gate->k, m, gate->group, r, num_sms(), &pl) ? Path::kBatch
+                                                                                                  : Path::kGemv;
 }
-bool down_uses_gemm(int m, const wq_qweight *down, int r_next) {
-  if (m > gemv_prefer_tokens(down->n)) return true;
+Path down_path(int m, const wq_qweight *down, int r_next) {
+  if (m > kMaxTokens) return Path::kGemm;
   GemvPlan pl;
-  return !plan_gemv(kDownW4, down->n, down->k, m, down->group, r_next, num_sms(), &pl);
+  return m > kBatchAbove || !plan_gemv(kDownW4, down->n, down->k, m, down->group, r_next, num_sms(), &pl)
+             ? Path::kBatch : Path::kGemv;
 }
 
 // gate/up (2-bit with LoRA, or 4-bit) for one layer.  tp_in: tile partials of
@@ -346,10 +365,72 @@ wq_status run_down(const void *h, int m, const wq_qweight *down, const void *res
   a.nb_out = (size_t)m * down->n * (y_f32 ? 4 : 2);
   a.nb_an = (size_t)2 * rr * down->n * 2;
   a.nb_tp_out = tp_out ? (size_t)((down->n + 15) / 16) * m * WQ_TP_STRIDE(rr) * 4 : 0;
-  a.nb_part = (L.gemm ? L.x16 : L.stack ? L.sxw : L.total) - L.part2;
+  a.nb_part = (L.batch ? L.bpx : L.stack ? L.sxw : L.total) - L.part2;
   a.nb_cnt = (size_t)((down->n + 15) / 16) * 4;
   cudaError_t e = launch_gemv(kDownW4, plan, a, s, true);
   if (e != cudaSuccess) return cuda_fail(e, "down launch");
+  return WQ_OK;
+}
+
+// ---- batched-decode path (to kBatchMaxTokens tokens) ----
+// gate/up: the panel of x, RMSNorm scales and lora_scale * x A^T first, then
+// the projections.  With panel_down, h is also left as the panel that the down
+// launch with that matrix reads, and h itself may be null.
+wq_status run_gateup_batch(GemvKind kind, const void *x, int m, const wq_qweight *gate, const wq_qweight *up,
+                           const void *lora_a, const void *lora_bg, const void *lora_bu, int r, float lora_scale,
+                           unsigned flags, void *h, const wq_qweight *panel_down, const WsLayout &L, uint8_t *ws,
+                           cudaStream_t s) {
+  if (!L.batch) return fail(WQ_ERR_WORKSPACE, "workspace laid out without the batched-decode buffers");
+  BatchArgs a = {};
+  a.panel = ws + L.bpx;
+  float *rs = (flags & WQ_PRENORM) ? reinterpret_cast<float *>(ws + L.brs) : nullptr;
+  uint8_t *tf = r > 0 ? ws + L.btf : nullptr;
+  cudaError_t e = launch_batch_prep(x, m, gate->k, gate->bits, gate->group, lora_a, r, lora_scale, ws + L.bpx, rs, tf, s);
+  if (e != cudaSuccess) return cuda_fail(e, "batched input launch");
+  a.M = m;
+  a.N = gate->n;
+  a.K = gate->k;
+  a.group = gate->group;
+  a.codes[0] = gate->codes;
+  a.codes[1] = up->codes;
+  a.meta[0] = gate->meta;
+  a.meta[1] = up->meta;
+  a.tfrag = tf;
+  a.r = r;
+  a.lora_b[0] = lora_bg;
+  a.lora_b[1] = lora_bu;
+  a.rs = rs;
+  a.out = h;
+  a.panel_out = panel_down ? ws + L.bph : nullptr;
+  a.group_out = panel_down ? panel_down->group : 128;
+  a.part = reinterpret_cast<float *>(ws + L.bpart);
+  a.cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
+  if ((e = launch_batch(kind, a, s)) != cudaSuccess) return cuda_fail(e, "batched gate/up launch");
+  return WQ_OK;
+}
+
+// down; h null: the panel that run_gateup_batch left.
+wq_status run_down_batch(const void *h, int m, const wq_qweight *down, const void *residual, void *y, int y_f32,
+                         const WsLayout &L, uint8_t *ws, cudaStream_t s) {
+  if (!L.batch) return fail(WQ_ERR_WORKSPACE, "workspace laid out without the batched-decode buffers");
+  cudaError_t e;
+  if (h && (e = launch_batch_prep(h, m, down->k, 4, down->group, nullptr, 0, 0.f, ws + L.bph, nullptr, nullptr, s)) !=
+               cudaSuccess)
+    return cuda_fail(e, "batched input launch");
+  BatchArgs a = {};
+  a.panel = ws + L.bph;
+  a.M = m;
+  a.N = down->n;
+  a.K = down->k;
+  a.group = down->group;
+  a.codes[0] = down->codes;
+  a.meta[0] = down->meta;
+  a.residual = residual;
+  a.out = y;
+  a.out_f32 = y_f32;
+  a.part = reinterpret_cast<float *>(ws + L.bpart);
+  a.cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
+  if ((e = launch_batch(kDownW4, a, s)) != cudaSuccess) return cuda_fail(e, "batched down launch");
   return WQ_OK;
 }
 
@@ -480,12 +561,19 @@ wq_status gateup_entry(GemvKind kind, const void *x, int m, const wq_qweight *ga
   if (!aligned16(x) || !aligned16(h)) return fail(WQ_ERR_ALIGN, "x or h not 16-byte aligned");
   WsLayout L;
   if ((st = check_ws(ws, ws_bytes, m, gate->k, gate->n, &L)) != WQ_OK) return st;
-  if (gateup_uses_gemm(kind, m, gate, r))
-    st = run_gateup_gemm(kind, x, m, gate, up, lora_a, bg, bu, r, lora_scale, flags, h, L,
-                         static_cast<uint8_t *>(ws), static_cast<cudaStream_t>(stream));
-  else
-    st = run_gateup(kind, x, m, gate, up, lora_a, bg, bu, r, lora_scale, flags, h, nullptr, L,
-                    static_cast<uint8_t *>(ws), static_cast<cudaStream_t>(stream));
+  uint8_t *w8 = static_cast<uint8_t *>(ws);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  switch (gateup_path(kind, m, gate, r)) {
+    case Path::kGemm:
+      st = run_gateup_gemm(kind, x, m, gate, up, lora_a, bg, bu, r, lora_scale, flags, h, L, w8, s);
+      break;
+    case Path::kBatch:
+      st = run_gateup_batch(kind, x, m, gate, up, lora_a, bg, bu, r, lora_scale, flags, h, nullptr, L, w8, s);
+      break;
+    case Path::kGemv:
+      st = run_gateup(kind, x, m, gate, up, lora_a, bg, bu, r, lora_scale, flags, h, nullptr, L, w8, s);
+      break;
+  }
   return st == WQ_OK ? ok() : st;
 }
 
@@ -680,12 +768,13 @@ wq_status wq_down_w4(const void *h, int m, const wq_qweight *down, const void *r
     return fail(WQ_ERR_ALIGN, "h, y or residual not 16-byte aligned");
   WsLayout L;
   if ((st = check_ws(ws, ws_bytes, m, down->n, down->k, &L)) != WQ_OK) return st;
-  if (down_uses_gemm(m, down, 0))
-    st = run_down_gemm(h, m, down, residual, y, y_dtype == WQ_F32, L, static_cast<uint8_t *>(ws),
-                       static_cast<cudaStream_t>(stream));
-  else
-    st = run_down(h, m, down, residual, y, y_dtype == WQ_F32, nullptr, 0, nullptr, L, static_cast<uint8_t *>(ws),
-                  static_cast<cudaStream_t>(stream));
+  uint8_t *w8 = static_cast<uint8_t *>(ws);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  switch (down_path(m, down, 0)) {
+    case Path::kGemm: st = run_down_gemm(h, m, down, residual, y, y_dtype == WQ_F32, L, w8, s); break;
+    case Path::kBatch: st = run_down_batch(h, m, down, residual, y, y_dtype == WQ_F32, L, w8, s); break;
+    case Path::kGemv: st = run_down(h, m, down, residual, y, y_dtype == WQ_F32, nullptr, 0, nullptr, L, w8, s); break;
+  }
   return st == WQ_OK ? ok() : st;
 }
 
@@ -748,11 +837,12 @@ wq_status check_stack(int m, const wq_mlp_layer *layers, int n_layers, unsigned 
   return WQ_OK;
 }
 
-// How a stack runs: the per-layer dequant-GEMV launch chain, the
-// dequant-GEMM launch chain (every layer's launches need a GEMV plan for the
-// first; above gemv_prefer_tokens tokens the second), or the single-launch
-// stack kernel (1..8 tokens, every layer with the same bits, groups and rank,
-// unless the caller asks for the chain).
+// How a stack runs: the per-layer launch chain of the decode kernels, the
+// batched launch chain (above gemv_prefer_tokens tokens, or where some layer
+// has no GEMV plan), or the single-launch stack kernel (1..8 tokens, every
+// layer with the same bits, groups and rank, unless the caller asks for the
+// chain).  Both chains take the batched-decode launches for more than
+// kBatchAbove and up to kBatchMaxTokens tokens.
 enum StackRoute { kRouteGemvChain = 0, kRouteGemmChain = 1, kRouteStack = 2 };
 
 bool cooperative_ok() {
@@ -798,8 +888,9 @@ StackRoute stack_route(int m, const wq_mlp_layer *layers, int n_layers, unsigned
   for (int l = 0; l < n_layers; ++l) {
     const wq_mlp_layer &Ly = layers[l];
     const bool next_tp = l + 1 < n_layers && ((flags & WQ_PRENORM) || layers[l + 1].r > 0);
-    if (gateup_uses_gemm(gateup_kind(Ly.gate.bits), m, &Ly.gate, Ly.r) ||
-        (Ly.down.bits == 4 && down_uses_gemm(m, &Ly.down, next_tp ? layers[l + 1].r : 0)))
+    if (m > kBatchAbove) continue;  // the batched-decode launches take every shape
+    if (gateup_path(gateup_kind(Ly.gate.bits), m, &Ly.gate, Ly.r) != Path::kGemv ||
+        (Ly.down.bits == 4 && down_path(m, &Ly.down, next_tp ? layers[l + 1].r : 0) != Path::kGemv))
       return kRouteGemmChain;
   }
   return kRouteGemvChain;
@@ -888,6 +979,29 @@ wq_status mlp_forward_impl(const void *x, int m, const wq_mlp_layer *layers, int
       cur = a.y_out;
     }
     return ok();
+  }
+  if (m <= kBatchMaxTokens && (m > kBatchAbove || route == kRouteGemmChain)) {
+    // batched-decode chain: per layer the panel of x with its RMSNorm scales
+    // and LoRA-A products, gate/up (which leaves the panel of h), down
+    const void *cur = x;
+    for (int l = 0; l < n_layers; ++l) {
+      const wq_mlp_layer &Ly = layers[l];
+      void *out = layer_out(l);
+      const bool dense_down = Ly.down.bits == 16;
+      void *hbuf = dense_down || h_states ? layer_h(l) : nullptr;
+      st = run_gateup_batch(gateup_kind(Ly.gate.bits), cur, m, &Ly.gate, &Ly.up, Ly.lora_a, Ly.lora_b_gate,
+                            Ly.lora_b_up, Ly.r, Ly.lora_scale, flags, hbuf, dense_down ? nullptr : &Ly.down, L, w8, s);
+      if (st != WQ_OK) return fail(st, "layer %d: %s", l, g_last_error.c_str());
+      if (dense_down) {
+        cudaError_t e = launch_down_bf16(hbuf, m, Ly.down.codes, d, inter, cur, out, false, s);
+        if (e != cudaSuccess) return cuda_fail(e, "bf16 down launch");
+      } else {
+        st = run_down_batch(nullptr, m, &Ly.down, cur, out, 0, L, w8, s);
+        if (st != WQ_OK) return fail(st, "layer %d: %s", l, g_last_error.c_str());
+      }
+      cur = out;
+    }
+    return finish();
   }
   if (route == kRouteGemmChain) {
     // dequant-GEMM chain: per layer the GEMM inputs of x, gate/up, the
@@ -987,6 +1101,10 @@ wq_status wq_mlp_forward_info(int m, const wq_mlp_layer *layers, int n_layers, u
   if (route == kRouteGemvChain) {
     const wq_mlp_layer &L0 = layers[0];
     const GemvKind kind = gateup_kind(L0.gate.bits);
+    if (m > kBatchAbove) {  // the batched-decode launches have no GEMV plan; gate/up leaves the down launch's panel
+      info[13] = L0.down.bits == 4 ? 1 : 0;
+      return ok();
+    }
     const bool next_tp = n_layers > 1 && ((flags & WQ_PRENORM) || layers[1].r > 0);
     const int r_next = next_tp ? layers[1].r : 0;
     GemvPlan pg, pd{};
@@ -1116,8 +1234,11 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
     const GemvKind kind = gateup_kind(bits);
     const bool need_tp = (flags & WQ_PRENORM) || M.r > 0;
     const int r_o = need_tp ? M.r : 0;
-    if (gu_ok && !gateup_uses_gemm(kind, batch, &M.gate, M.r) && !down_uses_gemm(batch, &M.down, 0) &&
-        !down_uses_gemm(batch, &Ly.o, r_o) && (r_o == 0 || d % 8 == 0)) {
+    const bool gemv = gu_ok && gateup_path(kind, batch, &M.gate, M.r) == Path::kGemv &&
+                      down_path(batch, &M.down, 0) == Path::kGemv && down_path(batch, &Ly.o, r_o) == Path::kGemv &&
+                      (r_o == 0 || d % 8 == 0);
+    const bool batched = gu_ok && batch > kBatchAbove && batch <= kBatchMaxTokens;
+    if (gemv || batched) {
       if (!y) return fail(WQ_ERR_ARG, "null y");
       if (!aligned16(y)) return fail(WQ_ERR_ALIGN, "y not 16-byte aligned");
       WsLayout Lm, Lo;
@@ -1125,6 +1246,16 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
           (st = check_ws(w8 + W.proj_o, W.n_o, batch, d, H * hd, &Lo)) != WQ_OK)
         return st;
       cudaStream_t s = static_cast<cudaStream_t>(stream);
+      if (batched) {
+        if ((st = run_down_batch(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, 0, Lo, w8 + W.proj_o, s)) != WQ_OK)
+          return fail(st, "output projection: %s", g_last_error.c_str());
+        if ((st = run_gateup_batch(kind, w8 + W.x1, batch, &M.gate, &M.up, M.lora_a, M.lora_b_gate, M.lora_b_up, M.r,
+                                   M.lora_scale, flags, nullptr, &M.down, Lm, w8 + W.mlp, s)) != WQ_OK)
+          return fail(st, "gate/up: %s", g_last_error.c_str());
+        if ((st = run_down_batch(nullptr, batch, &M.down, w8 + W.x1, y, 0, Lm, w8 + W.mlp, s)) != WQ_OK)
+          return fail(st, "down: %s", g_last_error.c_str());
+        return ok();
+      }
       float *tp = need_tp ? reinterpret_cast<float *>(w8 + W.mlp + Lm.tp) : nullptr;
       if ((st = run_down(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, 0, need_tp ? M.lora_a : nullptr, r_o, tp, Lo,
                          w8 + W.proj_o, s)) != WQ_OK)
@@ -1361,6 +1492,9 @@ wq_status wq_device_status(int *status) {
   if (e != cudaSuccess) return cuda_fail(e, "device status read");
   if (*status == 0) *status = g;
   e = read_attn_status(&g);
+  if (e != cudaSuccess) return cuda_fail(e, "device status read");
+  if (*status == 0) *status = g;
+  e = read_batch_status(&g);
   if (e != cudaSuccess) return cuda_fail(e, "device status read");
   if (*status == 0) *status = g;
   return ok();

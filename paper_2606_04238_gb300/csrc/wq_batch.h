@@ -1,0 +1,75 @@
+// wq_batch.h -- the batched-decode dequant-GEMM (wq_batch.cuh): host interface.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+#include "wq_internal.h"
+
+namespace wq {
+
+constexpr int kBatchMaxTokens = 64;  // tokens a launch can take (8 MMA tiles of 8)
+
+// 8-token MMA tiles a launch of m tokens computes (the kernels exist for
+// 1, 2, 3, 4, 6 and 8).
+inline int batch_nt(int m) {
+  const int n = (m + 7) / 8;
+  return n <= 4 ? n : n <= 6 ? 6 : 8;
+}
+
+// Activation panel: one record per 128-feature block,
+//   [NT][4][32 lanes][16 bytes]  the binary16 m16n8k16 B fragments of two
+//                                16-feature steps a lane, scaled by 2^e per
+//                                (block, token) -- e puts the largest |x| in
+//                                [2^14, 2^15) -- and by 4^-c (2- and 3-bit
+//                                codes) or 16^-c (4-bit) for the bit-position
+//                                class c of the codes they meet
+//   [NT * 8] fp32                2^(24 - e) per token
+//   [128 / group][NT * 8] fp32   sums of x over each quantization group
+inline __host__ __device__ uint32_t batch_rec_bytes(int nt, int group) {
+  return (uint32_t)nt * (2048u + 32u + 32u * (128u / (uint32_t)group));
+}
+
+struct BatchArgs {
+  const uint8_t *panel;      // [ceil(K / 128)] records
+  int M, N, K, group;
+  const uint32_t *codes[2];  // gate, up; or down
+  const uint16_t *meta[2];
+  // gate/up: lora_scale * x A^T as bf16 high and low parts, m16n8k16 B
+  // fragments [projection][ceil(r / 16)][NT][32 lanes][16 bytes] (null: no
+  // adapter); LoRA-B bf16 [N][r]; RMSNorm scale per token (null: 1)
+  const uint8_t *tfrag;
+  int r;
+  const void *lora_b[2];
+  const float *rs;
+  const void *residual;      // down: bf16 [M][N] or null
+  void *out;                 // bf16 (down: or fp32) [M][N]; gate/up: may be null with panel_out
+  int out_f32;
+  uint8_t *panel_out;        // gate/up: also the 4-bit down launch's panel of h (null: none)
+  int group_out;             // its quantization group
+  float *part;               // batch_scratch_floats() fp32
+  unsigned *cnt;             // [ceil(N / 128)] arrival counters, zero between launches
+};
+
+// Panel of x bf16 [M, K] for codes of `bits` bits and groups of `group`, and
+// with rs / tfrag (either may be null) the RMSNorm scales and LoRA-A products.
+cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, const void *lora_a, int r,
+                              float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, cudaStream_t s);
+cudaError_t launch_batch(GemvKind kind, const BatchArgs &a, cudaStream_t s);
+size_t batch_scratch_floats(int M, int nproj, int num_sms);
+size_t batch_tfrag_bytes(int M, int r);
+cudaError_t read_batch_status(int *status);
+
+// One translation unit per kind.
+cudaError_t launch_batch_gu2(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_gu3(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_dn4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t read_batch_status_gu2(int *status);
+cudaError_t read_batch_status_gu3(int *status);
+cudaError_t read_batch_status_gu4(int *status);
+cudaError_t read_batch_status_dn4(int *status);
+
+}  // namespace wq

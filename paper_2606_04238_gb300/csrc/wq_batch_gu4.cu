@@ -1,0 +1,12 @@
+// wq_batch_gu4.cu -- instantiations of the batched-decode dequant-GEMM: 4-bit gate/up.
+#include "wq_batch.cuh"
+
+namespace wq {
+
+cudaError_t launch_batch_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s) {
+  return launch_batch_g<4, 2>(a, nt, ctas, s);
+}
+
+cudaError_t read_batch_status_gu4(int *status) { return read_batch_status_tu(status); }
+
+}  // namespace wq

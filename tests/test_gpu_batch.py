@@ -1,0 +1,125 @@
+"""The batched-decode kernels (9 to 64 tokens) vs the fp64 oracle at the sizes
+where their split can go wrong: every count of 8-token tiles and its edges,
+ragged row blocks and feature blocks, one unit to many parts a row block,
+adapter ranks that are no multiple of 16, every code width and group, rows
+that are no multiple of 4 (scalar stores), and the panel gate/up hands down.
+
+Products are exact and sums fp32, so the bound and the share of bit-equal
+bf16 outputs are those of the other decode kernels (check_bf16's defaults).
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from paper_2606_04238_gb300 import synth
+from tests.gpu_util import check_bf16, check_f32, upload_packed
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wq():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2606_04238_gb300 import wq as mod
+    return mod
+
+
+def _q(shape, group, bits, seed):
+    w = (np.random.default_rng(seed).standard_normal(shape) * 0.02).astype(np.float32)
+    return orc.quantize(w, group, bits)[:3]
+
+
+GATEUP = [
+    # bits, d, inter, group, r, token counts
+    (2, 128, 16, 128, 0, (9, 64)),             # one unit in all
+    (2, 2048, 130, 64, 24, (10, 17, 25)),      # two row blocks, the second with 2 rows; rank 24
+    (2, 96, 1000, 32, 8, (33, 41, 49)),        # less than a feature block; rank 8
+    (3, 640, 384, 32, 16, (9, 31, 57)),
+    (3, 512, 200, 128, 64, (16, 48)),
+    (4, 1152, 264, 64, 0, (24, 40, 64)),
+]
+
+
+@pytest.mark.parametrize("bits,d,inter,group,r,ms", GATEUP)
+def test_batch_gateup(wq, bits, d, inter, group, r, ms):
+    qg, qu = _q((inter, d), group, bits, d + inter), _q((inter, d), group, bits, d + inter + 1)
+    g, u = upload_packed(*qg, group, bits), upload_packed(*qu, group, bits)
+    kw, bl = {}, (None, None, None)
+    if r:
+        a, bg, bu = synth.lora(d, inter, r, d + r)
+        kw = dict(lora_a=a.cuda(), lora_b_gate=bg.cuda(), lora_b_up=bu.cuda())
+        bl = tuple(synth.bf16_bits(t) for t in (a, bg, bu))
+    for m in ms:
+        x = synth.activations((m, d), 10 + m)
+        for prenorm in (True, False):
+            if bits == 4:
+                h = wq.gateup_w4(x.cuda(), g, u, prenorm=prenorm)
+            else:
+                fn = wq.gateup_w2_lora if bits == 2 else wq.gateup_w3_lora
+                h = fn(x.cuda(), g, u, lora_scale=2.0, prenorm=prenorm, **kw)
+            torch.cuda.synchronize()
+            assert wq.device_status() == 0
+            ref, _ = orc.gateup(synth.bf16_bits(x), qg, qu, group, *bl, lora_scale=2.0 if r else 0.0, prenorm=prenorm)
+            check_bf16(h, ref, f"batch h bits={bits} d={d} I={inter} g={group} r={r} m={m} prenorm={prenorm}")
+
+
+DOWN = [
+    # d, inter, group, token counts
+    (16, 128, 128, (9,)),
+    (202, 1056, 32, (12, 64)),        # rows no multiple of 4; ragged feature block
+    (130, 20480, 128, (17, 63)),      # 2 row blocks, 160 blocks: about 76 parts each
+    (2560, 704, 64, (32, 33)),
+]
+
+
+@pytest.mark.parametrize("d,inter,group,ms", DOWN)
+def test_batch_down(wq, d, inter, group, ms):
+    qd = _q((d, inter), group, 4, d * 3 + inter)
+    dn = upload_packed(*qd, group, 4)
+    for m in ms:
+        h = (synth.activations((m, inter), 20 + m) * 0.5).to(torch.bfloat16)
+        res = synth.activations((m, d), 30 + m)
+        y = wq.down_w4(h.cuda(), dn, residual=res.cuda())
+        y32 = wq.down_w4(h.cuda(), dn, out_f32=True)
+        torch.cuda.synchronize()
+        assert wq.device_status() == 0
+        ref, _ = orc.down(synth.bf16_bits(h), qd, group, synth.bf16_bits(res))
+        ref0, _ = orc.down(synth.bf16_bits(h), qd, group, None)
+        check_bf16(y, ref, f"batch y d={d} I={inter} g={group} m={m}")
+        check_f32(y32, ref0, f"batch y fp32 d={d} m={m}")
+
+
+@pytest.mark.parametrize("bits,group,group_down,r", [(2, 64, 32, 8), (3, 32, 128, 16), (4, 128, 64, 0)])
+@pytest.mark.parametrize("m", [9, 40])
+def test_batch_stack_hands_down_the_panel(wq, bits, group, group_down, r, m):
+    """Two layers through wq_mlp_forward, each kernel teacher-forced; the run that
+    keeps h and the run that only hands on its panel give the same y."""
+    d, inter = 384, 896
+    layers, ents = [], []
+    for l in range(2):
+        qg, qu = _q((inter, d), group, bits, 70 + l), _q((inter, d), group, bits, 80 + l)
+        qd = _q((d, inter), group_down, 4, 90 + l)
+        kw, bl = {}, (None, None, None)
+        if r:
+            a, bg, bu = synth.lora(d, inter, r, 50 + l)
+            kw = dict(lora_a=a.cuda(), lora_b_gate=bg.cuda(), lora_b_up=bu.cuda(), lora_scale=2.0)
+            bl = tuple(synth.bf16_bits(t) for t in (a, bg, bu))
+        layers.append(wq.MLPLayer(upload_packed(*qg, group, bits), upload_packed(*qu, group, bits),
+                                  upload_packed(*qd, group_down, 4), **kw))
+        ents.append((qg, qu, qd, bl))
+    x = synth.activations((m, d), 7).cuda()
+    ws = wq.workspace(m, d, inter, r)
+    y, states, h_states = wq.mlp_forward_states(x, layers, prenorm=True, ws=ws, with_h=True)
+    y_plain = wq.mlp_forward(x, layers, prenorm=True, ws=ws)
+    torch.cuda.synchronize()
+    assert wq.device_status() == 0
+    assert torch.equal(y.view(torch.int16), y_plain.view(torch.int16))
+    prev = synth.bf16_bits(x.cpu())
+    for l, (qg, qu, qd, bl) in enumerate(ents):
+        ref, _ = orc.gateup(prev, qg, qu, group, *bl, lora_scale=2.0 if r else 0.0, prenorm=True)
+        check_bf16(h_states[l], ref, f"batch stack bits={bits} m={m} layer {l} h")
+        ref, _ = orc.down(synth.bf16_bits(h_states[l].cpu()), qd, group_down, prev)
+        check_bf16(states[l], ref, f"batch stack bits={bits} m={m} layer {l} y")
+        prev = synth.bf16_bits(states[l].cpu())
