@@ -380,8 +380,10 @@ typedef struct {
  *   expert_idx (int32 [m, top_k]), expert_w (fp32 [m, top_k]), h_slots
  *   (bf16 [m top_k, inter]) and y_slots (fp32 [m top_k, d]): optional device
  *   outputs of steps 1-2, slot t*top_k + j (NULL: kept in the workspace).
- * Four launches on `stream` (routing with the tile partials, gate/up and down
- * over the slots, combine); only the selected experts' weights are read.
+ * Up to 12 slots, four launches on `stream` (routing with the tile partials,
+ * gate/up and down over the slots, combine); above, five (routing and grouping
+ * of the slots by expert, the groups' inputs, gate/up and down over the groups,
+ * combine).  Only the selected experts' weights are read.
  * Workspace: wq_moe_workspace_bytes for this layer, token count and flags,
  * zero-filled before first use (wq_workspace_init).
  */

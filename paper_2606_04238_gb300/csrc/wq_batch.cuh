@@ -125,7 +125,7 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <int BITS, int NPROJ, int GROUP, int NT>
+template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED>
 __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 1)
     batch_kernel(const __grid_constant__ BatchArgs a) {
   using C = BatchCfg<BITS, NPROJ, GROUP, NT>;
@@ -135,10 +135,17 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::OFF_BAR), *empty = full + RX, *aux = empty + RX;
   volatile int *abort_s = reinterpret_cast<volatile int *>(aux + 1), *last_s = abort_s + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int U = (a.K + 127) / 128, T = (a.N + kBatchRows - 1) / kBatchRows;
-  const long long W = (long long)T * U, P = gridDim.x;
-  const long long g0 = W * blockIdx.x / P;
-  const int n = (int)(W * (blockIdx.x + 1) / P - g0);  // units of this CTA
+  const int U = (a.K + 127) / 128, RB = (a.N + kBatchRows - 1) / kBatchRows;
+  // Routed: row block `tile` is block tile % RB of segment tile / RB's expert.
+  // The route was written two launches back (the launch in between lets this
+  // one start only after its own wait), so it may be read before the wait.
+  const int T = ROUTED ? __ldcg(&a.route->n_segs) * RB : RB;
+  auto seg_of = [&](int tile) { return __ldcg(&a.route->seg[tile / RB]); };
+  // the CTAs that take units, 2 each at least (routed: the grid is sized for the most segments)
+  const long long W = (long long)T * U, P = min((long long)gridDim.x, max(1LL, W / 2));
+  const bool takes = blockIdx.x < P;
+  const long long g0 = takes ? W * blockIdx.x / P : 0;
+  const int n = takes ? (int)(W * (blockIdx.x + 1) / P - g0) : 0;  // units of this CTA
   const int tile0 = (int)(g0 / U), kb0 = (int)(g0 - (long long)tile0 * U);
   if (tid == 0) {
     for (int s = 0; s < RX; ++s) {
@@ -173,19 +180,21 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   int pi = wk, pslot = 0, ptile = tile0, pkb = kb0 + wk;
   auto aim = [&]() {
     while (pkb >= U) pkb -= U, ++ptile;
+    const int rb8 = (ROUTED ? ptile % RB : ptile) * 8;
+    const size_t rte = ROUTED && pi < n ? (size_t)seg_of(ptile).x * RT : 0;  // the expert's first row tile
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int c = lane + 32 * q, tl = c / CPT, off = c - tl * CPT;
-      const int rt = ptile * 8 + (NPROJ == 2 ? rg : 2 * rg + tl);
+      const int rt = rb8 + (NPROJ == 2 ? rg : 2 * rg + tl);
       cin[q] = rt < RT;
       csrc[q] = reinterpret_cast<const uint8_t *>(NPROJ == 2 && tl ? a.codes[1] : a.codes[0]) +
-                (cin[q] ? ((size_t)rt * U + pkb) * BPK + off * 16 : 0);
+                (cin[q] ? ((rte + rt) * U + pkb) * BPK + off * 16 : 0);
     }
     const int tl = lane / MPT, off = lane - tl * MPT;
-    const int rt = ptile * 8 + (NPROJ == 2 ? rg : 2 * rg + tl);
+    const int rt = rb8 + (NPROJ == 2 ? rg : 2 * rg + tl);
     min_ = lane < 2 * MPT && rt < RT;
     msrc = reinterpret_cast<const uint8_t *>(NPROJ == 2 && tl ? a.meta[1] : a.meta[0]) +
-           (min_ ? ((size_t)rt * U + pkb) * (GPB * 64) + off * 16 : 0);
+           (min_ ? ((rte + rt) * U + pkb) * (GPB * 64) + off * 16 : 0);
   };
   aim();
   auto issue = [&]() {
@@ -214,21 +223,22 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   uint64_t *sfull = full + wk * RXR, *sempty = empty + wk * RXR;
   uint8_t *xring = smem + wk * RXR * C::REC;
   const int nset = (n - wk + WK - 1) / WK;  // units of this set (n >= wk or 0)
-  int rkb = kb0 + wk;                       // block of the next record
+  int rkb = kb0 + wk, rtile = tile0;        // block (and row block) of the next record
   int rj = 0, rst = 0, rph = 1;             // its index, stage, and the parity its stage's `empty` was last completed with
   int issued = -1;                          // the last record this warp copied
   auto produce = [&](int turn) {
     if (rj < nset && turn == rg && elect_one()) {
-      while (rkb >= U) rkb -= U;
+      while (rkb >= U) rkb -= U, ++rtile;
+      const uint8_t *panel = a.panel + (ROUTED ? (size_t)(rtile / RB) * U * C::REC : 0);
       if (rj < RXR || wait(&sempty[rst], rph)) {
         mbar_arrive_expect_tx(&sfull[rst], (uint32_t)C::REC);
-        bulk_g2s(xring + rst * C::REC, a.panel + (size_t)rkb * C::REC, (uint32_t)C::REC, &sfull[rst]);
+        bulk_g2s(xring + rst * C::REC, panel + (size_t)rkb * C::REC, (uint32_t)C::REC, &sfull[rst]);
         issued = rj;
       }
     }
     ++rj;
     rkb += WK;
-    while (rkb >= U) rkb -= U;
+    while (rkb >= U) rkb -= U, ++rtile;
     if (++rst == RXR) rst = 0, rph ^= 1;
   };
 #pragma unroll 1
@@ -237,7 +247,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   pdl_launch_dependents();
 #pragma unroll
   for (int q = 0; q < LEAD; ++q) produce(q);
-  if (NPROJ == 2 && warp == LEAD && elect_one()) {
+  if (NPROJ == 2 && !ROUTED && warp == LEAD && elect_one()) {
     const uint32_t tfb = BITS != 4 && a.tfrag != nullptr ? 2u * ((a.r + 15) / 16) * NT * 512u : 0u;
     const uint32_t rsb = a.rs != nullptr ? NT * 32u : 0u;
     mbar_arrive_expect_tx(aux, tfb + rsb);
@@ -252,8 +262,9 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
     const int len = min(U - ub, n - i0);
     if (NPROJ == 2 && a.tfrag != nullptr && wk == 0 && lane < a.r / 4) {
       // this part's LoRA-B rows towards L2
-      const size_t off = (size_t)(tile * kBatchRows + rg * 16) * a.r * 2 + lane * 128;
-      if (off < (size_t)a.N * a.r * 2) {
+      const size_t row0 = (ROUTED ? tile % RB : tile) * kBatchRows + rg * 16;
+      const size_t off = ((ROUTED ? (size_t)seg_of(tile).x * a.N : 0) + row0) * a.r * 2 + lane * 128;
+      if (row0 * a.r * 2 + lane * 128 < (size_t)a.N * a.r * 2) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint8_t *>(a.lora_b[0]) + off));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint8_t *>(a.lora_b[1]) + off));
       }
@@ -447,9 +458,13 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
           }
       }
     }
-    const int n0 = (tile - 1) * kBatchRows;
+    const int seg = ROUTED ? (tile - 1) / RB : 0, rblk = tile - 1 - seg * RB, n0 = rblk * kBatchRows;
+    const int4 sg = ROUTED ? seg_of(tile - 1) : make_int4(0, a.M, 0, 0);
+    const int M = sg.y;
+    // output row of token m
+    auto orow = [&](int m) -> size_t { return ROUTED ? (size_t)__ldcg(&a.route->list[sg.z + m]) : (size_t)m; };
     if (NPROJ == 2) {
-      wait(aux, 0);
+      if (!ROUTED) wait(aux, 0);
       // Eq. 1's unmerged adapter: tot += B t, t as two bf16 parts
       if (BITS != 4 && a.tfrag != nullptr) {
         const int RK = (a.r + 15) / 16;
@@ -459,9 +474,9 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const int row = n0 + rg * 16 + g + 8 * (q & 1), col = kk * 16 + 2 * t + 8 * (q >> 1);
+              const size_t at = (ROUTED ? (size_t)sg.x * a.N + row : (size_t)row) * a.r + col;
               bf[p][q] = row < a.N && col < a.r
-                             ? __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(a.lora_b[p]) +
-                                                                        ((size_t)row * a.r + col) * 2))
+                             ? __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(a.lora_b[p]) + at * 2))
                              : 0u;
             }
         };
@@ -474,7 +489,10 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
           for (int p = 0; p < 2; ++p)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
-              const uint4 tv = lds128(smem + C::OFF_TF + (((p * RK + kk) * NT + nt) * 32 + lane) * 16);
+              const uint32_t at = (((p * RK + kk) * NT + nt) * 32 + lane) * 16;
+              const uint4 tv = ROUTED ? __ldcg(reinterpret_cast<const uint4 *>(
+                                            a.tfrag + (size_t)seg * (2 * RK * NT * 512) + at))
+                                      : lds128(smem + C::OFF_TF + at);
               mma_bf16_16816(tot[p][nt], bf[p], tv.x, tv.y);
               mma_bf16_16816(tot[p][nt], bf[p], tv.z, tv.w);
             }
@@ -493,7 +511,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int m = nt * 8 + 2 * t + e;
-          const float rs = a.rs != nullptr && m < a.M ? rs_s[m] : 1.f;
+          const float rs = a.rs == nullptr || m >= M ? 1.f : ROUTED ? __ldcg(a.rs + seg * NT * 8 + m) : rs_s[m];
 #pragma unroll
           for (int rr = 0; rr < 2; ++rr) {
             const float gv = rs * tot[0][nt][2 * rr + e], uv = rs * tot[1][nt][2 * rr + e];
@@ -504,8 +522,8 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
       const int nb = n0 + 4 * lane;
       for (int m = rg; m < NT * 8; m += RG) {
         const uint2 raw = lds64(hs + m * kHsStride + 4 * lane);
-        if (a.out != nullptr && m < a.M && nb < a.N) {
-          __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(a.out) + (size_t)m * a.N + nb;
+        if (a.out != nullptr && m < M && nb < a.N) {
+          __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(a.out) + orow(m) * a.N + nb;
           if ((a.N & 3) == 0) {
             *reinterpret_cast<uint2 *>(o) = raw;
           } else {
@@ -517,7 +535,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
           const float f[4] = {__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
                               __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u)};
           batch_panel_token(a.panel_out + (size_t)(tile - 1) * batch_rec_bytes(NT, a.group_out), NT, a.group_out, true, m,
-                            lane, f);
+                            lane, f);  // routed: RB records a segment
         }
       }
     } else {
@@ -535,23 +553,23 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
       const int nb = n0 + 4 * lane;
       const bool vec = (a.N & 3) == 0;
       constexpr int MU = 4;  // tokens of a warp in flight
-      for (int mb = rg; mb < a.M; mb += RG * MU) {
+      for (int mb = rg; mb < M; mb += RG * MU) {
         uint2 res[MU];
 #pragma unroll
         for (int q = 0; q < MU; ++q) {
           const int m = mb + q * RG;
           res[q] = make_uint2(0u, 0u);
-          if (a.residual != nullptr && vec && m < a.M && nb < a.N)
+          if (a.residual != nullptr && vec && m < M && nb < a.N)
             res[q] = __ldcg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(a.residual) +
                                                             (size_t)m * a.N + nb));
         }
 #pragma unroll
         for (int q = 0; q < MU; ++q) {
           const int m = mb + q * RG;
-          if (m >= a.M || nb >= a.N) continue;
+          if (m >= M || nb >= a.N) continue;
           const float4 v4 = *reinterpret_cast<const float4 *>(ys + m * kYsStride + 4 * lane);
           float v[4] = {v4.x, v4.y, v4.z, v4.w};
-          const size_t o = (size_t)m * a.N + nb;
+          const size_t o = orow(m) * a.N + nb;
           if (vec) {
             v[0] += __uint_as_float(res[q].x << 16);
             v[1] += __uint_as_float(res[q].x & 0xffff0000u);
@@ -582,14 +600,14 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   // after a timeout: let the copies in flight land before the CTA ends
   if (*abort_s && elect_one()) {
     if (issued >= 0) mbar_wait(&sfull[issued % RXR], (issued / RXR) & 1);
-    if (NPROJ == 2 && warp == LEAD) mbar_wait(aux, 0);
+    if (NPROJ == 2 && !ROUTED && warp == LEAD) mbar_wait(aux, 0);
   }
 }
 
-template <int BITS, int NPROJ, int GROUP, int NT>
+template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED = false>
 cudaError_t launch_batch_t(const BatchArgs &a, int ctas, cudaStream_t s) {
   using C = BatchCfg<BITS, NPROJ, GROUP, NT>;
-  auto kern = batch_kernel<BITS, NPROJ, GROUP, NT>;
+  auto kern = batch_kernel<BITS, NPROJ, GROUP, NT, ROUTED>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -624,6 +642,26 @@ cudaError_t launch_batch_g(const BatchArgs &a, int nt, int ctas, cudaStream_t s)
     case 32: return launch_batch_n<BITS, NPROJ, 32>(a, nt, ctas, s);
     case 64: return launch_batch_n<BITS, NPROJ, 64>(a, nt, ctas, s);
     case 128: return launch_batch_n<BITS, NPROJ, 128>(a, nt, ctas, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int BITS, int NPROJ, int GROUP>
+cudaError_t launch_batch_routed_n(const BatchArgs &a, int nt, int ctas, cudaStream_t s) {
+  switch (nt) {
+    case 1: return launch_batch_t<BITS, NPROJ, GROUP, 1, true>(a, ctas, s);
+    case 2: return launch_batch_t<BITS, NPROJ, GROUP, 2, true>(a, ctas, s);
+    case 4: return launch_batch_t<BITS, NPROJ, GROUP, 4, true>(a, ctas, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int BITS, int NPROJ>
+cudaError_t launch_batch_routed_g(const BatchArgs &a, int nt, int ctas, cudaStream_t s) {
+  switch (a.group) {
+    case 32: return launch_batch_routed_n<BITS, NPROJ, 32>(a, nt, ctas, s);
+    case 64: return launch_batch_routed_n<BITS, NPROJ, 64>(a, nt, ctas, s);
+    case 128: return launch_batch_routed_n<BITS, NPROJ, 128>(a, nt, ctas, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -32,6 +32,19 @@ inline __host__ __device__ uint32_t batch_rec_bytes(int nt, int group) {
   return (uint32_t)nt * (2048u + 32u + 32u * (128u / (uint32_t)group));
 }
 
+// Slots of a routed call grouped by expert (written by launch_batch_route):
+// segment s holds slots list[seg[s].z .. + seg[s].y) of expert seg[s].x.
+constexpr int kRouteMaxSlots = 1024, kRouteMaxSegs = 1024;
+struct BatchRoute {
+  int n_segs;
+  int4 seg[kRouteMaxSegs];
+  int list[kRouteMaxSlots];
+};
+// Segments that m tokens of top_k choices can make at most.
+inline int batch_max_segs(int slots, int experts, int nt) {
+  return (slots < experts ? slots : experts) + slots / (8 * nt);
+}
+
 struct BatchArgs {
   const uint8_t *panel;      // [ceil(K / 128)] records
   int M, N, K, group;
@@ -50,7 +63,12 @@ struct BatchArgs {
   uint8_t *panel_out;        // gate/up: also the 4-bit down launch's panel of h (null: none)
   int group_out;             // its quantization group
   float *part;               // batch_scratch_floats() fp32
-  unsigned *cnt;             // [ceil(N / 128)] arrival counters, zero between launches
+  unsigned *cnt;             // [ceil(N / 128)] (routed: per segment) arrival counters, zero between launches
+  // Routed experts: the launch computes segments of up to 8 nt (token, choice)
+  // slots of one expert each.  codes, meta, lora_b: the experts' matrices
+  // stacked row-wise, N rows an expert (a multiple of 16); panel, tfrag, rs,
+  // panel_out: one per segment; out: one row a slot.
+  const BatchRoute *route;   // null: one dense matrix, M tokens
 };
 
 // Panel of x bf16 [M, K] for codes of `bits` bits and groups of `group`, and
@@ -58,15 +76,29 @@ struct BatchArgs {
 cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, const void *lora_a, int r,
                               float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, cudaStream_t s);
 cudaError_t launch_batch(GemvKind kind, const BatchArgs &a, cudaStream_t s);
-size_t batch_scratch_floats(int M, int nproj, int num_sms);
-size_t batch_tfrag_bytes(int M, int r);
+// Routed: the top_k experts of each token with their softmax weights (slot
+// t * top_k + j), and the slots grouped by expert in segments of 8 nt.
+cudaError_t launch_batch_route(const float *logits, int m, int E, int top_k, int nt, int *idx, float *w,
+                               BatchRoute *route, cudaStream_t s);
+// Panels, RMSNorm scales (rs not null) and LoRA-A products (tfrag not null) of
+// every segment; max_segs bounds the grid.
+cudaError_t launch_batch_route_prep(const void *x, int K, int bits, int group, int top_k, const void *lora_a, int r,
+                                    float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag,
+                                    const BatchRoute *route, int max_segs, int nt, cudaStream_t s);
+// Routed launch: nt 1, 2 or 4; max_segs for the grid.
+cudaError_t launch_batch_routed(GemvKind kind, const BatchArgs &a, int max_segs, int nt, cudaStream_t s);
+size_t batch_scratch_floats(int nt, int nproj, int num_sms);
+size_t batch_tfrag_bytes(int nt, int r);
 cudaError_t read_batch_status(int *status);
 
 // One translation unit per kind.
 cudaError_t launch_batch_gu2(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_gu2(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
 cudaError_t launch_batch_gu3(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
 cudaError_t launch_batch_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
 cudaError_t launch_batch_dn4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_dn4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
 cudaError_t read_batch_status_gu2(int *status);
 cudaError_t read_batch_status_gu3(int *status);
 cudaError_t read_batch_status_gu4(int *status);

@@ -2,7 +2,8 @@
 where their split can go wrong: every count of 8-token tiles and its edges,
 ragged row blocks and feature blocks, one unit to many parts a row block,
 adapter ranks that are no multiple of 16, every code width and group, rows
-that are no multiple of 4 (scalar stores), and the panel gate/up hands down.
+that are no multiple of 4 (scalar stores), the panel gate/up hands down, and
+the slots of a mixture of experts grouped by expert.
 
 Products are exact and sums fp32, so the bound and the share of bit-equal
 bf16 outputs are those of the other decode kernels (check_bf16's defaults).
@@ -123,3 +124,19 @@ def test_batch_stack_hands_down_the_panel(wq, bits, group, group_down, r, m):
         ref, _ = orc.down(synth.bf16_bits(h_states[l].cpu()), qd, group_down, prev)
         check_bf16(states[l], ref, f"batch stack bits={bits} m={m} layer {l} y")
         prev = synth.bf16_bits(states[l].cpu())
+
+
+@pytest.mark.parametrize("m,E,k,r,skew", [
+    (7, 8, 2, 8, 0.0),      # 14 slots, segments of up to 8
+    (33, 8, 2, 24, 0.0),    # 66 slots, segments of up to 16; rank 24
+    (64, 4, 3, 0, 0.0),     # 192 slots, segments of up to 32
+    (24, 32, 1, 8, 9.0),    # every token takes expert 0: three segments, 31 experts unread
+])
+def test_routed_batch(wq, m, E, k, r, skew):
+    from tests.test_gpu_moe import _build, _check_block
+    d, inter, group = 352, 224, 32  # ragged feature blocks and row blocks
+    layer, ents = _build(wq, d, inter, E, k, group, r, 300 + m)
+    x = synth.activations((m, d), 11 + m)
+    lg = np.random.default_rng(5 + m).standard_normal((m, E)).astype(np.float32)
+    lg[:, 0] += skew
+    _check_block(wq, layer, ents, x, torch.from_numpy(lg), group, f"routed m={m} E={E} k={k}", 2.0 if r else 0.0)
