@@ -7,6 +7,8 @@
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
+#include <array>
+#include <map>
 #include <mutex>
 #include <string>
 
@@ -194,8 +196,35 @@ void stack_layout(int m, int d, int inter, size_t off, WsLayout *L) {
   L->total = off;
 }
 
+// Results that depend on a few sizes only, kept because every call asks for
+// them again: a layout looks up over a hundred launch plans, and a workspace
+// size the layout of every token count up to m (a decoder layer of 16
+// sequences spent ~240 us a call on them, more than its launches take).
+// Bounded; safe with several host threads.
+template <class V, size_t N>
+class SizeMemo {
+ public:
+  using Key = std::array<int, N>;
+  bool find(const Key &k, V *v) {
+    std::lock_guard<std::mutex> lock(mu_);
+    const auto it = map_.find(k);
+    if (it == map_.end()) return false;
+    *v = it->second;
+    return true;
+  }
+  void put(const Key &k, const V &v) {
+    std::lock_guard<std::mutex> lock(mu_);
+    if (map_.size() >= 4096) map_.clear();
+    map_[k] = v;
+  }
+
+ private:
+  std::mutex mu_;
+  std::map<Key, V> map_;
+};
+
 // gemv_only: the decode path's buffers alone (the call without a workspace).
-bool ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only = false) {
+bool make_ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only) {
   *L = WsLayout{};
   size_t off = counter_block(d, inter, L);
   if (m > kMaxTokens) {
@@ -236,6 +265,14 @@ bool ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only = false) {
   return true;
 }
 
+bool ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only = false) {
+  static SizeMemo<WsLayout, 5> memo;
+  const SizeMemo<WsLayout, 5>::Key key{m, d, inter, gemv_only ? 1 : 0, num_sms()};
+  if (memo.find(key, L)) return true;
+  if (!make_ws_layout(m, d, inter, L, gemv_only)) return false;
+  memo.put(key, *L);
+  return true;
+}
 
 // Which kernels a call takes by its token count: the dequant-GEMM path above
 // kMaxTokens; the batched-decode launches above kBatchAbove, and below where
@@ -650,7 +687,10 @@ wq_status wq_merge_lora(const wq_qweight *src, const void *lora_b, const void *l
 size_t wq_workspace_bytes(int m, int d, int inter, int r) {
   (void)r;  // the LoRA-A product area is sized for the largest supported rank
   if (m <= 0 || d <= 0 || inter <= 0 || m > kMaxGemmTokens) return 0;
+  static SizeMemo<size_t, 4> memo;
+  const SizeMemo<size_t, 4>::Key key{m, d, inter, num_sms()};
   size_t most = 0;  // enough for every token count up to m
+  if (memo.find(key, &most)) return most;
   if (m > kMaxTokens) {
     WsLayout L;
     if (!ws_layout(m, d, inter, &L)) return 0;  // grows with m
@@ -661,6 +701,7 @@ size_t wq_workspace_bytes(int m, int d, int inter, int r) {
     if (!ws_layout(mm, d, inter, &L)) return 0;
     most = std::max(most, L.total);
   }
+  memo.put(key, most);
   return most;
 }
 
