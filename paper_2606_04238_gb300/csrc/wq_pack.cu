@@ -7,11 +7,15 @@
 // codes, scales and zeros are reproducible bit for bit:
 //   s = fp16((max - min) / qmax) (1.0 if zero), z = clamp(rint(-min/s), 0, qmax),
 //   q = clamp(rint(w/s) + z, 0, qmax).
-// Two kernels: one warp per (row, group) computes s and z into the packed
-// meta layout; then one thread per packed 32-bit word gathers its 16 (2-bit)
-// or 8 (4-bit) codes, or for 3-bit codes (App. B) 16 low-plane fields (q % 4)
-// or 32 high-plane bits (q / 4).  Offline work: not on the decode path.
-// A third kernel merges a trained adapter into a packed matrix before it is
+// One kernel, one warp per packed block of 16 rows x 128 features.  A lane
+// loads the features that its words of the packed layout hold (float2s; the 8
+// rows' sectors of an instruction are used in full), so each weight is read
+// once and the words are assembled in registers; min and max of a (row, group)
+// come from its 4 lanes by two shuffles.  Bound by HBM: 4 bytes in and bits/8
+// out a weight.  The per-weight division is a multiplication by the reciprocal
+// of s, with the exact division only where the product lies so near a rounding
+// boundary that the two could differ.  Offline work: not on the decode path.
+// A second kernel merges a trained adapter into a packed matrix before it is
 // quantized again (below).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -24,102 +28,90 @@
 namespace wq {
 namespace {
 
-__global__ void quant_meta_kernel(const float *__restrict__ w, int n, int k, int group, int bits, int RT, int NG,
-                                  uint16_t *__restrict__ meta, int *nonfinite) {
-  const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (long long)RT * 16 * NG) return;  // warp-uniform
-  const int row = (int)(gw / NG), j = (int)(gw % NG);
-  const int ngk = k / group;
-  unsigned short s16 = 0, z16 = 0;
-  if (row < n && j < ngk) {
-    const float *src = w + (size_t)row * k + (size_t)j * group;
-    float mn = INFINITY, mx = -INFINITY;
-    bool bad = false;
-    for (int i = lane; i < group; i += 32) {
-      const float v = src[i];
-      bad |= !isfinite(v);
-      mn = fminf(mn, v);
-      mx = fmaxf(mx, v);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    bad = __any_sync(0xffffffffu, bad);
-    const float qmax = (float)((1 << bits) - 1);
-    __half sh = __float2half_rn(__fdiv_rn(__fsub_rn(mx, mn), qmax));
-    if (__half2float(sh) == 0.f) sh = __float2half_rn(1.f);
-    const float sf = __half2float(sh);
-    const float zf = __fadd_rn(fminf(fmaxf(rintf(__fdiv_rn(-mn, sf)), 0.f), qmax), 0.f);
-    s16 = __half_as_ushort(sh);
-    z16 = __half_as_ushort(__float2half_rn(zf));
-    if (bad && lane == 0 && nonfinite) atomicOr(nonfinite, 1);
-  }
-  if (lane == 0) {
-    const int rt = row >> 4, i = row & 15;
-    const size_t base = ((size_t)rt * NG + j) * 32 + 4 * (i & 7) + (i >> 3);
-    meta[base] = s16;
-    meta[base + 2] = z16;
-  }
+constexpr int kPackWarps = 8;  // blocks a CTA
+
+// rint(v / sf) as the IEEE division gives it.  p = v * rcp is within |p| 2^-22
+// of the quotient (two roundings), as is the division's own result, so both
+// round to the same integer unless p is that near to a half.
+__device__ __forceinline__ float rint_div(float v, float sf, float rcp) {
+  const float p = __fmul_rn(v, rcp), r = rintf(p);
+  if (fabsf(p - r) < 0.5f - fabsf(p) * 0x1p-21f) return r;
+  return rintf(__fdiv_rn(v, sf));  // also nan and infinite quotients
 }
 
-__global__ void pack_codes_kernel(const float *__restrict__ w, int n, int k, int group, int bits, int RT, int KB,
-                                  int NG, const uint16_t *__restrict__ meta, uint32_t *__restrict__ codes) {
-  const int WPB = bits == 2 ? 128 : bits == 3 ? 192 : 256;
-  const size_t wid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (wid >= (size_t)RT * KB * WPB) return;
-  const size_t blk = wid / WPB;
-  const int wl = (int)(wid % WPB);
-  const int rt = (int)(blk / KB), kb = (int)(blk % KB);
-  const float qmax = (float)((1 << bits) - 1);
-  // code of (local row i, block feature c), or 0 outside the matrix
-  auto code_at = [&](int i, int c) -> uint32_t {
-    const int row = rt * 16 + i, col = kb * 128 + c;
-    if (row >= n || col >= k) return 0u;
-    const size_t mb = ((size_t)rt * NG + col / group) * 32 + 4 * (i & 7) + (i >> 3);
-    const float sf = __half2float(__ushort_as_half(meta[mb]));
-    const float zf = __half2float(__ushort_as_half(meta[mb + 2]));
-    return (uint32_t)fminf(fmaxf(__fadd_rn(rintf(__fdiv_rn(w[(size_t)row * k + col], sf)), zf), 0.f), qmax);
-  };
-  if (bits == 3) {
-    uint32_t word = 0;
-    if (wl < 128) {  // low plane: q % 4 where a 2-bit code would sit
-      const int lane = wl >> 2, wi = wl & 3;
-      for (int bit = 0; bit < 32; bit += 2) {
-        const int half = bit >> 4, rowhalf = (bit >> 3) & 1, cls = (bit & 7) >> 1;
-        const int c = wi * 32 + (cls >> 1) * 16 + (cls & 1) * 8 + (lane & 3) * 2 + half;
-        word |= (code_at((lane >> 2) + 8 * rowhalf, c) & 3u) << bit;
-      }
-    } else {  // high plane: word 128 + 2 lane + p holds q / 4 of the features c with (c / 32) / 2 = p
-      const int lane = (wl - 128) >> 1, pp = (wl - 128) & 1;
-      for (int bit = 0; bit < 32; ++bit) {
-        const int half = bit >> 4, cpar = (bit >> 3) & 1, cls = (bit & 7) >> 1, ihi = bit & 1;
-        const int c = (2 * pp + cpar) * 32 + (cls >> 1) * 16 + (cls & 1) * 8 + (lane & 3) * 2 + half;
-        word |= (code_at((lane >> 2) + 8 * ihi, c) >> 2) << bit;
-      }
-    }
-    codes[wid] = word;
-    return;
+template <int BITS, int GROUP>
+__global__ void __launch_bounds__(kPackWarps * 32) pack_kernel(const float *__restrict__ w, int n, int k, int RT, int KB,
+                                                               uint32_t *__restrict__ codes,
+                                                               uint16_t *__restrict__ meta, int *nonfinite) {
+  constexpr int WPB = BITS * 64, GPB = 128 / GROUP, JG = GROUP / 8;  // code words a block, groups, 8-feature steps a group
+  const long long blk = (long long)blockIdx.x * kPackWarps + (threadIdx.x >> 5);
+  if (blk >= (long long)RT * KB) return;  // warp-uniform
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int rt = (int)(blk / KB), kb = (int)(blk - (long long)rt * KB);
+  const int nj = min(16, (k - kb * 128) / 8);  // 8-feature steps inside the matrix (k a multiple of the group)
+  // rows g and g + 8 of the tile, features 8 j + 2 t, + 1 of the block
+  float2 v[2][16];
+  bool in[2], bad = false;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int row = rt * 16 + g + 8 * h;
+    in[h] = row < n;
+    const float *src = w + (size_t)(in[h] ? row : 0) * k + kb * 128 + 2 * t;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      v[h][j] = in[h] && j < nj ? __ldcs(reinterpret_cast<const float2 *>(src + 8 * j)) : make_float2(0.f, 0.f);
   }
-  const int tile = bits == 2 ? 0 : wl >> 7;  // 64-feature half of a 4-bit block
-  const int wl2 = wl & 127;
-  const int lane = wl2 >> 2, wi = wl2 & 3;
-  uint32_t word = 0;
-  for (int bit = 0; bit < 32; bit += bits) {
-    const int half = bit >> 4, rowhalf = (bit >> 3) & 1;
-    int c;
-    if (bits == 2) {
-      const int cls = (bit & 7) >> 1;  // 2 * (16-feature step parity) + (upper 8 features)
-      c = wi * 32 + (cls >> 1) * 16 + (cls & 1) * 8 + (lane & 3) * 2 + half;
-    } else {
-      const int hi = (bit & 7) >> 2;
-      c = tile * 64 + wi * 16 + hi * 8 + (lane & 3) * 2 + half;
+  const float qmax = (float)((1 << BITS) - 1);
+  uint32_t lo[BITS == 4 ? 8 : 4] = {}, hi[2] = {};
+#pragma unroll
+  for (int gi = 0; gi < GPB; ++gi) {
+    unsigned short s16[2], z16[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float mn = INFINITY, mx = -INFINITY;
+#pragma unroll
+      for (int j = gi * JG; j < (gi + 1) * JG; ++j) {
+        mn = fminf(mn, fminf(v[h][j].x, v[h][j].y));
+        mx = fmaxf(mx, fmaxf(v[h][j].x, v[h][j].y));
+        bad |= !isfinite(v[h][j].x) || !isfinite(v[h][j].y);
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      __half sh = __float2half_rn(__fdiv_rn(__fsub_rn(mx, mn), qmax));
+      if (__half2float(sh) == 0.f) sh = __float2half_rn(1.f);
+      const float sf = __half2float(sh);
+      const float zf = __fadd_rn(fminf(fmaxf(rintf(__fdiv_rn(-mn, sf)), 0.f), qmax), 0.f);
+      const bool real = in[h] && gi * JG < nj;  // codes, scale and zero are 0 outside the matrix
+      s16[h] = real ? __half_as_ushort(sh) : 0;
+      z16[h] = real ? __half_as_ushort(__float2half_rn(zf)) : 0;
+      const float rcp = __frcp_rn(sf);
+#pragma unroll
+      for (int j = gi * JG; j < (gi + 1) * JG; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float q = fminf(fmaxf(__fadd_rn(rint_div(e ? v[h][j].y : v[h][j].x, sf, rcp), zf), 0.f), qmax);
+          const uint32_t c = real ? (uint32_t)q : 0u;
+          if (BITS == 4) {
+            lo[j >> 1] |= c << (16 * e + 8 * h + 4 * (j & 1));
+          } else {
+            lo[j >> 2] |= (c & 3u) << (16 * e + 8 * h + 2 * (j & 3));
+            if (BITS == 3) hi[j >> 3] |= (c >> 2) << (16 * e + 8 * ((j >> 2) & 1) + 2 * (j & 3) + h);
+          }
+        }
     }
-    word |= code_at((lane >> 2) + 8 * rowhalf, c) << bit;
+    if (t == 0) {
+      const uint2 m2 = make_uint2((uint32_t)s16[0] | ((uint32_t)s16[1] << 16), (uint32_t)z16[0] | ((uint32_t)z16[1] << 16));
+      *reinterpret_cast<uint2 *>(meta + (((size_t)rt * KB + kb) * GPB + gi) * 32 + 4 * g) = m2;
+    }
   }
-  codes[wid] = word;
+  uint32_t *dst = codes + (size_t)blk * WPB;
+  *reinterpret_cast<uint4 *>(dst + lane * 4) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  if (BITS == 4) *reinterpret_cast<uint4 *>(dst + 128 + lane * 4) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+  if (BITS == 3) *reinterpret_cast<uint2 *>(dst + 128 + lane * 2) = make_uint2(hi[0], hi[1]);
+  if (nonfinite != nullptr && __any_sync(0xffffffffu, bad) && lane == 0) atomicOr(nonfinite, 1);
 }
 
 // Adapter merge (Sec. 4.2 lets the trained adapters be merged into the
@@ -188,18 +180,27 @@ cudaError_t launch_merge_lora(const uint32_t *codes, const uint16_t *meta, int n
   return cudaGetLastError();
 }
 
+template <int BITS>
+static void launch_pack_g(const float *w, int n, int k, int group, uint32_t *codes, uint16_t *meta, int *nonfinite,
+                          cudaStream_t stream) {
+  const int RT = (n + 15) / 16, KB = (k + 127) / 128;
+  const unsigned ctas = (unsigned)(((long long)RT * KB + kPackWarps - 1) / kPackWarps);
+  if (group == 32)
+    pack_kernel<BITS, 32><<<ctas, kPackWarps * 32, 0, stream>>>(w, n, k, RT, KB, codes, meta, nonfinite);
+  else if (group == 64)
+    pack_kernel<BITS, 64><<<ctas, kPackWarps * 32, 0, stream>>>(w, n, k, RT, KB, codes, meta, nonfinite);
+  else
+    pack_kernel<BITS, 128><<<ctas, kPackWarps * 32, 0, stream>>>(w, n, k, RT, KB, codes, meta, nonfinite);
+}
+
 cudaError_t launch_pack(const float *w, int n, int k, int group, int bits, uint32_t *codes, uint16_t *meta,
                         int *nonfinite, cudaStream_t stream) {
-  const int RT = (n + 15) / 16, KB = (k + 127) / 128, NG = KB * 128 / group;
-  const long long warps = (long long)RT * 16 * NG;
-  const int tpb = 256;
-  quant_meta_kernel<<<(unsigned)((warps * 32 + tpb - 1) / tpb), tpb, 0, stream>>>(w, n, k, group, bits, RT, NG, meta,
-                                                                                 nonfinite);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const long long words = (long long)RT * KB * (bits == 2 ? 128 : bits == 3 ? 192 : 256);
-  pack_codes_kernel<<<(unsigned)((words + tpb - 1) / tpb), tpb, 0, stream>>>(w, n, k, group, bits, RT, KB, NG, meta,
-                                                                             codes);
+  if (bits == 2)
+    launch_pack_g<2>(w, n, k, group, codes, meta, nonfinite, stream);
+  else if (bits == 3)
+    launch_pack_g<3>(w, n, k, group, codes, meta, nonfinite, stream);
+  else
+    launch_pack_g<4>(w, n, k, group, codes, meta, nonfinite, stream);
   return cudaGetLastError();
 }
 
