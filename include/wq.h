@@ -22,15 +22,16 @@
  *   - Supported: group in {32, 64, 128}; in-features a multiple of the group
  *     (WQ_ERR_SHAPE otherwise); 1 <= m <= 16384 tokens (m == 0 is a no-op);
  *     LoRA rank r a multiple of 8, r <= 64 (r == 0: no adapter).
- *   - Three paths behind the same calls: up to 8 tokens the dequant-GEMV
- *     kernels, up to 64 tokens (and below, for a layer shape the GEMV kernels
- *     have no launch configuration for) the batched-decode kernels -- both
- *     form exact products of the codes and binary16 activations on the
- *     mma.sync tensor-core path and sum in fp32 -- and above 64 tokens the
- *     batched dequant-GEMM on the tcgen05 tensor cores (activations and each
- *     dequantized weight s (q - z) rounded once to binary16, fp32
- *     accumulation; with fp32 output of wq_down_w4 the weights enter as two
- *     exact binary16 parts).  The workspace size covers the path a call takes.
+ *   - Three paths behind the same calls.  Up to 8 tokens the dequant-GEMV
+ *     kernels; up to 64 tokens (for large matrices already from one to three
+ *     tokens on, and for a layer shape the GEMV kernels have no launch
+ *     configuration for) the batched-decode kernels -- both form exact products
+ *     of the codes and binary16 activations on the mma.sync tensor-core path
+ *     and sum in fp32 -- and above 64 tokens the batched dequant-GEMM on the
+ *     tcgen05 tensor cores (activations and each dequantized weight s (q - z)
+ *     rounded once to binary16, fp32 accumulation; with fp32 output of
+ *     wq_down_w4 the weights enter as two exact binary16 parts).  The workspace
+ *     size covers the path a call takes.
  *   - On error the call returns a negative wq_status and wq_last_error()
  *     describes it (per host thread).  Kernel-side waits are bounded; a wait
  *     that runs out records WQ_ERR_TIMEOUT, read back by wq_device_status().
@@ -288,12 +289,13 @@ wq_status wq_down_bf16(const void *h, int m, const void *wd, int d, int inter, c
  *   - the single-launch stack kernel: every layer in one cooperative launch
  *     (one CTA per SM; up to 32 layers a launch), for 1..8 tokens when every
  *     layer has the same bits, groups and rank, where it is the measured-faster
- *     route (2-bit gate/up at 2..8 tokens, or d >= 4096) or WQ_LAUNCH_STACK asks;
+ *     route (2-bit gate/up: 2..8 tokens, or one token at d 4096) or
+ *     WQ_LAUNCH_STACK asks;
  *   - the launch chain: 2 kernels per layer (plus one for the first layer's
  *     input statistics) with programmatic dependent launch, each down launch
  *     also producing the next layer's RMSNorm and LoRA-A partial sums;
- *   - the batched chain above 16 tokens (8 for d >= 4096): the dequant-GEMM
- *     above 64 tokens.  From 9 to 64 tokens both chains run the batched-decode
+ *   - the batched chain above 16 tokens (8 for d >= 4096; fewer where a layer's
+ *     matrices have 50M weights and more): the dequant-GEMM above 64 tokens.  From 9 to 64 tokens both chains run the batched-decode
  *     kernels: per layer the activation panel of x with its RMSNorm scales and
  *     LoRA-A products, gate/up (which leaves the panel of h), down.
  * Every route can be captured into a CUDA graph.

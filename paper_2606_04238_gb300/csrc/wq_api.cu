@@ -108,13 +108,43 @@ size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 // more (where one token's share of the GEMV kernels' work is largest).
 int gemv_prefer_tokens(int d) { return d >= 4096 ? 8 : kGemvPreferTokens; }
 
-// Above this many tokens (to kBatchMaxTokens) the launches are the
-// batched-decode ones.  Measured at the line (us a layer, W2 g128, kernels
-// before vs batched): d 2560 at 9 tokens 35.3 (GEMV) vs 26.7, d 4096 102.7
-// (tcgen05) vs 41.1, d 5120 135.8 vs 51.7; 64 tokens 75.7, 110.8 and 145.4
-// (tcgen05) vs 52.0, 89.8 and 121.3.  Above 64 tokens each weight's expansion
-// for tcgen05 is shared by 128 and more tokens.
-constexpr int kBatchAbove = 8;
+// Above these token counts (to kBatchMaxTokens) the launches are the
+// batched-decode ones.  The GEMV kernels convert the activations and add up
+// k-split sums in every CTA, work that grows with the token count; the batched
+// ones cost the same from 1 to 8 tokens, plus the input launch.  The lines
+// follow the weights of a launch, measured (us, GEMV or stack kernel vs
+// batched; W2 g128 unless said):
+//   gate/up: 49.8M weights (d 2560, inter 9728) 1 token 11.0 vs 11.2, 2 tokens
+//     15.2 vs 11.3, 8 tokens 20.6 vs 11.1; 117M (d 4096) 1 token 23.9 vs 22.1;
+//     178M (d 5120) 30.2 vs 25.1; 5.8M 4 tokens 8.3 vs 8.4, 8 tokens 12.3 vs 7.9;
+//   down: 24.9M 8 tokens 11.7 vs 12.5; 58.7M 2 tokens 13.4 vs 15.1, 3 tokens 32
+//     vs 14.7; 89M 1 token 19.9 vs 16.7; a 15.7M projection 8 tokens 9.7 vs 9.7;
+//   a layer of a stack: d 4096 1 token 32.9 vs 33.5, 2 tokens 37.6 vs 33.6, 8
+//     tokens 69 vs 33.5 (W3 g32 1 token 49.9 vs 42.1, W4 35.4 vs 33.3); d 5120
+//     1 token 48.2 vs 41.4; d 2560 W4 5 tokens 22.7 vs 23.8, 6 tokens 24.6 vs
+//     23.9 (W3 g32 5 tokens 27.4 vs 27.4); at 9 tokens 35.3 vs 26.7, and above
+//     64 tokens each weight's expansion for tcgen05 is shared by 128 and more.
+int gateup_batch_above(const wq_qweight &gate) {
+  const long long w = 2LL * gate.n * gate.k;
+  return w >= 100000000 ? 0 : w >= 30000000 ? 1 : 8;
+}
+int down_batch_above(const wq_qweight &down) {
+  const long long w = (long long)down.n * down.k;
+  return w >= 80000000 ? 0 : w >= 50000000 ? 2 : 8;
+}
+int layer_batch_above(const wq_mlp_layer &l) {
+  const long long w = (long long)l.gate.n * l.gate.k;
+  if (w >= 80000000) return 0;
+  if (w >= 50000000) return l.gate.bits == 2 ? 1 : 0;
+  return w >= 20000000 && l.gate.bits != 2 ? 5 : 8;
+}
+// A stack takes them when every layer does.
+bool stack_takes_batch(int m, const wq_mlp_layer *layers, int n_layers) {
+  if (m > kBatchMaxTokens) return false;
+  for (int l = 0; l < n_layers; ++l)
+    if (m <= layer_batch_above(layers[l])) return false;
+  return true;
+}
 
 size_t partial_bytes(const GemvPlan &p, int nproj) {
   return p.P > 1 ? (size_t)p.RT * p.P * nproj * 16 * p.M * 4 : 0;
@@ -248,9 +278,7 @@ bool make_ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only) {
   L->part2 = off; off = up256(off + p2);
   L->total = off;
   if (gemv_only) return true;
-  // above kBatchAbove, or for a shape that lacks a GEMV plan for some group or
-  // rank at this token count, the calls take the batched-decode path
-  if (m > kBatchAbove || !all_fit) {
+  {  // the batched-decode path's
     const int sms = num_sms(), nt = batch_nt(m);
     if (sms <= 0) return false;
     L->bpx = off;   off = up256(off + (size_t)((std::max(d, inter) + 127) / 128) * batch_rec_bytes(nt, 32));
@@ -275,19 +303,20 @@ bool ws_layout(int m, int d, int inter, WsLayout *L, bool gemv_only = false) {
 }
 
 // Which kernels a call takes by its token count: the dequant-GEMM path above
-// kMaxTokens; the batched-decode launches above kBatchAbove, and below where
-// the GEMV kernels have no launch plan; the GEMV kernels otherwise.
+// kMaxTokens; the batched-decode launches above gateup_batch_above /
+// down_batch_above, and below where the GEMV kernels have no launch plan; the
+// GEMV kernels otherwise.
 enum class Path { kGemv, kBatch, kGemm };
 Path gateup_path(GemvKind kind, int m, const wq_qweight *gate, int r) {
   if (m > kMaxTokens) return Path::kGemm;
   GemvPlan pl;
-  return m > kBatchAbove || !plan_gemv(kind, gate->n, gate->k, m, gate->group, r, num_sms(), &pl) ? Path::kBatch
+  return m > gateup_batch_above(*gate) || !plan_gemv(kind, gate->n, gate->k, m, gate->group, r, num_sms(), &pl) ? Path::kBatch
                                                                                                   : Path::kGemv;
 }
 Path down_path(int m, const wq_qweight *down, int r_next) {
   if (m > kMaxTokens) return Path::kGemm;
   GemvPlan pl;
-  return m > kBatchAbove || !plan_gemv(kDownW4, down->n, down->k, m, down->group, r_next, num_sms(), &pl)
+  return m > down_batch_above(*down) || !plan_gemv(kDownW4, down->n, down->k, m, down->group, r_next, num_sms(), &pl)
              ? Path::kBatch : Path::kGemv;
 }
 
@@ -882,8 +911,9 @@ wq_status check_stack(int m, const wq_mlp_layer *layers, int n_layers, unsigned 
 // batched launch chain (above gemv_prefer_tokens tokens, or where some layer
 // has no GEMV plan), or the single-launch stack kernel (1..8 tokens, every
 // layer with the same bits, groups and rank, unless the caller asks for the
-// chain).  Both chains take the batched-decode launches for more than
-// kBatchAbove and up to kBatchMaxTokens tokens.
+// chain).  From 9 to kBatchMaxTokens tokens both chains take the batched-decode
+// launches, and so does the batched chain below, which large layers take from
+// fewer tokens on (stack_takes_batch).
 enum StackRoute { kRouteGemvChain = 0, kRouteGemmChain = 1, kRouteStack = 2 };
 
 bool cooperative_ok() {
@@ -921,6 +951,8 @@ bool stack_preferred(int m, const wq_mlp_layer &L0) { return L0.gate.bits == 2 &
 
 StackRoute stack_route(int m, const wq_mlp_layer *layers, int n_layers, unsigned flags) {
   StackPlan sp;
+  const bool batch = stack_takes_batch(m, layers, n_layers);
+  if (m <= 8 && batch && !(flags & (WQ_LAUNCH_STACK | WQ_LAUNCH_CHAIN))) return kRouteGemmChain;
   if (((flags & WQ_LAUNCH_STACK) || stack_preferred(m, layers[0])) && stack_kernel_plan(m, layers, n_layers, flags, &sp))
     return kRouteStack;
   for (int l = 0; l < n_layers; ++l)
@@ -929,9 +961,11 @@ StackRoute stack_route(int m, const wq_mlp_layer *layers, int n_layers, unsigned
   for (int l = 0; l < n_layers; ++l) {
     const wq_mlp_layer &Ly = layers[l];
     const bool next_tp = l + 1 < n_layers && ((flags & WQ_PRENORM) || layers[l + 1].r > 0);
-    if (m > kBatchAbove) continue;  // the batched-decode launches take every shape
-    if (gateup_path(gateup_kind(Ly.gate.bits), m, &Ly.gate, Ly.r) != Path::kGemv ||
-        (Ly.down.bits == 4 && down_path(m, &Ly.down, next_tp ? layers[l + 1].r : 0) != Path::kGemv))
+    if (m > 8) continue;  // the batched-decode launches take every shape
+    GemvPlan pl;
+    if (!plan_gemv(gateup_kind(Ly.gate.bits), Ly.gate.n, Ly.gate.k, m, Ly.gate.group, Ly.r, num_sms(), &pl) ||
+        (Ly.down.bits == 4 && !plan_gemv(kDownW4, Ly.down.n, Ly.down.k, m, Ly.down.group,
+                                         next_tp ? layers[l + 1].r : 0, num_sms(), &pl)))
       return kRouteGemmChain;
   }
   return kRouteGemvChain;
@@ -1021,7 +1055,7 @@ wq_status mlp_forward_impl(const void *x, int m, const wq_mlp_layer *layers, int
     }
     return ok();
   }
-  if (m <= kBatchMaxTokens && (m > kBatchAbove || route == kRouteGemmChain)) {
+  if (m <= kBatchMaxTokens && (m > 8 || route == kRouteGemmChain)) {
     // batched-decode chain: per layer the panel of x with its RMSNorm scales
     // and LoRA-A products, gate/up (which leaves the panel of h), down
     const void *cur = x;
@@ -1142,7 +1176,7 @@ wq_status wq_mlp_forward_info(int m, const wq_mlp_layer *layers, int n_layers, u
   if (route == kRouteGemvChain) {
     const wq_mlp_layer &L0 = layers[0];
     const GemvKind kind = gateup_kind(L0.gate.bits);
-    if (m > kBatchAbove) {  // the batched-decode launches have no GEMV plan; gate/up leaves the down launch's panel
+    if (m > 8) {  // the batched-decode launches have no GEMV plan; gate/up leaves the down launch's panel
       info[13] = L0.down.bits == 4 ? 1 : 0;
       return ok();
     }
@@ -1275,10 +1309,12 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
     const GemvKind kind = gateup_kind(bits);
     const bool need_tp = (flags & WQ_PRENORM) || M.r > 0;
     const int r_o = need_tp ? M.r : 0;
-    const bool gemv = gu_ok && gateup_path(kind, batch, &M.gate, M.r) == Path::kGemv &&
-                      down_path(batch, &M.down, 0) == Path::kGemv && down_path(batch, &Ly.o, r_o) == Path::kGemv &&
-                      (r_o == 0 || d % 8 == 0);
-    const bool batched = gu_ok && batch > kBatchAbove && batch <= kBatchMaxTokens;
+    const bool batched = gu_ok && stack_takes_batch(batch, &M, 1);
+    GemvPlan pl;
+    const bool gemv = gu_ok && !batched && batch <= 8 && (r_o == 0 || d % 8 == 0) &&
+                      plan_gemv(kind, inter, d, batch, M.gate.group, M.r, num_sms(), &pl) &&
+                      plan_gemv(kDownW4, d, inter, batch, M.down.group, 0, num_sms(), &pl) &&
+                      plan_gemv(kDownW4, d, H * hd, batch, Ly.o.group, r_o, num_sms(), &pl);
     if (gemv || batched) {
       if (!y) return fail(WQ_ERR_ARG, "null y");
       if (!aligned16(y)) return fail(WQ_ERR_ALIGN, "y not 16-byte aligned");

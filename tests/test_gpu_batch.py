@@ -1,4 +1,4 @@
-"""The batched-decode kernels (9 to 64 tokens) vs the fp64 oracle at the sizes
+"""The batched-decode kernels (9 to 64 tokens, fewer for large matrices) vs the fp64 oracle at the sizes
 where their split can go wrong: every count of 8-token tiles and its edges,
 ragged row blocks and feature blocks, one unit to many parts a row block,
 adapter ranks that are no multiple of 16, every code width and group, rows
@@ -40,6 +40,7 @@ GATEUP = [
     (3, 640, 384, 32, 16, (9, 31, 57)),
     (3, 512, 200, 128, 64, (16, 48)),
     (4, 1152, 264, 64, 0, (24, 40, 64)),
+    (2, 2560, 6144, 128, 16, (2, 8)),          # few tokens: launches of 30M weights and more
 ]
 
 
@@ -72,6 +73,7 @@ DOWN = [
     (202, 1056, 32, (12, 64)),        # rows no multiple of 4; ragged feature block
     (130, 20480, 128, (17, 63)),      # 2 row blocks, 160 blocks: about 76 parts each
     (2560, 704, 64, (32, 33)),
+    (4096, 20480, 128, (1, 3)),       # few tokens: 80M weights and more
 ]
 
 
@@ -140,3 +142,23 @@ def test_routed_batch(wq, m, E, k, r, skew):
     lg = np.random.default_rng(5 + m).standard_normal((m, E)).astype(np.float32)
     lg[:, 0] += skew
     _check_block(wq, layer, ents, x, torch.from_numpy(lg), group, f"routed m={m} E={E} k={k}", 2.0 if r else 0.0)
+
+
+@pytest.mark.parametrize("bits,m", [(2, 2), (3, 1)])
+def test_batch_stack_of_a_large_layer(wq, bits, m):
+    """One layer of 50M weights a matrix takes the batched chain at a few tokens."""
+    d, inter, group, r = 4096, 12800, 128, 8
+    qg, qu, qd = _q((inter, d), group, bits, 1), _q((inter, d), group, bits, 2), _q((d, inter), group, 4, 3)
+    a, bg, bu = synth.lora(d, inter, r, 4)
+    layer = wq.MLPLayer(upload_packed(*qg, group, bits), upload_packed(*qu, group, bits), upload_packed(*qd, group, 4),
+                        lora_a=a.cuda(), lora_b_gate=bg.cuda(), lora_b_up=bu.cuda(), lora_scale=2.0)
+    assert wq.mlp_forward_info(m, [layer])["route"] == wq.ROUTE_GEMM_CHAIN
+    x = synth.activations((m, d), 5).cuda()
+    y, _, h = wq.mlp_forward_states(x, [layer], prenorm=True, with_h=True)
+    torch.cuda.synchronize()
+    assert wq.device_status() == 0
+    bl = tuple(synth.bf16_bits(t) for t in (a, bg, bu))
+    ref, _ = orc.gateup(synth.bf16_bits(x.cpu()), qg, qu, group, *bl, lora_scale=2.0, prenorm=True)
+    check_bf16(h[0], ref, f"large layer h bits={bits} m={m}")
+    ref, _ = orc.down(synth.bf16_bits(h[0].cpu()), qd, group, synth.bf16_bits(x.cpu()))
+    check_bf16(y, ref, f"large layer y bits={bits} m={m}")
