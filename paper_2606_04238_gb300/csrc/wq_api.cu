@@ -86,7 +86,7 @@ wq_status check_down(const wq_qweight *q) {
 struct WsLayout {
   // arrival counters: at fixed offsets for every token count (zero once, kept
   // at zero -- or, for the stack kernel's, at a multiple of its grid -- by the calls)
-  size_t cnt1, cnt2, sctr, sk_cnt;
+  size_t cnt1, cnt2, sctr, bcnt;
   size_t tp, xa, xb, h, hq, hsc, hxs, part1, part2;
   // dequant-GEMM path (m > kMaxTokens)
   size_t x16, rs, ta, h16, hsx, sk_part;
@@ -183,14 +183,13 @@ bool max_partials(int m, int d, int inter, size_t *p1, size_t *p2, bool *all_fit
 
 // The counter block every layout starts with: the GEMV split-panel counters
 // of gate/up and down, the stack kernel's grid-barrier counter and the
-// stream-K tile counters of the GEMM path (sized for its largest token count).
+// batched-decode row blocks' arrival counters.
 size_t counter_block(int d, int inter, WsLayout *L) {
   size_t off = 0;
   L->cnt1 = off;   off = up256(off + (size_t)((inter + 15) / 16) * 4);
   L->cnt2 = off;   off = up256(off + (size_t)((d + 15) / 16) * 4);
   L->sctr = off;   off = up256(off + 8);
-  const size_t cnt = std::max(gemm_counters(kMaxGemmTokens, inter), gemm_counters(kMaxGemmTokens, d));
-  L->sk_cnt = off; off = up256(off + cnt * 4);
+  L->bcnt = off;  off = up256(off + (size_t)((std::max(d, inter) + 127) / 128) * 4);
   return off;
 }
 
@@ -470,7 +469,7 @@ wq_status run_gateup_batch(GemvKind kind, const void *x, int m, const wq_qweight
   a.panel_out = panel_down ? ws + L.bph : nullptr;
   a.group_out = panel_down ? panel_down->group : 128;
   a.part = reinterpret_cast<float *>(ws + L.bpart);
-  a.cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
+  a.cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
   if ((e = launch_batch(kind, a, s)) != cudaSuccess) return cuda_fail(e, "batched gate/up launch");
   return WQ_OK;
 }
@@ -495,7 +494,7 @@ wq_status run_down_batch(const void *h, int m, const wq_qweight *down, const voi
   a.out = y;
   a.out_f32 = y_f32;
   a.part = reinterpret_cast<float *>(ws + L.bpart);
-  a.cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
+  a.cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
   if ((e = launch_batch(kDownW4, a, s)) != cudaSuccess) return cuda_fail(e, "batched down launch");
   return WQ_OK;
 }
@@ -533,7 +532,6 @@ wq_status run_gateup_gemm(GemvKind kind, const void *x, int m, const wq_qweight 
   a.rs = rs;
   a.out = h;
   a.sk_part = reinterpret_cast<float *>(ws + L.sk_part);
-  a.sk_cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
   e = launch_gemm(kind, a, s);
   if (e != cudaSuccess) return cuda_fail(e, "gate/up GEMM launch");
   return WQ_OK;
@@ -562,7 +560,6 @@ wq_status run_down_gemm(const void *h, int m, const wq_qweight *down, const void
   a.out = y;
   a.out_f32 = y_f32;
   a.sk_part = reinterpret_cast<float *>(ws + L.sk_part);
-  a.sk_cnt = reinterpret_cast<unsigned *>(ws + L.sk_cnt);
   e = launch_gemm(kDownW4, a, s);
   if (e != cudaSuccess) return cuda_fail(e, "down GEMM launch");
   return WQ_OK;

@@ -10,11 +10,13 @@
 //     h = SiLU(rs D_g) * (rs D_u) with rs the RMSNorm scale of the token;
 //   * down: y = residual + h deq(Wd)^T.
 // A CTA computes a tile of 128 or 256 tokens x 128 output rows (x 2
-// projections for gate/up) over the whole feature axis, 64 features (half a
+// projections for gate/up; down may take 256 rows) over the whole feature axis, 64 features (half a
 // block of the packed format) per pipeline stage; with 256 tokens the two
 // halves of 128 multiply the same dequantized B tile into accumulators of
 // their own, so each weight is dequantized once per 256 tokens.  Warp roles:
-//   warps 0..15 dequantize the stage's codes: code q of row n, group j gives
+//   warps 0..15 dequantize, in two groups of 8 that take alternate stages (a
+//               group's hand-overs and load latencies then have two stages):
+//               code q of row n, group j gives
 //               the binary16 value s_nj (q - z_nj), rounded once; they write
 //               it in the tcgen05 K-major layout (8-row x 16-byte core
 //               matrices), then run the epilogue from TMEM;
@@ -27,13 +29,19 @@
 //               the 62 ns the tensor pipe needs for one of 128 x 256 x 16, so
 //               the issuing thread bounded the main loop (a layer of d 5120,
 //               inter 17408 at 512 tokens: 327 us, with elect.sync 282 us; of
-//               d 2560, inter 9728 at 3001 tokens: 512 us, now 454 us);
+//               d 2560, inter 9728 at 3001 tokens: 512 us, then 454 us);
 //   warp 18     loads the packed codes and scales/zeros of the CTA's 8 row
 //               tiles (TMA, one box each per projection and block) into their
 //               own ring.
 // The activation tiles, the B tiles and the packed codes have rings of their
 // own depths: each slot is released by what last reads it (the MMAs' commit,
 // or the dequantizing warps for the codes).
+// What bounds it now (clock stamps, gate/up): a stage of 64 features takes ~1100
+// clocks where its MMAs need 1024, a tile ~4400 before its first MMA and ~7800
+// for its epilogue, half of them the 2 x 32768 exponentials and reciprocals.
+// Measured with 256-row down tiles, the reduction kernel, 3 B tiles and the
+// sector-wide stores: the d 5120 layer at 512 tokens 212 us, the d 2560 layer at
+// 3001 tokens 364 us.
 // Stages are handed over with mbarriers; every wait is bounded (a timeout
 // sets the device status word and the CTA skips the rest of its work).
 #include <algorithm>
@@ -55,7 +63,8 @@ namespace {
 
 constexpr int kBM = 128;                         // tokens per CTA tile (MMA M)
 constexpr int kBN = 128;                         // output rows per CTA tile and projection (MMA N)
-constexpr int kDeqWarps = 16;                    // dequantizing warps
+constexpr int kDeqWarps = 16;                    // dequantizing warps, two groups that take alternate stages
+constexpr int kDeqGroup = kDeqWarps / 2;
 constexpr int kProducerWarp = kDeqWarps;         // activation tiles
 constexpr int kMmaWarp = kDeqWarps + 1;          // TMEM owner and MMA issuer
 constexpr int kRawWarp = kDeqWarps + 2;          // packed-code ring
@@ -76,26 +85,34 @@ struct GemmCfg {
   static constexpr int BPK = BITS == 2 ? 512 : 1024;      // code bytes per (16-row tile, block)
   static constexpr int GPB = 128 / GROUP;
   static constexpr int NB = NPROJ * (EXACT ? 2 : 1);      // B tiles a stage
-  static constexpr int RAW_TILE = BPK + GPB * 64;          // codes + scales/zeros of a (tile, block)
+  // The ring of packed codes holds whole blocks (two stages) of 2-bit codes,
+  // whose two halves interleave, and half blocks (a stage) of 4-bit codes.
+  static constexpr bool HALFRAW = BITS == 4;
+  static constexpr int CPR = HALFRAW ? BPK / 2 : BPK;               // code bytes of a row tile in a ring slot
+  static constexpr int GPR = HALFRAW && GPB > 1 ? GPB / 2 : GPB;    // groups whose scales/zeros it holds
+  static constexpr int RAW_TILE = CPR + GPR * 64;          // codes + scales/zeros of a row tile
   static constexpr int RAWP = 8 * RAW_TILE;                // a projection's: [8 tiles][codes], then [8 tiles][meta]
-  static constexpr int RAW = NPROJ * RAWP;                 // a block's packed weights (two stages)
+  static constexpr int RAW = NPROJ * RAWP;                 // a slot of the ring
   static constexpr int BT = NB * kTileBytes;               // a stage's B tiles
   static constexpr int AT = kHalves * kTileBytes;          // a stage's activation tiles (both token halves)
   // 1 KB for the barriers, 1 KB to align the tiles on 1024 bytes
   static constexpr int AVAIL = (int)kGemmSmemLimit - 2048;
-  // Three rings.  The activation tiles come from L2 with a long latency, so
-  // their ring is the deepest (up to 8 stages); the B tiles are made on chip
-  // and need only 3 (2 where 3 would leave fewer than 4 activation stages);
-  // the packed codes (blocks of two stages) take what is left, at most 6.
-  static constexpr int SB = (AVAIL - 3 * BT - 3 * RAW) / AT >= 4 ? 3 : 2;
-  static constexpr int SA = std::min(8, (AVAIL - SB * BT - 3 * RAW) / AT);
-  static constexpr int R = std::min(6, (AVAIL - SA * AT - SB * BT) / RAW);
+  // Three rings.  B tiles: 3 (2 where 3 would leave fewer than 3 activation
+  // stages) -- with 2 the dequantization of a tile and its hand-over have to
+  // fit into one stage of MMAs; the third, bought with a fourth activation
+  // stage, took gate/up at 3001 tokens of d 2560 from 213 to 194 us.
+  // Activation tiles (from L2): what is left, at most 8; then the packed codes.
+  static constexpr int SB = (AVAIL - 3 * BT - 3 * RAW) / AT >= 3 ? 3 : 2;
+  // (small slots: 8, so that enough of the weights is in flight at few tokens)
+  static constexpr int RMIN = HALFRAW && NB == 1 ? 8 : 3;
+  static constexpr int SA = std::min(8, (AVAIL - SB * BT - RMIN * RAW) / AT);
+  static constexpr int R = std::min(HALFRAW ? 12 : 6, (AVAIL - SA * AT - SB * BT) / RAW);
   static_assert(SA >= 2 && R >= 2, "GEMM pipeline does not fit");
   static constexpr int OFF_A = 0;
   static constexpr int OFF_B = SA * AT;
   static constexpr int OFF_RAW = OFF_B + SB * BT;
   static constexpr int OFF_BAR = OFF_RAW + R * RAW;
-  static constexpr int SMEM = OFF_BAR + (2 * SA + 2 * SB + 2 * R + 2) * 8 + 16 + 1024;  // + alignment slack
+  static constexpr int SMEM = OFF_BAR + (2 * SA + 3 * SB + 3 * R + 2) * 8 + 16 + 1024;  // + alignment slack
   static constexpr int NCH = NPROJ * kBN;                  // TMEM columns of a token half (fp32 accumulators)
   static constexpr int NCOLS = kHalves * NCH;
   static_assert(SMEM <= (int)kGemmSmemLimit, "GEMM stage does not fit");
@@ -138,41 +155,34 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
       : "memory");
 }
 
-// The epilogue of one part of a tile (the 16 dequantizing warps, after the
-// part's accumulators are complete; `have`: no timeout so far).  Warp w reads
-// TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 (the tokens of each half) and
-// columns 32 (w / 4) .. 32 (w / 4) + 31.  A whole tile is finished from TMEM;
-// a part of a split tile is written to its scratch slot, and the CTA that adds
-// the tile's last part to its counter sums the parts in k order (their CTAs
-// are consecutive) and finishes the tile.  Kept out of line so that the
-// dequantization loop keeps its registers.
 // ---------------------------------------------------------------------------
 // Pieces shared by the two kernels below.
 // ---------------------------------------------------------------------------
 
 // Dequantizes the stage hb (features 64 hb .. 64 hb + 63) of a block of
-// packed codes `raw` into the B tiles `Bs`; thread dt of the 16 dequantizing
-// warps takes the items (projection, 16-row tile, lane of the fragment layout)
-// dt, dt + 512, ...
+// packed codes `raw` into the B tiles `Bs`: thread dt of a group of 8 warps
+// takes lane dt % 32 of the fragment layout of 16-row tile dt / 32, for every
+// projection.
 template <int BITS, int NPROJ, int GROUP, bool EXACT>
 __device__ __forceinline__ void gemm_deq_stage(const uint8_t *raw, uint8_t *Bs, int hb, int dt) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
   constexpr int GPB = C::GPB, GS = GROUP / 16;
-  for (int item = dt; item < NPROJ * 8 * 32; item += kDeqWarps * 32) {
-    const int p = item >> 8, j = (item >> 5) & 7, L = item & 31;
+#pragma unroll
+  for (int p = 0; p < NPROJ; ++p) {
+    const int j = dt >> 5, L = dt & 31;
     const int g = L >> 2;
     uint8_t *Bp = Bs + p * kTileBytes;
     // the lane's code words of this half block: 2-bit, words 2 hb, 2 hb + 1
     // of its 16 bytes; 4-bit, the 16 bytes of half hb
     uint32_t wds[BITS == 2 ? 2 : 4];
-    const uint8_t *cb = raw + p * C::RAWP + j * C::BPK;               // codes of tile j
-    const uint8_t *mb = raw + p * C::RAWP + 8 * C::BPK + j * GPB * 64;  // its scales/zeros
+    const uint8_t *cb = raw + p * C::RAWP + j * C::CPR;                       // codes of tile j
+    const uint8_t *mb = raw + p * C::RAWP + 8 * C::CPR + j * C::GPR * 64;  // its scales/zeros
     if (BITS == 2) {
       const uint2 w0 = lds64(cb + L * 16 + hb * 8);
       wds[0] = w0.x;
       wds[1] = w0.y;
     } else {
-      const uint4 w0 = lds128(cb + hb * 512 + L * 16);
+      const uint4 w0 = lds128(cb + L * 16);
       wds[0] = w0.x;
       wds[1] = w0.y;
       wds[2] = w0.z;
@@ -183,7 +193,7 @@ __device__ __forceinline__ void gemm_deq_stage(const uint8_t *raw, uint8_t *Bs, 
     for (int gl = 0; gl < (GS >= 4 ? 1 : 4 / GS); ++gl) {
       const int gi = (4 * hb) / GS + gl;
       // scales and zeros of rows g and g + 8 in group gi (zero for tiles outside the matrix)
-      const uint2 sz = lds64(mb + gi * 64 + g * 8);
+      const uint2 sz = lds64(mb + (C::HALFRAW ? gl : gi) * 64 + g * 8);
       // scales of rows g ("lo" row) and g + 8 ("hi" row); EXACT splits each
       // into a head with the 4 lowest mantissa bits cleared and the tail
       const uint32_t sg = sz.x & 0xffffu, sg8 = sz.x >> 16;
@@ -238,12 +248,28 @@ __device__ __forceinline__ void gemm_deq_stage(const uint8_t *raw, uint8_t *Bs, 
   }
 }
 
+// Ring slot of packed codes and scales/zeros (TMA; one thread): block kb (with
+// HALFRAW its half hb) of the 8 row tiles from n0 / 16 of each projection (TALL:
+// of the next 8 row tiles); row tiles past the matrix read as zeros.
+template <class C, int NPROJ, bool TALL>
+__device__ __forceinline__ void gemm_load_raw(const GemmMaps &tm, uint8_t *dst, int n0, int kb, int hb, uint64_t *full) {
+  mbar_arrive_expect_tx(full, (uint32_t)C::RAW);
+  const int y = kb * (C::BPK / 128) + (C::HALFRAW ? hb * (C::CPR / 128) : 0);
+  const int ym = kb * C::GPB + (C::GPR < C::GPB ? hb * C::GPR : 0);
+#pragma unroll
+  for (int p = 0; p < NPROJ; ++p) {
+    const int z = n0 / 16 + (TALL ? 8 * p : 0);
+    tma_load_3d(dst + p * C::RAWP, &tm.codes[TALL ? 0 : p], 0, y, z, full);
+    tma_load_3d(dst + p * C::RAWP + 8 * C::CPR, &tm.meta[TALL ? 0 : p], 0, ym, z, full);
+  }
+}
+
 // LoRA stage l, B side: rows n0 .. n0 + 127 of B_p (bf16 [N][r]), rank
 // columns 32 l .. 32 l + 31 -> binary16, zeros past r.
 template <int NPROJ>
 __device__ __forceinline__ void gemm_lora_b_stage(const GemmArgs &a, uint8_t *Bs, int n0, int l, int dt) {
   constexpr uint32_t sbo = 4 * 128u;
-  for (int i = dt; i < NPROJ * kBN * 4; i += kDeqWarps * 32) {
+  for (int i = dt; i < NPROJ * kBN * 4; i += kDeqGroup * 32) {
     const int p = i / (kBN * 4), rem = i - p * kBN * 4;
     const int nl = rem >> 2, c = rem & 3;
     const int n = n0 + nl, col = l * kLoraK + c * 8;
@@ -328,101 +354,171 @@ __device__ __forceinline__ void gemm_issue_stage(uint32_t tmem, uint32_t as0, ui
   }
 }
 
-// Output of 8 consecutive rows nb .. nb + 7 of token m from the fp32 sums g
-// (and u for gate/up): h = SiLU(rs g) * (rs u),
-// or y = rs g + residual in bf16 or fp32 (rs: the token's factor that undoes
-// the power-of-two scale of its binary16 activations, times its RMSNorm scale
-// for gate/up).  `vec`: 16-byte stores (N a multiple of 8).
-template <int NPROJ>
-__device__ __forceinline__ void gemm_finish(const GemmArgs &a, int m, int nb, float rs, const float (&g)[8],
-                                            const float (&u)[8], bool vec) {
-  if (m >= a.M || nb >= a.N) return;
-  float v[8];
-  if (NPROJ == 2) {
+// 4 x 4 transpose of 16-byte chunks over groups of 4 lanes: afterwards v[i] is
+// chunk lane % 4 of lane (lane & ~3) + i.
+__device__ __forceinline__ void transpose4(uint4 (&v)[4], int lane) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float gv = rs * g[e], uv = rs * u[e];
-      v[e] = __bfloat162float(__float2bfloat16_rn(__fdividef(gv, 1.f + __expf(-gv)) * uv));  // h as stored
-    }
-  } else {
+  for (int st = 1; st <= 2; st <<= 1) {
+    const bool hi = (lane & st) != 0;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = rs * g[e];
-    if (a.residual) {
-      if (vec) {
-        const uint4 rv =
-            *reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(a.residual) + (size_t)m * a.N + nb);
-        const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] += __uint_as_float(e & 1 ? (rw[e >> 1] & 0xffff0000u) : (rw[e >> 1] << 16));
-      } else {
-        for (int e = 0; e < 8 && nb + e < a.N; ++e)
-          v[e] += __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(a.residual)[(size_t)m * a.N + nb + e]);
-      }
-    }
-  }
-  if (vec) {
-    if (NPROJ == 1 && a.out_f32) {
-      float4 *o = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + (size_t)m * a.N + nb);
-      o[0] = make_float4(v[0], v[1], v[2], v[3]);
-      o[1] = make_float4(v[4], v[5], v[6], v[7]);
-    } else {
-      uint32_t w[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-        w[e] = *reinterpret_cast<const uint32_t *>(&b2);
-      }
-      *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + (size_t)m * a.N + nb) =
-          make_uint4(w[0], w[1], w[2], w[3]);
-    }
-  } else {
-    for (int e = 0; e < 8 && nb + e < a.N; ++e) {
-      const size_t o = (size_t)m * a.N + nb + e;
-      if (NPROJ == 1 && a.out_f32) {
-        reinterpret_cast<float *>(a.out)[o] = v[e];
-      } else {
-        reinterpret_cast<__nv_bfloat16 *>(a.out)[o] = __float2bfloat16_rn(v[e]);
-      }
+    for (int q = 0; q < 2; ++q) {
+      const int lo_i = st == 1 ? 2 * q : q, hi_i = lo_i + st;
+      uint4 give = hi ? v[lo_i] : v[hi_i];
+      give.x = __shfl_xor_sync(0xffffffffu, give.x, st);
+      give.y = __shfl_xor_sync(0xffffffffu, give.y, st);
+      give.z = __shfl_xor_sync(0xffffffffu, give.z, st);
+      give.w = __shfl_xor_sync(0xffffffffu, give.w, st);
+      if (hi) v[lo_i] = give; else v[hi_i] = give;
     }
   }
 }
 
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// h = SiLU(rs g) (rs u) of 16 columns, in place of g.
+__device__ __forceinline__ void gemm_silu16(float *g, const float (&u)[16], float rs) {
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    const float gv = rs * g[e];
+    g[e] = __fdividef(gv, 1.f + __expf(-gv)) * (rs * u[e]);
+  }
+}
+
+// Stores 32 output rows nb .. nb + 31 of the tokens mw + lane (one a lane): v,
+// for down plus the residual.  Four lanes exchange their 16-byte chunks first,
+// so that a store instruction writes 64 contiguous bytes of 8 tokens (whole
+// sectors) instead of 16 bytes of 32; the residual is read the same way.
+template <bool GATEUP>
+__device__ __forceinline__ void gemm_emit32(const GemmArgs &a, int mw, int nb, float (&v)[32], int lane) {
+  if ((a.N & 7) != 0 || (!GATEUP && a.out_f32)) {  // ragged rows, or fp32 output: a token a lane
+    if (mw + lane >= a.M) return;
+    const size_t row = (size_t)(mw + lane) * a.N + nb;
+    const bool f32 = !GATEUP && a.out_f32;
+    if (!GATEUP && a.residual) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e)
+        if (nb + e < a.N) v[e] += __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(a.residual)[row + e]);
+    }
+    if (f32 && (a.N & 7) == 0) {
+#pragma unroll
+      for (int e = 0; e < 32; e += 4)
+        if (nb + e < a.N)
+          *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row + e) =
+              make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+      return;
+    }
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      if (nb + e >= a.N) continue;
+      if (f32)
+        reinterpret_cast<float *>(a.out)[row + e] = v[e];
+      else
+        reinterpret_cast<__nv_bfloat16 *>(a.out)[row + e] = __float2bfloat16_rn(v[e]);
+    }
+    return;
+  }
+  const int col = nb + 8 * (lane & 3), m4 = mw + (lane & ~3);
+  uint4 o[4];
+  if (!GATEUP && a.residual) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      o[i] = m4 + i < a.M && col < a.N
+                 ? *reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(a.residual) +
+                                                    (size_t)(m4 + i) * a.N + col)
+                 : make_uint4(0u, 0u, 0u, 0u);
+    transpose4(o, lane);  // chunk i of this lane's token
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w[4] = {o[i].x, o[i].y, o[i].z, o[i].w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        v[8 * i + e] += __uint_as_float(e & 1 ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    o[i] = make_uint4(pack_bf16(v[8 * i], v[8 * i + 1]), pack_bf16(v[8 * i + 2], v[8 * i + 3]),
+                      pack_bf16(v[8 * i + 4], v[8 * i + 5]), pack_bf16(v[8 * i + 6], v[8 * i + 7]));
+  transpose4(o, lane);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (m4 + i < a.M && col < a.N)
+      *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + (size_t)(m4 + i) * a.N + col) = o[i];
+}
+
+// A warp's share of a finished tile from TMEM: its 32 tokens of half h, 32
+// columns of each accumulator (gate and up; down: one, or with TALL the two
+// 128-row halves of the tile).
+template <int NPROJ, bool TALL>
+__device__ __forceinline__ void gemm_emit_tmem(const GemmArgs &a, uint32_t taddr, int mw, int nb, int lane) {
+  const float rs = a.rs != nullptr && mw + lane < a.M ? a.rs[mw + lane] : 1.f;
+#pragma unroll 1
+  for (int p = 0; p < (TALL ? 2 : 1); ++p) {
+    float g[32];
+    tmem_ld32(taddr + p * kBN, reinterpret_cast<uint32_t(&)[32]>(g));
+    if (NPROJ == 2 && !TALL) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        float u[16];
+        tmem_ld16(taddr + kBN + 16 * q, reinterpret_cast<uint32_t(&)[16]>(u));
+        tmem_ld_wait();
+        gemm_silu16(g + 16 * q, u, rs);
+      }
+    } else {
+      tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < 32; ++e) g[e] *= rs;
+    }
+    gemm_emit32<NPROJ == 2 && !TALL>(a, mw, nb + p * kBN, g, lane);
+  }
+}
+
 // Shared memory of a launch: the barriers behind the rings, then the TMEM
-// base address, the abort flag and the stream-K "last part" flag.
+// base address and the abort flag.
+// raw_full and b_empty have two barriers a slot, for its even and its odd uses:
+// a dequantizing group waits for its own stages only, every other one, so that
+// with one barrier the phase it waits for could have the parity of an earlier
+// one that it never waited for.  With two, the barrier's next phase belongs to
+// a use that cannot begin before this one, and its previous phase has completed
+// before the group's last stage.
 template <class C>
 struct GemmSmem {
   uint8_t *base;
   uint64_t *raw_full, *raw_empty, *a_full, *a_empty, *b_full, *b_empty, *acc_full;
   uint32_t *tmem_s;
-  volatile int *abort_s, *last_s;
+  volatile int *abort_s;
   __device__ explicit GemmSmem(uint8_t *smem_raw) {
     // the swizzled activation tiles need 1024-byte alignment
     base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     raw_full = reinterpret_cast<uint64_t *>(base + C::OFF_BAR);
-    raw_empty = raw_full + C::R;
+    raw_empty = raw_full + 2 * C::R;
     a_full = raw_empty + C::R;
     a_empty = a_full + C::SA;
     b_full = a_empty + C::SA;
     b_empty = b_full + C::SB;
-    acc_full = b_empty + C::SB;
+    acc_full = b_empty + 2 * C::SB;
     tmem_s = reinterpret_cast<uint32_t *>(acc_full + 2);
     abort_s = reinterpret_cast<volatile int *>(tmem_s + 1);
-    last_s = abort_s + 1;
   }
   // thread 0: barrier initialisation; the MMA warp: TMEM allocation
   __device__ void init(int tid, int warp) {
     if (tid == 0) {
       for (int q = 0; q < C::R; ++q) {
-        mbar_init(&raw_full[q], 1);
-        mbar_init(&raw_empty[q], kDeqWarps);
+        mbar_init(&raw_full[2 * q], 1);
+        mbar_init(&raw_full[2 * q + 1], 1);
+        mbar_init(&raw_empty[q], C::HALFRAW ? kDeqGroup : kDeqWarps);
       }
       for (int s = 0; s < C::SA; ++s) {
         mbar_init(&a_full[s], 1);
         mbar_init(&a_empty[s], 1);
       }
       for (int s = 0; s < C::SB; ++s) {
-        mbar_init(&b_full[s], kDeqWarps);
-        mbar_init(&b_empty[s], 1);
+        mbar_init(&b_full[s], kDeqGroup);
+        mbar_init(&b_empty[2 * s], 1);
+        mbar_init(&b_empty[2 * s + 1], 1);
       }
       mbar_init(acc_full, 1);
       *abort_s = 0;
@@ -438,7 +534,7 @@ struct GemmSmem {
 // ---------------------------------------------------------------------------
 // One tile a CTA: grid (token tiles, row tiles).
 // ---------------------------------------------------------------------------
-template <int BITS, int NPROJ, int GROUP, bool EXACT>
+template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmArgs a, const __grid_constant__ GemmMaps tm) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
   constexpr int SA = C::SA, SB = C::SB, R = C::R, GPB = C::GPB;
@@ -446,17 +542,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
   GemmSmem<C> sm(smem_raw);
   uint8_t *smem = sm.base;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * a.mt * kBM, n0 = blockIdx.y * kBN;
+  const int m0 = blockIdx.x * a.mt * kBM, n0 = blockIdx.y * (TALL ? 2 * kBN : kBN);
   const int mth = min(a.mt, (a.M - m0 + kBM - 1) / kBM);  // token halves with tokens in them
   const int KB = (a.K + 127) / 128;
   const int nws = 2 * KB;  // weight stages (64 features each)
-  const int nlora = NPROJ == 2 && a.r > 0 ? (a.r + kLoraK - 1) / kLoraK : 0;
+  const int nlora = NPROJ == 2 && !TALL && a.r > 0 ? (a.r + kLoraK - 1) / kLoraK : 0;
   const int nit = nws + nlora;
   sm.init(tid, warp);
   const uint32_t tmem = *sm.tmem_s;
 
   // bounded wait; a timeout (or an earlier one) makes the caller skip its work
   auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if (mbar_try_wait(bar, parity)) return true;
     if (*sm.abort_s) return false;
     if (mbar_wait_sleep(bar, parity)) return true;
     *sm.abort_s = 1;
@@ -468,15 +565,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
     // ---- packed codes and scales/zeros (TMA) into their ring; row tiles
     // past the matrix read as zeros ----
     if (elect_one())
-      for (int it = 0; it < KB; ++it) {
+      for (int it = 0; it < (C::HALFRAW ? nws : KB); ++it) {
         const int q = it % R;
         if (it >= R && !wait(&sm.raw_empty[q], (it / R - 1) & 1)) break;
-        mbar_arrive_expect_tx(&sm.raw_full[q], (uint32_t)C::RAW);
-        for (int p = 0; p < NPROJ; ++p) {
-          uint8_t *dst = smem + C::OFF_RAW + q * C::RAW + p * C::RAWP;
-          tma_load_3d(dst, &tm.codes[p], 0, it * (C::BPK / 128), n0 / 16, &sm.raw_full[q]);
-          tma_load_3d(dst + 8 * C::BPK, &tm.meta[p], 0, it * GPB, n0 / 16, &sm.raw_full[q]);
-        }
+        gemm_load_raw<C, NPROJ, TALL>(tm, smem + C::OFF_RAW + q * C::RAW, n0, C::HALFRAW ? it >> 1 : it, it & 1,
+                                      &sm.raw_full[2 * q + (it / R & 1)]);
       }
     __syncwarp();
   } else if (warp == kProducerWarp) {
@@ -507,27 +600,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
                                        smem_addr(smem + C::OFF_B + sb * C::BT), mth, it < nws, it == 0);
         // both slots are free once these MMAs have read them
         umma_commit(&sm.a_empty[sa]);
-        umma_commit(&sm.b_empty[sb]);
+        umma_commit(&sm.b_empty[2 * sb + (it / SB & 1)]);
       }
       umma_commit(sm.acc_full);
     }
     __syncwarp();
   } else {
     // ---- dequantization into the B tiles ----
-    for (int it = 0; it < nit; ++it) {
-      const int s = it % SB, kb = it >> 1, hb = it & 1, q = kb % R;
-      if (it < nws && !wait(&sm.raw_full[q], (kb / R) & 1)) break;
-      if (it >= SB && !wait(&sm.b_empty[s], (it / SB - 1) & 1)) break;
+    const int hb = warp / kDeqGroup, dt = tid & (kDeqGroup * 32 - 1);
+    for (int it = hb; it < nit; it += 2) {
+      const int s = it % SB, kr = C::HALFRAW ? it : it >> 1, q = kr % R;
+      const int ur = kr / R, ub = it / SB - 1;  // the slots' uses waited for
+      if (it < nws && !wait(&sm.raw_full[2 * q + (ur & 1)], (ur >> 1) & 1)) break;
+      if (it >= SB && !wait(&sm.b_empty[2 * s + (ub & 1)], (ub >> 1) & 1)) break;
       uint8_t *Bs = smem + C::OFF_B + s * C::BT;
       if (it < nws)
-        gemm_deq_stage<BITS, NPROJ, GROUP, EXACT>(smem + C::OFF_RAW + q * C::RAW, Bs, hb, tid);
+        gemm_deq_stage<BITS, NPROJ, GROUP, EXACT>(smem + C::OFF_RAW + q * C::RAW, Bs, hb, dt);
       else
-        gemm_lora_b_stage<NPROJ>(a, Bs, n0, it - nws, tid);
+        gemm_lora_b_stage<NPROJ>(a, Bs, n0, it - nws, dt);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(&sm.b_full[s]);
-        if (it < nws && hb == 1) mbar_arrive(&sm.raw_empty[q]);  // both halves of this block's codes are read
+        if (it < nws) mbar_arrive(&sm.raw_empty[q]);  // this warp's half of the block's codes is read
       }
     }
 
@@ -536,25 +631,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
     if (wait(sm.acc_full, 0)) {
       tc_fence_after();
       const int quarter = warp & 3, c0 = (warp >> 2) * 32;
-      const bool vec = (a.N & 7) == 0;
-      for (int h = 0; h < mth; ++h) {
-        const int m = m0 + h * kBM + quarter * 32 + lane;
-        const float rs = (a.rs != nullptr && m < a.M) ? a.rs[m] : 1.f;
-        const uint32_t tl = tmem + h * C::NCH + ((uint32_t)(quarter * 32) << 16);
-        for (int c = c0; c < c0 + 32; c += 8) {
-          uint32_t gw[8], uw[8];
-          tmem_ld8(tl + c, gw);
-          if (NPROJ == 2) tmem_ld8(tl + kBN + c, uw);
-          tmem_ld_wait();
-          float g[8], u[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            g[e] = __uint_as_float(gw[e]);
-            u[e] = NPROJ == 2 ? __uint_as_float(uw[e]) : 0.f;
-          }
-          gemm_finish<NPROJ>(a, m, n0 + c, rs, g, u, vec);
-        }
-      }
+      for (int h = 0; h < mth; ++h)
+        gemm_emit_tmem<NPROJ, TALL>(a, tmem + h * C::NCH + ((uint32_t)(quarter * 32) << 16) + c0,
+                                    m0 + h * kBM + quarter * 32, n0 + c0, lane);
     }
   }
 
@@ -576,105 +655,49 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
 // part's accumulators are complete; `have`: no timeout so far).  Warp w reads
 // TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 (the tokens of each half) and
 // columns 32 (w / 4) .. 32 (w / 4) + 31.  A whole tile is finished from TMEM;
-// a part of a split tile is written to its scratch slot, and the CTA that adds
-// the tile's last part to its counter sums the parts in k order (their CTAs
-// are consecutive) and finishes the tile.  Kept out of line so that the
-// dequantization loop keeps its registers.
-template <int BITS, int NPROJ, int GROUP, bool EXACT>
+// a part of a split tile is written to its scratch slot, and gemm_reduce_kernel
+// adds a tile's parts and finishes it: with all SMs, where the CTA of the last
+// part alone took 25 to 35 us for a tile of 256 tokens x 256 rows in 5 parts.
+// Kept out of line so that the dequantization loop keeps its registers.
+template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 __device__ __noinline__ void gemm_part_epilogue(const GemmArgs &a, uint32_t tmem, int tile, int ub, int ue, int U,
-                                                long long W, long long P, long long g0, bool have,
-                                                volatile int *abort_s, volatile int *last_s) {
+                                                long long g0, bool have) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int quarter = warp & 3, c0 = (warp >> 2) * 32;
   const int MT = (a.M + a.mt * kBM - 1) / (a.mt * kBM);
-  const int m0 = (tile % MT) * a.mt * kBM, n0 = (tile / MT) * kBN;
+  const int m0 = (tile % MT) * a.mt * kBM, n0 = (tile / MT) * (TALL ? 2 * kBN : kBN);
   const int mth = min(a.mt, (a.M - m0 + kBM - 1) / kBM);
-  const bool vec = (a.N & 7) == 0;
-  constexpr int SLOT = kHalves * kBM * C::NCH;  // floats of a scratch slot: [half][NCH / 8][128 tokens][8]
+  // a scratch slot: [half][accumulator][column / 4][128 tokens][4] floats, so that
+  // a warp's accesses are contiguous
+  constexpr int SLOT = kHalves * kBM * C::NCH;
+  auto part_at = [&](float *slot, int h, int p) {
+    return reinterpret_cast<float4 *>(slot) + (((size_t)h * NPROJ + p) * (kBN / 4) + c0 / 4) * kBM + quarter * 32 + lane;
+  };
   const bool whole = ub == 0 && ue == U;
   // a split part's scratch slot: the CTA's first part (0) or its last (1)
   float *mine = whole ? nullptr : a.sk_part + ((size_t)blockIdx.x * 2 + ((long long)tile * U + ub == g0 ? 0 : 1)) * SLOT;
   for (int h = 0; h < mth && have; ++h) {
-    const int m = m0 + h * kBM + quarter * 32 + lane;
-    const float rs = (a.rs != nullptr && m < a.M) ? a.rs[m] : 1.f;
-    const uint32_t tl = tmem + h * C::NCH + ((uint32_t)(quarter * 32) << 16);
-    for (int c = c0; c < c0 + 32; c += 8) {
-      uint32_t gw[8], uw[8];
-      tmem_ld8(tl + c, gw);
-      if (NPROJ == 2) tmem_ld8(tl + kBN + c, uw);
-      tmem_ld_wait();
-      float g[8], u[8];
+    const uint32_t tl = tmem + h * C::NCH + ((uint32_t)(quarter * 32) << 16) + c0;
+    if (whole) {
+      gemm_emit_tmem<NPROJ, TALL>(a, tl, m0 + h * kBM + quarter * 32, n0 + c0, lane);
+    } else {
+#pragma unroll 1
+      for (int p = 0; p < NPROJ; ++p) {
+        uint32_t v[32];
+        tmem_ld32(tl + p * kBN, v);
+        tmem_ld_wait();
+        float4 *dst = part_at(mine, h, p);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        g[e] = __uint_as_float(gw[e]);
-        u[e] = NPROJ == 2 ? __uint_as_float(uw[e]) : 0.f;
+        for (int q = 0; q < 8; ++q)
+          __stcg(dst + q * kBM, make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                                            __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])));
       }
-      if (whole) {
-        gemm_finish<NPROJ>(a, m, n0 + c, rs, g, u, vec);
-      } else {
-        // fp32 partial sums, 32 bytes a (token, 8 columns): lanes contiguous
-        float4 *pg = reinterpret_cast<float4 *>(mine + (((size_t)h * (C::NCH / 8) + c / 8) * kBM + quarter * 32 + lane) * 8);
-        __stcg(pg, make_float4(g[0], g[1], g[2], g[3]));
-        __stcg(pg + 1, make_float4(g[4], g[5], g[6], g[7]));
-        if (NPROJ == 2) {
-          float4 *pu = reinterpret_cast<float4 *>(
-              mine + (((size_t)h * (C::NCH / 8) + (kBN + c) / 8) * kBM + quarter * 32 + lane) * 8);
-          __stcg(pu, make_float4(u[0], u[1], u[2], u[3]));
-          __stcg(pu + 1, make_float4(u[4], u[5], u[6], u[7]));
-        }
-      }
-    }
-  }
-  if (whole) return;
-  // the tile's parts lie in CTAs c_lo .. c_hi; the one that brings the
-  // counter to their number sums them and finishes the tile
-  const long long t0u = (long long)tile * U;
-  const int c_lo = (int)(((t0u + 1) * P + W - 1) / W - 1), c_hi = (int)(((t0u + U) * P + W - 1) / W - 1);
-  named_barrier_sync(1, kDeqWarps * 32);
-  if (tid == 0) {
-    int last = 0;
-    if (!*abort_s) {
-      __threadfence();
-      last = atomicAdd(&a.sk_cnt[tile], 1u) == (unsigned)(c_hi - c_lo) ? 1 : 0;
-      if (last) {
-        a.sk_cnt[tile] = 0;  // ready for the next launch
-        __threadfence();
-      }
-    }
-    *last_s = last;
-  }
-  named_barrier_sync(1, kDeqWarps * 32);
-  if (!*last_s) return;
-  for (int h = 0; h < mth; ++h) {
-    const int m = m0 + h * kBM + quarter * 32 + lane;
-    const float rs = (a.rs != nullptr && m < a.M) ? a.rs[m] : 1.f;
-    for (int c = c0; c < c0 + 32; c += 8) {
-      float g[8], u[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) g[e] = u[e] = 0.f;
-      for (int cc = c_lo; cc <= c_hi; ++cc) {
-        // CTA cc's part of this tile is its first (slot 0) unless the tile began inside its range
-        const float *src = a.sk_part + ((size_t)cc * 2 + (t0u <= W * cc / P ? 0 : 1)) * SLOT;
-        const float4 *pg =
-            reinterpret_cast<const float4 *>(src + (((size_t)h * (C::NCH / 8) + c / 8) * kBM + quarter * 32 + lane) * 8);
-        const float4 g0v = __ldcg(pg), g1v = __ldcg(pg + 1);
-        g[0] += g0v.x; g[1] += g0v.y; g[2] += g0v.z; g[3] += g0v.w;
-        g[4] += g1v.x; g[5] += g1v.y; g[6] += g1v.z; g[7] += g1v.w;
-        if (NPROJ == 2) {
-          const float4 *pu = reinterpret_cast<const float4 *>(
-              src + (((size_t)h * (C::NCH / 8) + (kBN + c) / 8) * kBM + quarter * 32 + lane) * 8);
-          const float4 u0v = __ldcg(pu), u1v = __ldcg(pu + 1);
-          u[0] += u0v.x; u[1] += u0v.y; u[2] += u0v.z; u[3] += u0v.w;
-          u[4] += u1v.x; u[5] += u1v.y; u[6] += u1v.z; u[7] += u1v.w;
-        }
-      }
-      gemm_finish<NPROJ>(a, m, n0 + c, rs, g, u, vec);
     }
   }
 }
 
-template <int BITS, int NPROJ, int GROUP, bool EXACT>
+template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_constant__ GemmArgs a,
                                                                    const __grid_constant__ GemmMaps tm) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
@@ -684,15 +707,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
   uint8_t *smem = sm.base;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int KB = (a.K + 127) / 128;
-  const int nlora = NPROJ == 2 && a.r > 0 ? (a.r + kLoraK - 1) / kLoraK : 0;
+  const int nlora = NPROJ == 2 && !TALL && a.r > 0 ? (a.r + kLoraK - 1) / kLoraK : 0;
   const int U = KB + (nlora > 0 ? 1 : 0);
-  const int MT = (a.M + a.mt * kBM - 1) / (a.mt * kBM), NT = (a.N + kBN - 1) / kBN;
+  constexpr int ROWS = TALL ? 2 * kBN : kBN;  // output rows of a tile
+  const int MT = (a.M + a.mt * kBM - 1) / (a.mt * kBM), NT = (a.N + ROWS - 1) / ROWS;
   const long long W = (long long)MT * NT * U, P = gridDim.x;
   const long long g0 = W * blockIdx.x / P, g1 = W * (blockIdx.x + 1) / P;
   sm.init(tid, warp);
   const uint32_t tmem = *sm.tmem_s;
 
   auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if (mbar_try_wait(bar, parity)) return true;
     if (*sm.abort_s) return false;
     if (mbar_wait_sleep(bar, parity)) return true;
     *sm.abort_s = 1;
@@ -713,23 +738,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
 
   if (warp == kRawWarp) {
     if (elect_one()) {
-      int gr = 0;  // blocks loaded so far
+      int gr = 0;  // ring slots loaded so far
       bool ok = true;
       WQ_FOR_EACH_PART {
         (void)nit;  // the codes ring follows the blocks only
-        const int n0 = (tile / MT) * kBN;
-        for (int kb = ub; kb < ub + wb && ok; ++kb, ++gr) {
+        const int n0 = (tile / MT) * ROWS;
+        for (int r = 0; r < (C::HALFRAW ? 2 * wb : wb) && ok; ++r, ++gr) {
           const int q = gr % R;
           if (gr >= R && !wait(&sm.raw_empty[q], (gr / R - 1) & 1)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&sm.raw_full[q], (uint32_t)C::RAW);
-          for (int p = 0; p < NPROJ; ++p) {
-            uint8_t *dst = smem + C::OFF_RAW + q * C::RAW + p * C::RAWP;
-            tma_load_3d(dst, &tm.codes[p], 0, kb * (C::BPK / 128), n0 / 16, &sm.raw_full[q]);
-            tma_load_3d(dst + 8 * C::BPK, &tm.meta[p], 0, kb * GPB, n0 / 16, &sm.raw_full[q]);
-          }
+          gemm_load_raw<C, NPROJ, TALL>(tm, smem + C::OFF_RAW + q * C::RAW, n0, ub + (C::HALFRAW ? r >> 1 : r), r & 1,
+                                        &sm.raw_full[2 * q + (gr / R & 1)]);
         }
       }
     }
@@ -775,7 +796,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
           gemm_issue_stage<NPROJ, EXACT>(tmem, smem_addr(smem + C::OFF_A + sa * C::AT),
                                          smem_addr(smem + C::OFF_B + sb * C::BT), mth, it < 2 * wb, it == 0);
           umma_commit(&sm.a_empty[sa]);
-          umma_commit(&sm.b_empty[sb]);
+          umma_commit(&sm.b_empty[2 * sb + (gs / SB & 1)]);
         }
         if (ok) umma_commit(sm.acc_full);  // the part's accumulators are complete
       }
@@ -784,33 +805,36 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
   } else {
     // dequantization, then each part's epilogue; a warp that met a timeout
     // skips its work but still passes the epilogue's named barriers
+    const int hb = warp / kDeqGroup, dt = tid & (kDeqGroup * 32 - 1);
     int gs = 0, gr = 0, part = 0;
     bool ok = true;
     WQ_FOR_EACH_PART {
-      const int n0 = (tile / MT) * kBN;
-      for (int it = 0; it < nit; ++it, ++gs) {
-        const int s = gs % SB, hb = it & 1, kr = gr + (it >> 1), q = kr % R;
+      const int n0 = (tile / MT) * ROWS;
+      for (int it = hb; it < nit; it += 2) {
+        const int st = gs + it, s = st % SB, kr = gr + (C::HALFRAW ? it : it >> 1), q = kr % R;
         const bool wstage = it < 2 * wb;
-        if (ok && wstage && !wait(&sm.raw_full[q], (kr / R) & 1)) ok = false;
-        if (ok && gs >= SB && !wait(&sm.b_empty[s], (gs / SB - 1) & 1)) ok = false;
+        const int ur = kr / R, vb = st / SB - 1;  // the slots' uses waited for
+        if (ok && wstage && !wait(&sm.raw_full[2 * q + (ur & 1)], (ur >> 1) & 1)) ok = false;
+        if (ok && st >= SB && !wait(&sm.b_empty[2 * s + (vb & 1)], (vb >> 1) & 1)) ok = false;
         if (!ok) continue;
         uint8_t *Bs = smem + C::OFF_B + s * C::BT;
         if (wstage)
-          gemm_deq_stage<BITS, NPROJ, GROUP, EXACT>(smem + C::OFF_RAW + q * C::RAW, Bs, hb, tid);
+          gemm_deq_stage<BITS, NPROJ, GROUP, EXACT>(smem + C::OFF_RAW + q * C::RAW, Bs, hb, dt);
         else
-          gemm_lora_b_stage<NPROJ>(a, Bs, n0, it - 2 * wb, tid);
+          gemm_lora_b_stage<NPROJ>(a, Bs, n0, it - 2 * wb, dt);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(&sm.b_full[s]);
-          if (wstage && hb == 1) mbar_arrive(&sm.raw_empty[q]);  // both halves of this block's codes are read
+          if (wstage) mbar_arrive(&sm.raw_empty[q]);  // this warp's half of the block's codes is read
         }
       }
-      gr += wb;
+      gs += nit;
+      gr += C::HALFRAW ? 2 * wb : wb;
       const bool have = ok && wait(sm.acc_full, part & 1);
       ++part;
       tc_fence_after();
-      gemm_part_epilogue<BITS, NPROJ, GROUP, EXACT>(a, tmem, tile, ub, ue, U, W, P, g0, have, sm.abort_s, sm.last_s);
+      gemm_part_epilogue<BITS, NPROJ, GROUP, EXACT, TALL>(a, tmem, tile, ub, ue, U, g0, have);
       // the next part's MMAs overwrite the accumulators only after this warp's
       // b_full arrival, which follows its TMEM reads
       tc_fence_before();
@@ -824,20 +848,104 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
   if (warp == kMmaWarp) tmem_dealloc(tmem, C::NCOLS);
 }
 
+// The split tiles of a stream-K launch of P CTAs: the parts' fp32 sums added in
+// k order (their CTAs c_lo .. c_hi are consecutive), then the epilogue.  A
+// thread takes one token and 16 columns of an accumulator (of gate and up):
+// grid (columns / 16, halves, tiles), 128 threads a half.
+template <int NPROJ, bool TALL>
+__global__ void __launch_bounds__(kBM) gemm_reduce_kernel(const GemmArgs a, int U, long long W, long long P) {
+  pdl_wait();
+  const int tile = blockIdx.z, h = blockIdx.y, cg = blockIdx.x % (kBN / 16), p = blockIdx.x / (kBN / 16);
+  const long long t0u = (long long)tile * U;
+  const int c_lo = (int)(((t0u + 1) * P + W - 1) / W - 1), c_hi = (int)(((t0u + U) * P + W - 1) / W - 1);
+  if (c_lo == c_hi) return;  // finished from TMEM
+  const int MT = (a.M + a.mt * kBM - 1) / (a.mt * kBM);
+  const int m = (tile % MT) * a.mt * kBM + h * kBM + threadIdx.x;
+  const int nb = (tile / MT) * (TALL ? 2 * kBN : kBN) + p * kBN + cg * 16;
+  if (m >= a.M || nb >= a.N) return;
+  constexpr int SLOT = kHalves * kBM * NPROJ * kBN;
+  auto sum = [&](int acc, float (&v)[16]) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = 0.f;
+#pragma unroll 4
+    for (int cc = c_lo; cc <= c_hi; ++cc) {
+      // CTA cc's part of this tile is its first (slot 0) unless the tile began inside its range
+      const float4 *src = reinterpret_cast<const float4 *>(a.sk_part + ((size_t)cc * 2 + (t0u <= W * cc / P ? 0 : 1)) * SLOT) +
+                          (((size_t)h * NPROJ + acc) * (kBN / 4) + cg * 4) * kBM + threadIdx.x;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 f = __ldcg(src + i * kBM);
+        v[4 * i] += f.x;
+        v[4 * i + 1] += f.y;
+        v[4 * i + 2] += f.z;
+        v[4 * i + 3] += f.w;
+      }
+    }
+  };
+  const float rs = a.rs != nullptr ? a.rs[m] : 1.f;
+  float v[16];
+  const size_t o = (size_t)m * a.N + nb;
+  sum(p, v);
+  if (NPROJ == 2 && !TALL) {
+    float u[16];
+    sum(1, u);
+    gemm_silu16(v, u, rs);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] *= rs;
+    const __nv_bfloat16 *res = reinterpret_cast<const __nv_bfloat16 *>(a.residual);
+    if (res && (a.N & 7) == 0) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (nb + 8 * i >= a.N) continue;
+        const uint4 q = *reinterpret_cast<const uint4 *>(res + o + 8 * i);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          v[8 * i + e] += __uint_as_float(e & 1 ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16));
+      }
+    } else if (res) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        if (nb + e < a.N) v[e] += __bfloat162float(res[o + e]);
+    }
+  }
+  const bool f32 = NPROJ == 1 && !TALL && a.out_f32;
+  if (!f32 && (a.N & 7) == 0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (nb + 8 * i < a.N)
+        *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(a.out) + o + 8 * i) =
+            make_uint4(pack_bf16(v[8 * i], v[8 * i + 1]), pack_bf16(v[8 * i + 2], v[8 * i + 3]),
+                       pack_bf16(v[8 * i + 4], v[8 * i + 5]), pack_bf16(v[8 * i + 6], v[8 * i + 7]));
+    return;
+  }
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    if (nb + e >= a.N) continue;
+    if (f32)
+      reinterpret_cast<float *>(a.out)[o + e] = v[e];
+    else
+      reinterpret_cast<__nv_bfloat16 *>(a.out)[o + e] = __float2bfloat16_rn(v[e]);
+  }
+}
+
 // Per token of x [M, K] (bf16, K a multiple of 32): the binary16 copy x16
 // [M][lda16] (the GEMM's A operand, zeros past K), the RMSNorm scale
 // rs = 1/sqrt(mean(x^2) + eps) and, with an adapter, ta = lora_scale * x A^T
 // as binary16 [M][2r] (gate rows, then up rows).
 // A CTA takes 16 tokens and 16 rows of A.  The products x A^T run on m16n8k16
 // bf16 MMAs (exact products, fp32 sums); the 16 warps take interleaved chunks
-// of 32 features, two chunks' loads in flight at a time, and their partial
-// sums are added in warp order.  A lane loads 8 consecutive features of a row
+// of 32 features, kPrepUnroll chunks' loads in flight at a time (2, or 5 where
+// the grid leaves each SM one CTA: 512 tokens of d 5120 15.8 -> 13.2 us), and
+// their partial sums are added in warp order.  A lane loads 8 consecutive features of a row
 // (16 bytes) and feeds features 0..3 and 4..7 of them to two k-steps in the
 // slots of k 2t, 2t+1, 2t+8, 2t+9: the same permutation of k for x and A, so
 // the sums are unchanged.  Every CTA sums x^2 of its tokens (row block 0
 // writes rs) and converts the chunks c with c % gridDim.y == blockIdx.y.
-constexpr int kPrepTok = 16, kPrepRows = 16, kPrepWarps = 16, kPrepUnroll = 2;
+constexpr int kPrepTok = 16, kPrepRows = 16, kPrepWarps = 16;
 
+template <int kPrepUnroll>
 __global__ void __launch_bounds__(kPrepWarps * 32) gemm_prep_kernel(const __nv_bfloat16 *x, int M, int K, int lda16,
                                                                    const __nv_bfloat16 *lora_a, int r2,
                                                                    float lora_scale, int prenorm, uint16_t *x16,
@@ -1080,7 +1188,7 @@ cudaError_t make_maps(const GemmArgs &a, int nproj, int bits, GemmMaps *m) {
     {
       const cuuint64_t dims[3] = {128, KB * bpk / 128, RT};
       const cuuint64_t strides[2] = {128, KB * bpk};
-      const cuuint32_t box[3] = {128, (cuuint32_t)(bpk / 128), 8};
+      const cuuint32_t box[3] = {128, 4, 8};  // a 2-bit block or half a 4-bit block
       if (fn(&m->codes[p], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint32_t *>(a.codes[src]), dims, strides, box, e1,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1089,7 +1197,7 @@ cudaError_t make_maps(const GemmArgs &a, int nproj, int bits, GemmMaps *m) {
     {
       const cuuint64_t dims[3] = {64, KB * gpb, RT};
       const cuuint64_t strides[2] = {64, KB * gpb * 64};
-      const cuuint32_t box[3] = {64, (cuuint32_t)gpb, 8};
+      const cuuint32_t box[3] = {64, (cuuint32_t)(bits == 4 && gpb > 1 ? gpb / 2 : gpb), 8};
       if (fn(&m->meta[p], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint16_t *>(a.meta[src]), dims, strides, box, e1,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1113,61 +1221,85 @@ cudaError_t num_sms_cached(int *sms) {
 
 // Work split of a launch.  A CTA takes two token halves (each weight
 // dequantized once for 256 tokens) whenever there are more than 128 tokens.
-// Tiles are mt * 128 tokens x 128 rows, U work units each (128-feature
-// blocks, plus one for the LoRA stages).  Stream-K -- P CTAs (one per SM at
-// most, 4 units each at least) dividing the T * U units evenly -- when it
-// shortens the critical path by more than its own cost, which was measured at
-// about 40 units (the split tiles' partial sums and fixups, and a slower main
-// loop); one CTA per tile otherwise.
-constexpr long long kStreamKCost = 40;  // work units
-
+// Tiles are mt * 128 tokens x 128 rows (down may take 256, below), U work units
+// each (128-feature blocks, plus one for the LoRA stages).  Stream-K -- P CTAs
+// (one per SM at most, 4 units each at least) dividing the T * U units evenly --
+// where it shortens the critical path by more than its cost in units: the split
+// tiles' parts and their reduction (~8; measured d 2560 down at 2048 tokens 137
+// -> 103 us, d 5120 at 1500 228 -> 216), and for gate/up, whose parts are twice
+// as large, a main loop about a tenth slower (d 4096 at 700 tokens 159 -> 152
+// with it, at 512 tokens 110 -> 116, d 5120 at 3001 658 -> 695; d 2560 at 65
+// tokens, half the SMs without it, 39 -> 34).  One CTA per tile otherwise.
 struct GemmSched {
   int mt, T, U, P;
   bool sk;
 };
-GemmSched gemm_schedule(int M, int N, int K, int nproj, int r, int sms) {
+GemmSched gemm_schedule(int M, int N, int K, int nproj, int r, int sms, int rows = kBN) {
   GemmSched g;
   g.mt = M > kBM ? 2 : 1;
-  g.T = (M + g.mt * kBM - 1) / (g.mt * kBM) * ((N + kBN - 1) / kBN);
+  g.T = (M + g.mt * kBM - 1) / (g.mt * kBM) * ((N + rows - 1) / rows);
   g.U = (K + 127) / 128 + (nproj == 2 && r > 0 ? 1 : 0);
   const long long W = (long long)g.T * g.U;
   const long long waves = (g.T + sms - 1) / sms, P = std::max(1LL, std::min((long long)sms, W / 4));
-  g.sk = W >= 8 && waves * g.U > (W + P - 1) / P + kStreamKCost;
+  const double share = (double)W / P;  // units a CTA
+  g.sk = W >= 8 && waves * g.U > (nproj == 2 ? 1.25 * share + 6 : share + 8);
   g.P = g.sk ? (int)P : g.T;
   return g;
 }
 
-template <int BITS, int NPROJ, int GROUP, bool EXACT>
+// Down launches of more than 128 tokens take tiles of 256 rows (TALL: one
+// N = 256 MMA over two 128-row tiles reads 96 bytes a clock of the 128 that
+// shared memory gives, an N = 128 one all 128) where they make at least
+// kTallTiles of them, so that few CTAs share a split tile (us, 128-row vs
+// 256-row: d 2560 at 3001 tokens 200 -> 144, d 5120 at 512 tokens 141 -> 87;
+// but d 2560 at 256 tokens, 10 tiles, 37 vs 44, and at 512, 20 tiles, 46 vs 48).
+constexpr int kTallTiles = 30;
+bool gemm_tall(int M, int N) {
+  return M > kBM && (long long)((M + 2 * kBM - 1) / (2 * kBM)) * ((N + 2 * kBN - 1) / (2 * kBN)) >= kTallTiles;
+}
+
+template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 cudaError_t launch_gemm_t(const GemmArgs &a, cudaStream_t s) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
-  auto tile_kern = qgemm_tile_kernel<BITS, NPROJ, GROUP, EXACT>;
-  auto sk_kern = qgemm_sk_kernel<BITS, NPROJ, GROUP, EXACT>;
+  constexpr int ROWS = TALL ? 2 * kBN : kBN;
+  auto tile_kern = qgemm_tile_kernel<BITS, NPROJ, GROUP, EXACT, TALL>;
+  auto sk_kern = qgemm_sk_kernel<BITS, NPROJ, GROUP, EXACT, TALL>;
   cudaError_t e = cudaFuncSetAttribute(tile_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   GemmMaps maps;
-  if ((e = make_maps(a, NPROJ, BITS, &maps)) != cudaSuccess) return e;
+  if ((e = make_maps(a, TALL ? 1 : NPROJ, BITS, &maps)) != cudaSuccess) return e;
   int sms = 0;
   if ((e = num_sms_cached(&sms)) != cudaSuccess) return e;
-  const GemmSched g = gemm_schedule(a.M, a.N, a.K, NPROJ, a.r, sms);
+  const GemmSched g = gemm_schedule(a.M, a.N, a.K, TALL ? 1 : NPROJ, a.r, sms, ROWS);
   GemmArgs ka = a;
   ka.mt = g.mt;
-  if (g.sk && a.sk_part && a.sk_cnt) {
+  if (g.sk && a.sk_part) {
     sk_kern<<<g.P, kGemmThreads, C::SMEM, s>>>(ka, maps);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((TALL ? 2 : 1) * kBN / 16, g.mt, g.T);
+    cfg.blockDim = dim3(kBM);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gemm_reduce_kernel<NPROJ, TALL>, ka, g.U, (long long)g.T * g.U, (long long)g.P);
   } else {
     ka.sk_part = nullptr;
-    ka.sk_cnt = nullptr;
-    tile_kern<<<dim3((a.M + g.mt * kBM - 1) / (g.mt * kBM), (a.N + kBN - 1) / kBN), kGemmThreads, C::SMEM, s>>>(ka, maps);
+    tile_kern<<<dim3((a.M + g.mt * kBM - 1) / (g.mt * kBM), (a.N + ROWS - 1) / ROWS), kGemmThreads, C::SMEM, s>>>(ka, maps);
   }
   return cudaGetLastError();
 }
 
-template <int BITS, int NPROJ, bool EXACT>
+template <int BITS, int NPROJ, bool EXACT, bool TALL = false>
 cudaError_t launch_gemm_g(const GemmArgs &a, cudaStream_t s) {
   switch (a.group) {
-    case 32: return launch_gemm_t<BITS, NPROJ, 32, EXACT>(a, s);
-    case 64: return launch_gemm_t<BITS, NPROJ, 64, EXACT>(a, s);
-    default: return launch_gemm_t<BITS, NPROJ, 128, EXACT>(a, s);
+    case 32: return launch_gemm_t<BITS, NPROJ, 32, EXACT, TALL>(a, s);
+    case 64: return launch_gemm_t<BITS, NPROJ, 64, EXACT, TALL>(a, s);
+    default: return launch_gemm_t<BITS, NPROJ, 128, EXACT, TALL>(a, s);
   }
 }
 
@@ -1178,26 +1310,35 @@ cudaError_t launch_gemm(GemvKind kind, const GemmArgs &a, cudaStream_t s) {
   switch (kind) {
     case kGateUpW2: return launch_gemm_g<2, 2, false>(a, s);
     case kGateUpW4: return launch_gemm_g<4, 2, false>(a, s);
-    default: return a.out_f32 ? launch_gemm_g<4, 1, true>(a, s) : launch_gemm_g<4, 1, false>(a, s);
+    default:
+      if (a.out_f32) return launch_gemm_g<4, 1, true>(a, s);
+      return gemm_tall(a.M, a.N) ? launch_gemm_g<4, 2, false, true>(a, s) : launch_gemm_g<4, 1, false>(a, s);
   }
 }
 
 size_t gemm_scratch_floats(int M, int N, int K, int nproj, int num_sms) {
   if (M <= 0 || N <= 0 || K <= 0 || num_sms <= 0) return 0;
   const GemmSched g = gemm_schedule(M, N, K, nproj, kMaxRank, num_sms);
-  return g.sk ? (size_t)2 * g.P * kHalves * kBM * nproj * kBN : 0;
+  size_t most = g.sk ? (size_t)2 * g.P * kHalves * kBM * nproj * kBN : 0;
+  if (nproj == 1 && gemm_tall(M, N)) {
+    const GemmSched t = gemm_schedule(M, N, K, 1, 0, num_sms, 2 * kBN);
+    if (t.sk) most = std::max(most, (size_t)2 * t.P * kHalves * kBM * 2 * kBN);
+  }
+  return most;
 }
-
-size_t gemm_counters(int M, int N) { return (size_t)((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN); }
 
 cudaError_t launch_gemm_prep(const void *x, int M, int K, int lda16, const void *lora_a, int r2, float lora_scale,
                              int prenorm, uint16_t *x16, float *rs, uint16_t *ta, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
   if (K % 32 != 0 || lda16 < K) return cudaErrorInvalidValue;
   const dim3 grid((M + kPrepTok - 1) / kPrepTok, r2 > 0 ? (r2 + kPrepRows - 1) / kPrepRows : 1);
-  gemm_prep_kernel<<<grid, kPrepWarps * 32, 0, s>>>(
-      reinterpret_cast<const __nv_bfloat16 *>(x), M, K, lda16, reinterpret_cast<const __nv_bfloat16 *>(lora_a), r2,
-      lora_scale, prenorm, x16, rs, ta);
+  int sms = 0;
+  cudaError_t e = num_sms_cached(&sms);
+  if (e != cudaSuccess) return e;
+  auto kern = (long long)grid.x * grid.y <= sms ? gemm_prep_kernel<5> : gemm_prep_kernel<2>;
+  kern<<<grid, kPrepWarps * 32, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(x), M, K, lda16,
+                                        reinterpret_cast<const __nv_bfloat16 *>(lora_a), r2, lora_scale, prenorm, x16, rs,
+                                        ta);
   return cudaGetLastError();
 }
 cudaError_t launch_to_f16(const void *x, int M, int K, int lda16, uint16_t *x16, float *sx, cudaStream_t s) {

@@ -113,10 +113,7 @@ struct GemmArgs {
   void *out;                 // bf16 (or fp32 for down with out_f32) [M][N]
   int out_f32;
   int mt;                    // token halves of 128 per CTA (1 or 2; set by launch_gemm)
-  // stream-K scratch (null: one CTA per tile): gemm_scratch_floats() fp32 and
-  // gemm_counters() arrival counters, zero between launches
-  float *sk_part;
-  unsigned *sk_cnt;
+  float *sk_part;            // stream-K scratch, gemm_scratch_floats() fp32 (null: one CTA per tile)
 };
 cudaError_t launch_gemm(GemvKind kind, const GemmArgs &args, cudaStream_t stream);
 // Per token m of x [M, K]: an exact power of two 2^e puts max|x[m]| in
@@ -129,9 +126,8 @@ cudaError_t launch_gemm_prep(const void *x, int M, int K, int lda16, const void 
 // max|x| in [2^4, 2^5); sx[m] = 2^-e (the down GEMM's epilogue factor).
 cudaError_t launch_to_f16(const void *x, int M, int K, int lda16, uint16_t *x16, float *sx, cudaStream_t stream);
 // Stream-K scratch a GEMM launch of this shape can need: fp32 partial sums
-// and per-tile arrival counters (num_sms: the device's SM count).
+// (num_sms: the device's SM count).
 size_t gemm_scratch_floats(int M, int N, int K, int nproj, int num_sms);
-size_t gemm_counters(int M, int N);
 int gemm_stages(GemvKind kind, int group);  // depth of the activation-tile ring
 // Reads and clears the GEMM kernels' device status word.
 cudaError_t read_gemm_status(int *status);

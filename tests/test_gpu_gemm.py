@@ -227,3 +227,25 @@ def test_gemm_stream_k_split_tiles(wq, m):
     ref, _ = orc.down(synth.bf16_bits(hd), qd, group, synth.bf16_bits(res))
     check_bf16(y, ref, f"GEMM y (stream-K) m={m}", min_exact=MIN_EXACT)
     check_f32(y32, ref, f"GEMM y(f32) (stream-K) m={m}")
+
+
+@pytest.mark.parametrize("d,inter,group,m", [
+    (7680, 256, 128, 129),    # 30 tiles of 256 rows, one part each; 2 stages
+    (7570, 1024, 32, 257),    # ragged last tile (rows no multiple of 8: scalar stores), 3 token halves
+    (3840, 8192, 64, 300),    # 30 tiles, split over the SMs
+])
+def test_gemm_down_tall_tiles(wq, d, inter, group, m):
+    """256-row down tiles (at least 30 of them above 128 tokens), whole and split."""
+    rng = np.random.default_rng(d + m)
+    qd = orc.quantize((rng.standard_normal((d, inter)) * 0.02).astype(np.float32), group, 4)[:3]
+    dn = upload_packed(*qd, group, 4)
+    h = (synth.activations((m, inter), 20 + m) * 0.5).to(torch.bfloat16)
+    res = synth.activations((m, d), 30 + m)
+    y = wq.down_w4(h.cuda(), dn, residual=res.cuda())
+    y0 = wq.down_w4(h.cuda(), dn)
+    torch.cuda.synchronize()
+    assert wq.device_status() == 0
+    rows = np.unique(np.concatenate([np.arange(0, m, 37), [127, 128, m - 1]]))
+    for got, r, what in ((y, res, "residual"), (y0, None, "plain")):
+        ref, _ = orc.down(synth.bf16_bits(h)[rows], qd, group, None if r is None else synth.bf16_bits(r)[rows])
+        check_bf16(got[torch.from_numpy(rows).cuda()], ref, f"tall {what} d={d} I={inter} m={m}", min_exact=MIN_EXACT)
