@@ -13,16 +13,31 @@
 //      and sine taken in fp32 on the reduced argument);
 //   3. k and v rounded to bf16 and appended to the cache at lens[b];
 //   4. o = softmax(q K^T / sqrt(hd)) V over positions 0..lens[b].
-// The context is cut into S splits (grid.y); a CTA of 8 warps takes one
-// (b, g) and one split; each warp takes chunks of 8 positions, the lanes the
-// head dimension.  A warp copies its next chunk's K and V rows into a shared-
-// memory buffer of its own (cp.async, 16 bytes a lane and copy) while it
-// computes the current chunk from the other buffer, so two chunks' rows are
-// in flight at a time.  The 32
-// partial dot products of a chunk (8 positions x 4 query heads) are reduced
-// by a butterfly reduce-scatter (31 shuffles), the softmax runs online (max,
-// sum, rescaled accumulators) in fp32.  The splits' partial results (max,
-// sum, accumulator) are merged in a fixed order by a second kernel.
+// The context is cut into S splits (grid.y); a CTA of 4 warps takes one (b, g)
+// and one split, each warp chunks of 16 positions.  A warp copies its next
+// chunk's K and V rows into a shared-memory buffer of its own (cp.async,
+// 16-byte chunks XOR-swizzled by the row) while it computes the current one.
+//
+// Scores and outputs are mma.sync products of the bf16 rows, with the fp32
+// operand in three bf16 parts (8 significand bits each, 24 in all), so that
+// every product is exact and the sums are fp32 as before: the 4 query heads'
+// parts are the columns of Q (head h: columns 2h, 2h + 1 of the first 8-column
+// tile and 2h of the second), the probabilities' parts the rows of P (row h +
+// 4 part), added up at the end.  A chunk takes 16 + 16 MMAs where the lanes'
+// dot products, their 31-shuffle reduction and the probabilities' 32 broadcasts
+// took ~1000 instructions.  The softmax runs online (max, sum, rescaled
+// accumulators) in fp32.  Parts of an infinite operand would cancel into NaN;
+// a warp whose result holds a NaN therefore computes its range again with
+// plain fp32 products (attn_plain).  The splits' partial results (max, sum,
+// accumulator) are merged in a fixed order by a second kernel.
+//
+// Bound by the latency of the chunks' loads and of the steps before them (the
+// layer input's norm, RoPE, the head norms); two chunks of 8 KB a warp and 12
+// warps an SM keep ~190 KB in flight.  Measured (GB300, cold, us, lanes' dot
+// products with 8 warps a CTA and two CTAs an SM before -> this): 16 sequences of 512
+// to 2048 positions, 32 / 8 heads of 128: 39.1 -> 24.4 for 84 MB of cache rows;
+// one of 8192: 17.5 -> 14.7 for 34 MB.  Share of bf16 outputs off the exact
+// rounding 0.00026 -> 0.00024 at 8192 positions, 0.00026 -> 0.00019 at 2048.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -42,24 +57,24 @@ __device__ int g_attn_status = 0;
 
 namespace {
 
-constexpr int kAttnWarps = 8;
-constexpr int kHG = 4;   // query heads a pass takes (padded with zero heads)
-constexpr int kPos = 8;  // positions a chunk takes (kHG * kPos = 32 lanes)
+constexpr int kAttnWarps = 4;
+constexpr int kAttnOcc = 3;   // CTAs an SM holds (64 KB of K and V buffers each)
+constexpr int kCombWarps = 8;
+constexpr int kHG = 4;        // query heads a pass takes (padded with zero heads)
+constexpr int kPos = 16;      // positions a chunk takes
 
 __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
-// HD/32 consecutive bf16 values of a row in shared memory (8 bytes for HD
-// 128, 4 for HD 64)
-template <int HD>
-__device__ __forceinline__ void load_row_s(const __nv_bfloat16 *p, float (&v)[HD / 32]) {
-  if (HD == 128) {
-    const uint2 w = *reinterpret_cast<const uint2 *>(p);
-    v[0] = bf_lo(w.x); v[1] = bf_hi(w.x); v[2] = bf_lo(w.y); v[3] = bf_hi(w.y);
-  } else {
-    const uint32_t w = *reinterpret_cast<const uint32_t *>(p);
-    v[0] = bf_lo(w); v[1] = bf_hi(w);
-  }
+// x = hi + mid + lo with bf16 parts (exact to 24 bits).
+__device__ __forceinline__ void split3(float x, float (&p)[3]) {
+  p[0] = __bfloat162float(__float2bfloat16_rn(x));
+  p[1] = __bfloat162float(__float2bfloat16_rn(x - p[0]));
+  p[2] = x - p[0] - p[1];
+}
+__device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t *>(&v);
 }
 
 }  // namespace
@@ -69,24 +84,59 @@ struct RopeFreq {
   double f[64];
 };
 
-// grid (B * n_kv, S), block kAttnWarps * 32.  part: [B][H][S][HD + 2] fp32
-// (accumulator, max, sum) of every split.
 // Copies of one chunk (positions cb .. cb + kPos - 1) of K and V rows into a
-// warp's buffer dst ([K, V][kPos][HD], already offset by the lane's column):
-// copy i of a lane takes row i * (32 / CPR) + lrow; positions outside
-// [p0, p1) and the new position pos are zero-filled.
+// warp's buffer ([K, V][kPos][HD], 16-byte chunk c of row r at c ^ (r % 8)):
+// positions outside [p0, p1) and the new position pos are zero-filled.
 template <int HD>
-__device__ __forceinline__ void attn_issue(__nv_bfloat16 *dst, const __nv_bfloat16 *kbase,
-                                           const __nv_bfloat16 *vbase, int lrow, int cb, int p0, int p1, int pos) {
-  constexpr int CPR = HD * 2 / 16;
+__device__ __forceinline__ void attn_issue(__nv_bfloat16 *buf, const __nv_bfloat16 *kbase, const __nv_bfloat16 *vbase,
+                                           int lane, int cb, int p0, int p1, int pos) {
+  constexpr int CPR = HD * 2 / 16;  // 16-byte copies a row
+  const int c = lane % CPR;
 #pragma unroll
   for (int i = 0; i < 2 * kPos * CPR / 32; ++i) {
-    const int r = i * (32 / CPR) + lrow;
+    const int r = i * (32 / CPR) + lane / CPR;
     const int p = cb + r % kPos;
     const bool in = p < p1 && p != pos;
-    const __nv_bfloat16 *src = (r < kPos ? kbase : vbase) + (size_t)(in ? p : p0) * HD;
-    cp_async16_zfill(dst + (size_t)r * HD, src, in ? 16u : 0u);
+    const __nv_bfloat16 *src = (r < kPos ? kbase : vbase) + (size_t)(in ? p : p0) * HD + c * 8;
+    cp_async16_zfill(buf + (size_t)r * HD + (c ^ (r & 7)) * 8, src, in ? 16u : 0u);
   }
+}
+
+// One warp's share of a split with plain fp32 products (a lane: HD / 32
+// dimensions): the same chunks, any values.  Leaves max, sum and accumulator in
+// shared memory as the fast loop does.
+template <int HD>
+__device__ __noinline__ void attn_plain(const float (*qs)[HD], const float (*kvn)[HD], const __nv_bfloat16 *kbase,
+                                        const __nv_bfloat16 *vbase, int h0, int rep, int first, int stride, int p1,
+                                        int pos, float *ws_m, float *ws_l, float (*ws_o)[HD]) {
+  constexpr int E = HD / 32;
+  const int lane = threadIdx.x & 31;
+  for (int hq = 0; hq < kHG; ++hq) {
+    float m = -INFINITY, l = 0.f, o[E];
+    for (int e = 0; e < E; ++e) o[e] = 0.f;
+    for (int cb = first; cb < p1; cb += stride)
+      for (int p = cb; p < min(p1, cb + kPos); ++p) {
+        float s = 0.f, v[E];
+        for (int e = 0; e < E; ++e) {
+          const int i = lane * E + e;
+          const float k = p == pos ? kvn[0][i] : __bfloat162float(kbase[(size_t)p * HD + i]);
+          v[e] = p == pos ? kvn[1][i] : __bfloat162float(vbase[(size_t)p * HD + i]);
+          s = fmaf(h0 + hq < rep ? qs[h0 + hq][i] : 0.f, k, s);
+        }
+        for (int x = 16; x >= 1; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+        const float mn = fmaxf(m, s), al = mn == -INFINITY ? 1.f : exp2f(m - mn);
+        const float pr = s == -INFINITY ? 0.f : exp2f(s - mn);
+        l = l * al + pr;
+        m = mn;
+        for (int e = 0; e < E; ++e) o[e] = fmaf(pr, v[e], o[e] * al);
+      }
+    if (lane == 0) {
+      ws_m[hq] = m;
+      ws_l[hq] = l;
+    }
+    for (int e = 0; e < E; ++e) ws_o[hq][lane * E + e] = o[e];
+  }
+  __syncwarp();
 }
 
 // Dynamic shared memory: per warp two chunk buffers of K and V rows,
@@ -94,19 +144,23 @@ __device__ __forceinline__ void attn_issue(__nv_bfloat16 *dst, const __nv_bfloat
 template <int HD>
 constexpr int attn_smem_bytes() { return kAttnWarps * 2 * 2 * kPos * HD * 2; }
 
+// grid (B * n_kv, S), block kAttnWarps * 32.  part: [B][H][S][HD + 2] fp32
+// (accumulator, max, sum) of every split.
 template <int HD>
-__global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
+__global__ void __launch_bounds__(kAttnWarps * 32, kAttnOcc) attn_split_kernel(
     const float *qkv, const __nv_bfloat16 *x, const int *lens, int d, int H, int Hkv, const RopeFreq fr,
     __nv_bfloat16 *k_cache, __nv_bfloat16 *v_cache, int max_len, float *part, int S) {
   constexpr int E = HD / 32;  // dimensions a lane holds
   extern __shared__ __align__(16) uint8_t attn_dyn[];
-  __shared__ float qs[kHG * 2][HD];  // the group's query heads (up to 8), scaled by 1/sqrt(HD)
+  __shared__ __align__(16) float qs[kHG * 2][HD];  // the group's query heads (up to 8), scaled by log2(e)/sqrt(HD)
   __shared__ float kvn[2][HD];       // the new token's k (normalized, rotated, bf16-rounded) and v
   __shared__ float red[kAttnWarps];
   __shared__ float rc[HD / 2], rsn[HD / 2];  // cos, sin of the RoPE angles at this position
   __shared__ float ws_m[kAttnWarps][kHG * 2], ws_l[kAttnWarps][kHG * 2];
-  __shared__ float ws_o[kAttnWarps][kHG][HD];
+  __shared__ __align__(16) float ps_s[kAttnWarps][kHG][kPos];  // a chunk's probabilities
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  pdl_launch_dependents();
   const int b = blockIdx.x / Hkv, g = blockIdx.x % Hkv, split = blockIdx.y;
   const int rep = H / Hkv;
   const int pos = lens[b];          // the new token's position
@@ -133,9 +187,14 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
   }
   // 1. rs of x[b]
   float ss = 0.f;
-  for (int i = tid; i < d; i += blockDim.x) {
-    const float v = __bfloat162float(x[(size_t)b * d + i]);
-    ss = fmaf(v, v, ss);
+  for (int i = tid; i < d / 8; i += blockDim.x) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(x + (size_t)b * d + 8 * i);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      ss = fmaf(bf_lo(w[e]), bf_lo(w[e]), ss);
+      ss = fmaf(bf_hi(w[e]), bf_hi(w[e]), ss);
+    }
   }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -174,7 +233,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
       }
     }
     if (hh < rep) {
-      const float qsc = __frsqrt_rn((float)HD);
+      const float qsc = 1.4426950408889634f * __frsqrt_rn((float)HD);  // scores in units of log 2: exp2f below
 #pragma unroll
       for (int e = 0; e < E; ++e) qs[hh][lane * E + e] = v[e] * qsc;
     } else {
@@ -190,117 +249,146 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
   __syncthreads();
 
   // 4. attention over [p0, p1): per pass, 4 query heads
+  const int gr = lane >> 2, tc = lane & 3;  // fragment row and column pair
+  constexpr int WBYTES = 2 * 2 * kPos * HD * 2;  // a warp's buffers; after the loop its accumulator [kHG][HD]
+  __nv_bfloat16 *wbuf = reinterpret_cast<__nv_bfloat16 *>(attn_dyn + warp * WBYTES);
+  auto ws_o = [&](int w) { return reinterpret_cast<float(*)[HD]>(attn_dyn + w * WBYTES); };
+  const __nv_bfloat16 *kbase = k_cache + cache_off, *vbase = v_cache + cache_off;
+  constexpr int stride = kAttnWarps * kPos;
+  const int first = p0 + warp * kPos;
+  // ldmatrix row of this lane: matrices (rows 0-7, 8-15) x (16-byte chunk 2 j, 2 j + 1)
+  const int lrow = (lane & 7) + (lane & 8), lchk = lane >> 4;
   for (int h0 = 0; h0 < rep; h0 += kHG) {
-    float q[kHG][E];
-#pragma unroll
-    for (int hq = 0; hq < kHG; ++hq)
-#pragma unroll
-      for (int e = 0; e < E; ++e) q[hq][e] = h0 + hq < rep ? qs[h0 + hq][lane * E + e] : 0.f;
-    float m_run = -INFINITY, l_run = 0.f;  // of head h0 + (lane & 3)
-    float acc[kHG][E];
-#pragma unroll
-    for (int hq = 0; hq < kHG; ++hq)
-#pragma unroll
-      for (int e = 0; e < E; ++e) acc[hq][e] = 0.f;
-    // this warp's chunk buffers; positions outside [p0, p1) and the new
-    // position (taken from kvn) are zero-filled
-    __nv_bfloat16 *wbuf = reinterpret_cast<__nv_bfloat16 *>(attn_dyn) + (size_t)warp * 2 * 2 * kPos * HD;
-    constexpr int CPR = HD * 2 / 16;  // 16-byte copies a row
-    // copy i of a lane: row r = i * (32 / CPR) + lane / CPR of the [K, V][kPos]
-    // rows, 16 bytes at column lane % CPR
-    const int lrow = lane / CPR, lcol = (lane % CPR) * 8;
-    const __nv_bfloat16 *kbase = k_cache + cache_off + lcol, *vbase = v_cache + cache_off + lcol;
-    constexpr int stride = kAttnWarps * kPos;
-    int bi = 0;
-    if (p0 + warp * kPos < p1)
-      attn_issue<HD>(wbuf + lcol, kbase, vbase, lrow, p0 + warp * kPos, p0, p1, pos);
+    if (first < p1) attn_issue<HD>(wbuf, kbase, vbase, lane, first, p0, p1, pos);
     cp_async_commit();
-    for (int c0 = p0 + warp * kPos; c0 < p1; c0 += stride, bi ^= 1) {
+    // Q's parts as B fragments: column gr of tile 0 is part gr % 2 of head gr / 2,
+    // of tile 1 (even gr) its third part
+    uint32_t qb[HD / 16][2][2];
+#pragma unroll
+    for (int ks = 0; ks < HD / 16; ++ks)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float pa[3] = {0.f, 0.f, 0.f}, pb[3] = {0.f, 0.f, 0.f};
+        if (h0 + (gr >> 1) < rep) {
+          const float2 qv = *reinterpret_cast<const float2 *>(&qs[h0 + (gr >> 1)][16 * ks + 8 * u + 2 * tc]);
+          split3(qv.x, pa);
+          split3(qv.y, pb);
+        }
+        qb[ks][0][u] = gr & 1 ? pack_bf2(pa[1], pb[1]) : pack_bf2(pa[0], pb[0]);
+        qb[ks][1][u] = gr & 1 ? 0u : pack_bf2(pa[2], pb[2]);
+      }
+    float m_run = -INFINITY, l_run = 0.f;  // of head h0 + tc (l_run: this lane's positions)
+    float acc[HD / 8][4];                  // rows gr, gr + 8 of P V: heads' parts
+#pragma unroll
+    for (int j = 0; j < HD / 8; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    int bi = 0;
+    for (int c0 = first; c0 < p1; c0 += stride, bi ^= 1) {
       if (c0 + stride < p1)
-        attn_issue<HD>(wbuf + (size_t)(bi ^ 1) * 2 * kPos * HD + lcol, kbase, vbase, lrow, c0 + stride, p0, p1, pos);
+        attn_issue<HD>(wbuf + (size_t)(bi ^ 1) * 2 * kPos * HD, kbase, vbase, lane, c0 + stride, p0, p1, pos);
       cp_async_commit();
       cp_async_wait_group1();  // this chunk's rows have landed
       __syncwarp();
-      const __nv_bfloat16 *cur = wbuf + (size_t)bi * 2 * kPos * HD;
-      // partial dots of 8 positions x 4 heads: index pp * 4 + hq
-      float sv[32];
-      float vv[kPos][E];
-#pragma unroll
-      for (int pp = 0; pp < kPos; ++pp) {
-        const int p = c0 + pp;
-        float kr[E];
-        if (p != pos) {
-          load_row_s<HD>(cur + (size_t)pp * HD + lane * E, kr);
-          load_row_s<HD>(cur + (size_t)(kPos + pp) * HD + lane * E, vv[pp]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            kr[e] = kvn[0][lane * E + e];
-            vv[pp][e] = kvn[1][lane * E + e];
-          }
+      __nv_bfloat16 *cur = wbuf + (size_t)bi * 2 * kPos * HD;
+      if (c0 <= pos && pos < c0 + kPos) {  // the new token's rows
+        const int r = pos - c0;
+        for (int i = lane; i < 2 * HD; i += 32) {
+          const int row = (i / HD) * kPos + r, e = i % HD;
+          cur[(size_t)row * HD + ((e >> 3) ^ (row & 7)) * 8 + (e & 7)] = __float2bfloat16_rn(kvn[i / HD][e]);
         }
-#pragma unroll
-        for (int hq = 0; hq < kHG; ++hq) {
-          float dsum = 0.f;
-#pragma unroll
-          for (int e = 0; e < E; ++e) dsum = fmaf(q[hq][e], kr[e], dsum);
-          sv[pp * kHG + hq] = dsum;
-        }
+        __syncwarp();
       }
-      // reduce-scatter: afterwards lane l holds the full dot of index l
+      const uint32_t krow = smem_addr(cur) + lrow * (HD * 2), vrow = krow + kPos * HD * 2;
+      // Each MMA starts from zero and is added in fp32 here (likewise for P V):
+      // the tensor core's own accumulation truncates, which showed as twice the
+      // outputs off the exact rounding.
+      float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int hb = 16; hb >= 1; hb >>= 1) {
+      for (int ks = 0; ks < HD / 16; ++ks) {
+        uint32_t ka[4];
+        ldmatrix_x4(ka, krow + (((2 * ks + lchk) ^ (lrow & 7)) << 4));
+        float t0[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16_16816(t0, ka, qb[ks][0][0], qb[ks][0][1]);
+        mma_bf16_16816(d1, ka, qb[ks][1][0], qb[ks][1][1]);
 #pragma unroll
-        for (int j = 0; j < hb; ++j) {
-          const bool up = (lane & hb) != 0;
-          const float keep = up ? sv[j + hb] : sv[j];
-          const float send = up ? sv[j] : sv[j + hb];
-          sv[j] = keep + __shfl_xor_sync(0xffffffffu, send, hb);
-        }
+        for (int e = 0; e < 4; ++e) d0[e] += t0[e];
       }
-      const int my_p = c0 + (lane >> 2);
-      const float s = my_p < p1 ? sv[0] : -INFINITY;
-      // online softmax per head (the 8 lanes of head lane & 3)
-      float mc = s;
+      // scores of positions c0 + gr, c0 + gr + 8 with head h0 + tc
+      const float s0 = c0 + gr < p1 ? (d0[0] + d0[1]) + d1[0] : -INFINITY;
+      const float s1 = c0 + gr + 8 < p1 ? (d0[2] + d0[3]) + d1[2] : -INFINITY;
+      float mc = fmaxf(s0, s1);
       mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 4));
       mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 8));
       mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 16));
       const float m_new = fmaxf(m_run, mc);
-      const float alpha = m_new == -INFINITY ? 1.f : __expf(m_run - m_new);
-      const float pr = s == -INFINITY ? 0.f : __expf(s - m_new);
-      float ps = pr;
-      ps += __shfl_xor_sync(0xffffffffu, ps, 4);
-      ps += __shfl_xor_sync(0xffffffffu, ps, 8);
-      ps += __shfl_xor_sync(0xffffffffu, ps, 16);
-      l_run = l_run * alpha + ps;
+      const float alpha = m_new == -INFINITY ? 1.f : exp2f(m_run - m_new);
+      const float e0 = s0 == -INFINITY ? 0.f : exp2f(s0 - m_new), e1 = s1 == -INFINITY ? 0.f : exp2f(s1 - m_new);
+      l_run = l_run * alpha + (e0 + e1);
       m_run = m_new;
-      // accumulators: rescale per head, add p v
+      ps_s[warp][tc][gr] = e0;
+      ps_s[warp][tc][gr + 8] = e1;
+      if (__any_sync(0xffffffffu, alpha != 1.f)) {
+        const float al = __shfl_sync(0xffffffffu, alpha, (lane & 28) | (gr & 3));  // of head gr % 4
 #pragma unroll
-      for (int hq = 0; hq < kHG; ++hq) {
-        const float al = __shfl_sync(0xffffffffu, alpha, hq);
+        for (int j = 0; j < HD / 8; ++j)
 #pragma unroll
-        for (int e = 0; e < E; ++e) acc[hq][e] *= al;
+          for (int e = 0; e < 4; ++e) acc[j][e] *= al;
+      }
+      __syncwarp();
+      // P's parts as the A fragment: row gr is part gr / 4 of head gr % 4, row gr
+      // + 8 (gr < 4) its third part
+      uint32_t pa[4];
+      {
+        const float2 x0 = *reinterpret_cast<const float2 *>(&ps_s[warp][gr & 3][2 * tc]);
+        const float2 x1 = *reinterpret_cast<const float2 *>(&ps_s[warp][gr & 3][2 * tc + 8]);
+        float q0[3], q1[3], q2[3], q3[3];
+        split3(x0.x, q0);
+        split3(x0.y, q1);
+        split3(x1.x, q2);
+        split3(x1.y, q3);
+        const bool lo = gr < 4;
+        pa[0] = lo ? pack_bf2(q0[0], q1[0]) : pack_bf2(q0[1], q1[1]);
+        pa[1] = lo ? pack_bf2(q0[2], q1[2]) : 0u;
+        pa[2] = lo ? pack_bf2(q2[0], q3[0]) : pack_bf2(q2[1], q3[1]);
+        pa[3] = lo ? pack_bf2(q2[2], q3[2]) : 0u;
       }
 #pragma unroll
-      for (int pp = 0; pp < kPos; ++pp)
+      for (int j = 0; j < HD / 16; ++j) {
+        uint32_t vb[4];
+        ldmatrix_x4_trans(vb, vrow + (((2 * j + lchk) ^ (lrow & 7)) << 4));
+        float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16_16816(t0, pa, vb[0], vb[1]);
+        mma_bf16_16816(t1, pa, vb[2], vb[3]);
 #pragma unroll
-        for (int hq = 0; hq < kHG; ++hq) {
-          const float pw = __shfl_sync(0xffffffffu, pr, pp * kHG + hq);
-#pragma unroll
-          for (int e = 0; e < E; ++e) acc[hq][e] = fmaf(pw, vv[pp][e], acc[hq][e]);
+        for (int e = 0; e < 4; ++e) {
+          acc[2 * j][e] += t0[e];
+          acc[2 * j + 1][e] += t1[e];
         }
+      }
       __syncwarp();  // every lane is done with this buffer before it is filled again
     }
     cp_async_wait_all();
-    // merge the warps (fixed order) and write the split's partials
+    // the parts added up: head h0 + gr (gr < 4), dimensions 8 j + 2 tc, + 1
+    bool bad = m_run != m_run;
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+#pragma unroll
+    for (int j = 0; j < HD / 8; ++j)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float mid = __shfl_xor_sync(0xffffffffu, acc[j][e], 16);
+        const float v = (acc[j][2 + e] + mid) + acc[j][e];
+        bad |= gr < 4 && v != v;
+        if (gr < 4) ws_o(warp)[gr][8 * j + 2 * tc + e] = v;
+      }
     if (lane < kHG) {
       ws_m[warp][lane] = m_run;
       ws_l[warp][lane] = l_run;
     }
-#pragma unroll
-    for (int hq = 0; hq < kHG; ++hq)
-#pragma unroll
-      for (int e = 0; e < E; ++e) ws_o[warp][hq][lane * E + e] = acc[hq][e];
+    if (__any_sync(0xffffffffu, bad || l_run != l_run))
+      attn_plain<HD>(qs, kvn, kbase, vbase, h0, rep, first, stride, p1, pos, ws_m[warp], ws_l[warp], ws_o(warp));
+    // merge the warps (fixed order) and write the split's partials
     __syncthreads();
     for (int i = tid; i < kHG * HD; i += blockDim.x) {
       const int hq = i / HD, e = i % HD;
@@ -309,9 +397,9 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
       for (int w = 0; w < kAttnWarps; ++w) M = fmaxf(M, ws_m[w][hq]);
       float Ls = 0.f, O = 0.f;
       for (int w = 0; w < kAttnWarps; ++w) {
-        const float f = ws_m[w][hq] == -INFINITY ? 0.f : __expf(ws_m[w][hq] - M);
+        const float f = ws_m[w][hq] == -INFINITY ? 0.f : exp2f(ws_m[w][hq] - M);
         Ls = fmaf(ws_l[w][hq], f, Ls);
-        O = fmaf(ws_o[w][hq][e], f, O);
+        O = fmaf(ws_o(w)[hq][e], f, O);
       }
       const int h = g * rep + h0 + hq;
       float *pt = part + (((size_t)b * H + h) * S + split) * (HD + 2);
@@ -325,29 +413,32 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) attn_split_kernel(
   }
 }
 
-// o[b][h * HD + e] = bf16( sum_s O_s e^(M_s - M) / sum_s L_s e^(M_s - M) ).
+// o[b][h * HD + e] = bf16( sum_s O_s 2^(M_s - M) / sum_s L_s 2^(M_s - M) ).
 // grid B * H, 8 warps: warp w merges the splits w, w + 8, .. in order (its
 // own max first), lane l the features l * HD/32 ..; then the warps' results
 // are merged in warp order -- a fixed order, so the result is deterministic.
 template <int HD>
-__global__ void __launch_bounds__(kAttnWarps * 32) attn_combine_kernel(const float *part, const int *lens, int H, int S,
+__global__ void __launch_bounds__(kCombWarps * 32) attn_combine_kernel(const float *part, const int *lens, int H, int S,
                                                                        int max_len, __nv_bfloat16 *o) {
   constexpr int E = HD / 32;
-  __shared__ float wm[kAttnWarps], wl[kAttnWarps], wo[kAttnWarps][HD];
+  __shared__ float wm[kCombWarps], wl[kCombWarps], wo[kCombWarps][HD];
   const int bh = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_launch_dependents();
   const int pos = lens[bh / H];
   if (pos < 0 || pos >= max_len) return;  // skipped by the split kernel
   const float *pt = part + (size_t)bh * S * (HD + 2);
   float M = -INFINITY;
-  for (int s = warp; s < S; s += kAttnWarps) M = fmaxf(M, pt[(size_t)s * (HD + 2) + HD]);
+#pragma unroll 8
+  for (int s = warp; s < S; s += kCombWarps) M = fmaxf(M, pt[(size_t)s * (HD + 2) + HD]);
   float L = 0.f, O[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) O[e] = 0.f;
 #pragma unroll 4
-  for (int s = warp; s < S; s += kAttnWarps) {
+  for (int s = warp; s < S; s += kCombWarps) {
     const float *ps = pt + (size_t)s * (HD + 2);
     const float ms = ps[HD];
-    const float f = ms == -INFINITY ? 0.f : __expf(ms - M);
+    const float f = ms == -INFINITY ? 0.f : exp2f(ms - M);
     L = fmaf(ps[HD + 1], f, L);
 #pragma unroll
     for (int e = 0; e < E; ++e) O[e] = fmaf(ps[lane * E + e], f, O[e]);
@@ -361,10 +452,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attn_combine_kernel(const flo
   __syncthreads();
   for (int e = threadIdx.x; e < HD; e += blockDim.x) {
     float Mt = -INFINITY;
-    for (int w = 0; w < kAttnWarps; ++w) Mt = fmaxf(Mt, wm[w]);
+    for (int w = 0; w < kCombWarps; ++w) Mt = fmaxf(Mt, wm[w]);
     float Lt = 0.f, Ot = 0.f;
-    for (int w = 0; w < kAttnWarps; ++w) {
-      const float f = wm[w] == -INFINITY ? 0.f : __expf(wm[w] - Mt);
+    for (int w = 0; w < kCombWarps; ++w) {
+      const float f = wm[w] == -INFINITY ? 0.f : exp2f(wm[w] - Mt);
       Lt = fmaf(wl[w], f, Lt);
       Ot = fmaf(wo[w][e], f, Ot);
     }
@@ -373,37 +464,52 @@ __global__ void __launch_bounds__(kAttnWarps * 32) attn_combine_kernel(const flo
 }
 
 int attn_splits(int B, int Hkv, int max_len, int num_sms) {
-  // enough CTAs to cover the SMs twice, at least 64 positions a split
-  const int want = std::max(1, (2 * num_sms + B * Hkv - 1) / (B * Hkv));
+  // as many CTAs as the SMs hold at once, at least 64 positions a split
+  const int want = std::max(1, kAttnOcc * num_sms / (B * Hkv));
   return std::max(1, std::min(want, (max_len + 63) / 64));
 }
+
+namespace {
+
+template <int HD>
+cudaError_t launch_attn_t(const float *qkv, const __nv_bfloat16 *x, const int *lens, int B, int d, int H, int Hkv,
+                          const RopeFreq &fr, __nv_bfloat16 *kc, __nv_bfloat16 *vc, int max_len, float *part, int S,
+                          __nv_bfloat16 *o, cudaStream_t s) {
+  constexpr int sm = attn_smem_bytes<HD>();
+  cudaError_t e = cudaFuncSetAttribute(attn_split_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(B * Hkv, S);
+  cfg.blockDim = dim3(kAttnWarps * 32);
+  cfg.dynamicSmemBytes = sm;
+  e = cudaLaunchKernelEx(&cfg, attn_split_kernel<HD>, qkv, x, lens, d, H, Hkv, fr, kc, vc, max_len, part, S);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3(B * H);
+  cfg.blockDim = dim3(kCombWarps * 32);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, attn_combine_kernel<HD>, (const float *)part, lens, H, S, max_len, o);
+}
+
+}  // namespace
 
 cudaError_t launch_attn_decode(const float *qkv, const void *x, const int *lens, int B, int d, int H, int Hkv, int HD,
                                double theta, void *k_cache, void *v_cache, int max_len, float *part, int S, void *o,
                                cudaStream_t s) {
-  const dim3 grid(B * Hkv, S);
   if (HD > 128) return cudaErrorInvalidValue;
   RopeFreq fr{};
   for (int i = 0; i < HD / 2; ++i) fr.f[i] = std::pow(theta, -2.0 * i / HD);
   const auto *xb = reinterpret_cast<const __nv_bfloat16 *>(x);
   auto *kc = reinterpret_cast<__nv_bfloat16 *>(k_cache), *vc = reinterpret_cast<__nv_bfloat16 *>(v_cache);
   auto *ob = reinterpret_cast<__nv_bfloat16 *>(o);
-  if (HD == 128) {
-    constexpr int sm = attn_smem_bytes<128>();
-    cudaError_t e = cudaFuncSetAttribute(attn_split_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e != cudaSuccess) return e;
-    attn_split_kernel<128><<<grid, kAttnWarps * 32, sm, s>>>(qkv, xb, lens, d, H, Hkv, fr, kc, vc, max_len, part, S);
-    attn_combine_kernel<128><<<B * H, kAttnWarps * 32, 0, s>>>(part, lens, H, S, max_len, ob);
-  } else if (HD == 64) {
-    constexpr int sm = attn_smem_bytes<64>();
-    cudaError_t e = cudaFuncSetAttribute(attn_split_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e != cudaSuccess) return e;
-    attn_split_kernel<64><<<grid, kAttnWarps * 32, sm, s>>>(qkv, xb, lens, d, H, Hkv, fr, kc, vc, max_len, part, S);
-    attn_combine_kernel<64><<<B * H, kAttnWarps * 32, 0, s>>>(part, lens, H, S, max_len, ob);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  if (HD == 128) return launch_attn_t<128>(qkv, xb, lens, B, d, H, Hkv, fr, kc, vc, max_len, part, S, ob, s);
+  if (HD == 64) return launch_attn_t<64>(qkv, xb, lens, B, d, H, Hkv, fr, kc, vc, max_len, part, S, ob, s);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t read_attn_status(int *status) {

@@ -164,6 +164,22 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_
                : "memory");
 }
 
+// Loads four 8x8 matrices of 16-bit elements into the fragment layout of
+// stmatrix_x4; lane l gives the address of row l % 8 of matrix l / 8.  _trans:
+// each matrix transposed.
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t saddr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(saddr)
+               : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t saddr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(saddr)
+               : "memory");
+}
+
 // True in one lane of a converged warp (the same one every time).  Used where
 // one thread issues tcgen05.mma or TMA instructions: elect.sync tells the
 // compiler that a single lane is active, which `lane == 0` does not.

@@ -1,0 +1,77 @@
+"""Decode attention at the edges of its 16-position chunks, 64-position warp
+strides and splits, against fp64 torch on the same cache; and an infinite cache
+entry, which the kernel's bf16 parts would turn into NaN, computed as plain
+products do."""
+import math
+
+import pytest
+import torch
+
+from paper_2606_04238_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wq():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2606_04238_gb300 import wq as mod
+    return mod
+
+
+def _rms(x):
+    return x / torch.sqrt((x * x).mean(-1, keepdim=True) + 1e-6)
+
+
+def _rope(v, pos, theta):
+    hd = v.shape[-1]
+    a = pos.double()[:, None, None] * theta ** (-2.0 * torch.arange(hd // 2, dtype=torch.float64) / hd)
+    lo, hi = v[..., :hd // 2], v[..., hd // 2:]
+    return torch.cat([lo * torch.cos(a) - hi * torch.sin(a), hi * torch.cos(a) + lo * torch.sin(a)], -1)
+
+
+def _case(wq, H, kv, hd, lens, max_len, seed, spoil=None):
+    B, d = len(lens), 256
+    g = torch.Generator().manual_seed(seed)
+    x = synth.activations((B, d), seed)
+    qkv = torch.randn((B, (H + 2 * kv) * hd), generator=g)
+    kc = torch.randn((B, kv, max_len, hd), generator=g).to(torch.bfloat16)
+    vc = torch.randn((B, kv, max_len, hd), generator=g).to(torch.bfloat16)
+    if spoil:
+        spoil(kc, vc)
+    L = torch.tensor(lens, dtype=torch.int32)
+    kd, vd = kc.cuda(), vc.cuda()
+    o = wq.attn_decode(qkv.cuda(), x.cuda(), L.cuda(), kd, vd, H, kv, 1e6)
+    torch.cuda.synchronize()
+    assert wq.device_status() == 0
+    xs = x.double()
+    q = (qkv.double() / torch.sqrt((xs * xs).mean(-1, keepdim=True) + 1e-6)).view(B, H + 2 * kv, hd)[:, :H]
+    q = _rope(_rms(q), L, 1e6)
+    kh, vh = kd.cpu().double(), vd.cpu().double()  # with the appended position, as stored
+    ref = torch.empty((B, H, hd), dtype=torch.float64)
+    for b in range(B):
+        n = lens[b] + 1
+        p = torch.softmax(q[b].view(kv, H // kv, hd) @ kh[b, :, :n].transpose(1, 2) / math.sqrt(hd), -1)
+        ref[b] = (p @ vh[b, :, :n]).view(H, hd)
+    return o.cpu().double().view(B, H, hd), ref
+
+
+@pytest.mark.parametrize("H,kv,hd", [(8, 2, 128), (6, 2, 64), (8, 1, 128)])
+def test_chunk_edges(wq, H, kv, hd):
+    lens = [0, 1, 14, 15, 16, 17, 63, 64, 65, 127, 128, 200, 255]
+    got, ref = _case(wq, H, kv, hd, lens, 256, 3)
+    # one bf16 rounding of the output (2^-9) and fp32 scores: 1e-5 of the largest value
+    tol = ref.abs() * 2.0 ** -8 + 1e-5 * ref.abs().max()
+    assert ((got - ref).abs() <= tol).all()
+
+
+def test_infinite_value_row(wq):
+    def spoil(kc, vc):
+        vc[0, 1, 20, 5] = float("inf")
+        vc[1, 0, 3, 7] = -float("inf")
+    got, ref = _case(wq, 8, 2, 128, [40, 90], 128, 4, spoil)
+    assert torch.isinf(ref).sum() == 8
+    assert torch.equal(torch.isinf(got), torch.isinf(ref)) and not torch.isnan(got).any()
+    f = torch.isfinite(ref)
+    assert ((got - ref)[f].abs() <= ref[f].abs() * 2.0 ** -8 + 1e-5 * ref[f].abs().max()).all()
