@@ -450,7 +450,10 @@ wq_status run_gateup_batch(GemvKind kind, const void *x, int m, const wq_qweight
   a.panel = ws + L.bpx;
   float *rs = (flags & WQ_PRENORM) ? reinterpret_cast<float *>(ws + L.brs) : nullptr;
   uint8_t *tf = r > 0 ? ws + L.btf : nullptr;
-  cudaError_t e = launch_batch_prep(x, m, gate->k, gate->bits, gate->group, lora_a, r, lora_scale, ws + L.bpx, rs, tf, s);
+  a.cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
+  const int n_cnt = (std::max(gate->k, gate->n) + 127) / 128;
+  cudaError_t e = launch_batch_prep(x, m, gate->k, gate->bits, gate->group, lora_a, r, lora_scale, ws + L.bpx, rs, tf,
+                                    a.cnt, n_cnt, s);
   if (e != cudaSuccess) return cuda_fail(e, "batched input launch");
   a.M = m;
   a.N = gate->n;
@@ -469,7 +472,6 @@ wq_status run_gateup_batch(GemvKind kind, const void *x, int m, const wq_qweight
   a.panel_out = panel_down ? ws + L.bph : nullptr;
   a.group_out = panel_down ? panel_down->group : 128;
   a.part = reinterpret_cast<float *>(ws + L.bpart);
-  a.cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
   if ((e = launch_batch(kind, a, s)) != cudaSuccess) return cuda_fail(e, "batched gate/up launch");
   return WQ_OK;
 }
@@ -479,8 +481,9 @@ wq_status run_down_batch(const void *h, int m, const wq_qweight *down, const voi
                          const WsLayout &L, uint8_t *ws, cudaStream_t s) {
   if (!L.batch) return fail(WQ_ERR_WORKSPACE, "workspace laid out without the batched-decode buffers");
   cudaError_t e;
-  if (h && (e = launch_batch_prep(h, m, down->k, 4, down->group, nullptr, 0, 0.f, ws + L.bph, nullptr, nullptr, s)) !=
-               cudaSuccess)
+  unsigned *cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
+  if (h && (e = launch_batch_prep(h, m, down->k, 4, down->group, nullptr, 0, 0.f, ws + L.bph, nullptr, nullptr, cnt,
+                                  (down->n + 127) / 128, s)) != cudaSuccess)
     return cuda_fail(e, "batched input launch");
   BatchArgs a = {};
   a.panel = ws + L.bph;
@@ -494,7 +497,7 @@ wq_status run_down_batch(const void *h, int m, const wq_qweight *down, const voi
   a.out = y;
   a.out_f32 = y_f32;
   a.part = reinterpret_cast<float *>(ws + L.bpart);
-  a.cnt = reinterpret_cast<unsigned *>(ws + L.bcnt);
+  a.cnt = cnt;
   if ((e = launch_batch(kDownW4, a, s)) != cudaSuccess) return cuda_fail(e, "batched down launch");
   return WQ_OK;
 }
@@ -1373,11 +1376,15 @@ namespace {
 // More slots than kMoeBatchAbove are grouped by expert instead and run on the
 // batched-decode kernels: segments of up to 8 nt slots of one expert, whose
 // weights are then read once a segment, not once a slot.
+//
+// Both layouts start with the slots' counters at the same offsets (zero once),
+// so calls of different token counts may share a workspace; the grouped
+// path's are zeroed by its input launch.
 struct MoeWs {
   GemvPlan gu, dn;
   size_t cnt_gu, cnt_dn, idx, w, tp, h, ys, part_gu, part_dn, total;
   int nt, max_segs;  // grouped: token tiles a segment, segments at most (0: slots)
-  size_t route, panel, hpanel, rs, tf, part;
+  size_t route, panel, hpanel, rs, tf, part, cnt_bu, cnt_bd;
 };
 
 // Measured (GPT-OSS-20B shape, 32 experts top-4, us a block, slots vs grouped):
@@ -1431,20 +1438,28 @@ wq_status moe_check(int m, const wq_moe_layer *layer) {
   return WQ_OK;
 }
 
+// The counter block every MoE layout starts with (up to kMoeBatchAbove slots).
+size_t moe_slot_counters(int d, int inter, MoeWs *W) {
+  size_t off = 0;
+  W->cnt_gu = off; off = up256(off + (size_t)kMoeBatchAbove * ((inter + 15) / 16) * 4);
+  W->cnt_dn = off; off = up256(off + (size_t)kMoeBatchAbove * ((d + 15) / 16) * 4);
+  return off;
+}
+
 bool moe_ws(int m, const wq_moe_layer &L, unsigned flags, MoeWs *W) {
   const wq_mlp_layer &X = L.experts;
   const int E = L.n_experts, S = m * L.top_k, d = X.gate.k, inter = X.gate.n / E, r = X.r;
   const GemvKind kgu = X.gate.bits == 4 ? kGateUpW4 : kGateUpW2;
   *W = MoeWs{};
-  if (S > kMoeBatchAbove && d % 32 == 0) {
+  if (S > kMoeBatchAbove) {
     const int sms = num_sms();
     if (sms <= 0) return false;
     W->nt = moe_batch_nt(S, E);
     W->max_segs = batch_max_segs(S, E, W->nt);
     const size_t segs = W->max_segs, KBd = (d + 127) / 128, KBi = (inter + 127) / 128;
-    size_t off = 0;
-    W->cnt_gu = off; off = up256(off + segs * KBi * 4);
-    W->cnt_dn = off; off = up256(off + segs * KBd * 4);
+    size_t off = moe_slot_counters(d, inter, W);
+    W->cnt_bu = off; off = up256(off + segs * KBi * 4);
+    W->cnt_bd = off; off = up256(off + segs * KBd * 4);
     W->idx = off;    off = up256(off + (size_t)S * 4);
     W->w = off;      off = up256(off + (size_t)S * 4);
     W->route = off;  off = up256(off + sizeof(BatchRoute));
@@ -1460,9 +1475,7 @@ bool moe_ws(int m, const wq_moe_layer &L, unsigned flags, MoeWs *W) {
   if (!moe_plan(kgu, inter, d, X.gate.group, r, S, &W->gu) || !moe_plan(kDownW4, d, inter, X.down.group, 0, S, &W->dn))
     return false;
   const bool need_tp = (flags & WQ_PRENORM) || r > 0;
-  size_t off = 0;
-  W->cnt_gu = off;  off = up256(off + (size_t)S * W->gu.RT * 4);
-  W->cnt_dn = off;  off = up256(off + (size_t)S * W->dn.RT * 4);
+  size_t off = moe_slot_counters(d, inter, W);
   W->idx = off;     off = up256(off + (size_t)S * 4);
   W->w = off;       off = up256(off + (size_t)S * 4);
   W->tp = off;      off = up256(off + (need_tp ? (size_t)S * (d / 16) * WQ_TP_STRIDE(r) * 4 : 0));
@@ -1515,10 +1528,11 @@ wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe
     const GemvKind kgu = X.gate.bits == 4 ? kGateUpW4 : kGateUpW2;
     float *rs = (flags & WQ_PRENORM) ? reinterpret_cast<float *>(w8 + W.rs) : nullptr;
     uint8_t *tf = r > 0 ? w8 + W.tf : nullptr;
+    unsigned *cnt_bu = reinterpret_cast<unsigned *>(w8 + W.cnt_bu);
     cudaError_t e = launch_batch_route(logits, m, E, k, W.nt, idx, wt, route, s);
     if (e != cudaSuccess) return cuda_fail(e, "MoE routing launch");
     e = launch_batch_route_prep(x, d, X.gate.bits, X.gate.group, k, X.lora_a, r, X.lora_scale, w8 + W.panel, rs, tf,
-                                route, W.max_segs, W.nt, s);
+                                cnt_bu, (int)((W.idx - W.cnt_bu) / 4), route, W.max_segs, W.nt, s);
     if (e != cudaSuccess) return cuda_fail(e, "MoE input launch");
     BatchArgs a = {};
     a.panel = w8 + W.panel;
@@ -1538,7 +1552,7 @@ wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe
     a.panel_out = w8 + W.hpanel;
     a.group_out = X.down.group;
     a.part = reinterpret_cast<float *>(w8 + W.part);
-    a.cnt = reinterpret_cast<unsigned *>(w8 + W.cnt_gu);
+    a.cnt = cnt_bu;
     a.route = route;
     if ((e = launch_batch_routed(kgu, a, W.max_segs, W.nt, s)) != cudaSuccess) return cuda_fail(e, "MoE gate/up launch");
     BatchArgs b = {};
@@ -1551,7 +1565,7 @@ wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe
     b.out = ys;
     b.out_f32 = 1;
     b.part = a.part;
-    b.cnt = reinterpret_cast<unsigned *>(w8 + W.cnt_dn);
+    b.cnt = reinterpret_cast<unsigned *>(w8 + W.cnt_bd);
     b.route = route;
     if ((e = launch_batch_routed(kDownW4, b, W.max_segs, W.nt, s)) != cudaSuccess) return cuda_fail(e, "MoE down launch");
     if ((e = launch_moe_combine(x, m, d, k, wt, ys, y, s)) != cudaSuccess) return cuda_fail(e, "MoE combine launch");

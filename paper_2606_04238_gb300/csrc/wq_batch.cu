@@ -23,7 +23,8 @@ __device__ __forceinline__ uint32_t word4(const uint4 &v, int q) { return q == 0
 // chunks of 32 features and their sums are added in warp order.  A lane loads
 // 8 consecutive features of a row and feeds them to two k-steps in the same
 // permuted order for x and A.  The remaining CTAs convert x into the panel,
-// one (128-feature block, token) a warp.  The rows of A are loaded before the
+// one (128-feature block, token) a warp, and zero the arrival counters of the
+// launches that follow.  The rows of A are loaded before the
 // wait on the launch that wrote x.
 // ROUTED: the same for every segment of the route (nt_total token tiles a
 // segment, max_segs segments at most); the segment's tokens are gathered and
@@ -33,7 +34,8 @@ template <bool ROUTED>
 __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __nv_bfloat16 *x, int M, int K, int wide,
                                                                  int group, const __nv_bfloat16 *lora_a, int r,
                                                                  float lora_scale, uint8_t *panel, float *rs,
-                                                                 uint8_t *tfrag, int nt_total, int row_tiles,
+                                                                 uint8_t *tfrag, unsigned *cnt, int n_cnt,
+                                                                 int nt_total, int row_tiles,
                                                                  const BatchRoute *route, int top_k, int max_segs) {
   __shared__ float part[kPrepWarps][16][9];
   __shared__ float ssp[kPrepWarps][8];
@@ -48,6 +50,8 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __nv_bfl
   };
   if ((int)blockIdx.x >= nsum) {
     if (!ROUTED) pdl_wait();
+    for (int i = ((int)blockIdx.x - nsum) * kPrepThreads + tid; i < n_cnt; i += ((int)gridDim.x - nsum) * kPrepThreads)
+      cnt[i] = 0;
     int item = ((int)blockIdx.x - nsum) * kPrepWarps + warp;
     const int KB = (K + 127) / 128, per = KB * nt_total * 8;
     int4 sg = make_int4(0, M, 0, 0);
@@ -281,7 +285,8 @@ cudaError_t batch_sms(int *sms) {
 }  // namespace
 
 cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, const void *lora_a, int r,
-                              float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, cudaStream_t s) {
+                              float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, unsigned *cnt, int n_cnt,
+                              cudaStream_t s) {
   if (M <= 0 || M > kBatchMaxTokens || K <= 0 || K % 32 != 0) return cudaErrorInvalidValue;
   const int nt = batch_nt(M), KB = (K + 127) / 128;
   const bool lora = tfrag != nullptr && r > 0;
@@ -291,7 +296,7 @@ cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, 
                                         dim3(kPrepThreads), s, attr);
   return cudaLaunchKernelEx(&cfg, batch_prep_kernel<false>, reinterpret_cast<const __nv_bfloat16 *>(x), M, K,
                             bits == 4 ? 1 : 0, group, reinterpret_cast<const __nv_bfloat16 *>(lora_a), r, lora_scale,
-                            panel, rs, lora ? tfrag : (uint8_t *)nullptr, nt, row_tiles,
+                            panel, rs, lora ? tfrag : (uint8_t *)nullptr, cnt, n_cnt, nt, row_tiles,
                             (const BatchRoute *)nullptr, 1, 1);
 }
 
@@ -305,8 +310,8 @@ cudaError_t launch_batch_route(const float *logits, int m, int E, int top_k, int
 }
 
 cudaError_t launch_batch_route_prep(const void *x, int K, int bits, int group, int top_k, const void *lora_a, int r,
-                                    float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag,
-                                    const BatchRoute *route, int max_segs, int nt, cudaStream_t s) {
+                                    float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, unsigned *cnt,
+                                    int n_cnt, const BatchRoute *route, int max_segs, int nt, cudaStream_t s) {
   if (K <= 0 || K % 32 != 0) return cudaErrorInvalidValue;
   const int KB = (K + 127) / 128;
   const bool lora = tfrag != nullptr && r > 0;
@@ -317,7 +322,8 @@ cudaError_t launch_batch_route_prep(const void *x, int K, int bits, int group, i
                    dim3(kPrepThreads), s, attr);
   return cudaLaunchKernelEx(&cfg, batch_prep_kernel<true>, reinterpret_cast<const __nv_bfloat16 *>(x), 0, K,
                             bits == 4 ? 1 : 0, group, reinterpret_cast<const __nv_bfloat16 *>(lora_a), r, lora_scale,
-                            panel, rs, lora ? tfrag : (uint8_t *)nullptr, nt, row_tiles, route, top_k, max_segs);
+                            panel, rs, lora ? tfrag : (uint8_t *)nullptr, cnt, n_cnt, nt, row_tiles, route, top_k,
+                            max_segs);
 }
 
 cudaError_t launch_batch_routed(GemvKind kind, const BatchArgs &a, int max_segs, int nt, cudaStream_t s) {

@@ -63,7 +63,7 @@ struct BatchArgs {
   uint8_t *panel_out;        // gate/up: also the 4-bit down launch's panel of h (null: none)
   int group_out;             // its quantization group
   float *part;               // batch_scratch_floats() fp32
-  unsigned *cnt;             // [ceil(N / 128)] (routed: per segment) arrival counters, zero between launches
+  unsigned *cnt;             // [ceil(N / 128)] (routed: per segment) arrival counters, zeroed by the input launch and left at zero
   // Routed experts: the launch computes segments of up to 8 nt (token, choice)
   // slots of one expert each.  codes, meta, lora_b: the experts' matrices
   // stacked row-wise, N rows an expert (a multiple of 16); panel, tfrag, rs,
@@ -73,18 +73,21 @@ struct BatchArgs {
 
 // Panel of x bf16 [M, K] for codes of `bits` bits and groups of `group`, and
 // with rs / tfrag (either may be null) the RMSNorm scales and LoRA-A products.
+// cnt [n_cnt] is zeroed: the arrival counters of the launches that follow (a
+// workspace used at several token counts holds other data there in between).
 cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, const void *lora_a, int r,
-                              float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, cudaStream_t s);
+                              float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, unsigned *cnt, int n_cnt,
+                              cudaStream_t s);
 cudaError_t launch_batch(GemvKind kind, const BatchArgs &a, cudaStream_t s);
 // Routed: the top_k experts of each token with their softmax weights (slot
 // t * top_k + j), and the slots grouped by expert in segments of 8 nt.
 cudaError_t launch_batch_route(const float *logits, int m, int E, int top_k, int nt, int *idx, float *w,
                                BatchRoute *route, cudaStream_t s);
 // Panels, RMSNorm scales (rs not null) and LoRA-A products (tfrag not null) of
-// every segment; max_segs bounds the grid.
+// every segment, and cnt [n_cnt] zeroed; max_segs bounds the grid.
 cudaError_t launch_batch_route_prep(const void *x, int K, int bits, int group, int top_k, const void *lora_a, int r,
-                                    float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag,
-                                    const BatchRoute *route, int max_segs, int nt, cudaStream_t s);
+                                    float lora_scale, uint8_t *panel, float *rs, uint8_t *tfrag, unsigned *cnt,
+                                    int n_cnt, const BatchRoute *route, int max_segs, int nt, cudaStream_t s);
 // Routed launch: nt 1, 2 or 4; max_segs for the grid.
 cudaError_t launch_batch_routed(GemvKind kind, const BatchArgs &a, int max_segs, int nt, cudaStream_t s);
 size_t batch_scratch_floats(int nt, int nproj, int num_sms);

@@ -162,3 +162,35 @@ def test_batch_stack_of_a_large_layer(wq, bits, m):
     check_bf16(h[0], ref, f"large layer h bits={bits} m={m}")
     ref, _ = orc.down(synth.bf16_bits(h[0].cpu()), qd, group, synth.bf16_bits(x.cpu()))
     check_bf16(y, ref, f"large layer y bits={bits} m={m}")
+
+
+def test_moe_workspace_of_several_token_counts(wq):
+    """One workspace for the largest token count serves smaller ones in between,
+    on the slots' and the grouped launches."""
+    from tests.test_gpu_moe import _build
+    d, inter, E, k, group = 1024, 512, 8, 2, 64
+    layer, _ = _build(wq, d, inter, E, k, group, 8, 900)
+    ws = wq.moe_workspace(64, layer)
+    for i, m in enumerate((64, 1, 7, 6, 33, 2, 64, 12)):
+        x = synth.activations((m, d), 60 + i).cuda()
+        lg = torch.from_numpy(np.random.default_rng(70 + i).standard_normal((m, E)).astype(np.float32)).cuda()
+        y, y0 = wq.moe_forward(x, lg, layer, ws=ws).clone(), wq.moe_forward(x, lg, layer)
+        assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), m
+    assert wq.device_status() == 0
+
+
+def test_decoder_workspace_of_several_batches(wq):
+    """The projections' counters lie elsewhere in a decoder workspace for every batch."""
+    d, inter, H, kv, hd, max_len = 512, 896, 4, 2, 128, 64
+    mk = lambda n, kk, bits, s: upload_packed(*_q((n, kk), 64, bits, s), 64, bits)
+    layer = wq.DecoderLayer(mk((H + 2 * kv) * hd, d, 4, 1), mk(d, H * hd, 4, 2),
+                            wq.MLPLayer(mk(inter, d, 2, 3), mk(inter, d, 2, 4), mk(d, inter, 4, 5)), H, kv, hd, 1e6)
+    ws = wq.decoder_workspace(24, layer, max_len)
+    for i, b in enumerate((24, 12, 1, 17, 9, 24)):
+        x = synth.activations((b, d), 80 + i).cuda()
+        lens = torch.full((b,), 10 + i, dtype=torch.int32, device="cuda")
+        kc, vc = (synth.activations((b, kv, max_len, hd), 90 + j).cuda() for j in range(2))
+        y = wq.decoder_layer_forward(x, lens, layer, kc, vc, ws=ws).clone()
+        y0 = wq.decoder_layer_forward(x, lens, layer, kc, vc)
+        assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), b
+    assert wq.device_status() == 0
