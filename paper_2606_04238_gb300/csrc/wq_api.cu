@@ -947,6 +947,7 @@ bool stack_kernel_plan(int m, const wq_mlp_layer *layers, int n_layers, unsigned
 //   d 4096 / inter 14336: m=1 33.0 vs 41.6, m=4 44.1 vs 61.5, m=8 68.8 vs 87.2;
 //   d 5120 / inter 17408: m=1 48.7 vs 52.6, m=4 80.1 vs 76.8, m=8 104.1 vs 132.9;
 //   4-bit gate/up, d 2560: m=1 20.9 vs 18.0, m=4 23.6 vs 22.5, m=8 28.0 vs 25.9.
+// Where the batched chain is faster than both (stack_takes_batch) it comes first.
 bool stack_preferred(int m, const wq_mlp_layer &L0) { return L0.gate.bits == 2 && (m >= 2 || L0.gate.k >= 4096); }
 
 StackRoute stack_route(int m, const wq_mlp_layer *layers, int n_layers, unsigned flags) {
@@ -1201,9 +1202,13 @@ size_t wq_attn_workspace_bytes(int batch, int n_heads, int n_kv, int head_dim, i
   return up256((size_t)batch * n_heads * S * (head_dim + 2) * 4);
 }
 
-wq_status wq_attn_decode(const float *qkv, const void *x, const int32_t *lens, int batch, int d, int n_heads, int n_kv,
-                         int head_dim, float theta, void *k_cache, void *v_cache, int max_len, void *o, void *ws,
-                         size_t ws_bytes, void *stream) {
+}  // extern "C"
+
+namespace {
+
+wq_status attn_decode_impl(const float *qkv, const void *x, const int32_t *lens, int batch, int d, int n_heads,
+                           int n_kv, int head_dim, float theta, void *k_cache, void *v_cache, int max_len, void *o,
+                           void *ws, size_t ws_bytes, bool early, void *stream) {
   if (batch < 0 || d <= 0 || d % 8 != 0) return fail(WQ_ERR_SHAPE, "batch %d, d %d (a positive multiple of 8)", batch, d);
   if (head_dim != 64 && head_dim != 128) return fail(WQ_ERR_UNSUPPORTED, "head_dim %d not 64 or 128", head_dim);
   if (n_kv <= 0 || n_heads <= 0 || n_heads % n_kv != 0 || n_heads / n_kv > 8)
@@ -1221,9 +1226,20 @@ wq_status wq_attn_decode(const float *qkv, const void *x, const int32_t *lens, i
   const int S = attn_splits(batch, n_kv, max_len, num_sms());
   cudaError_t e = launch_attn_decode(qkv, x, reinterpret_cast<const int *>(lens), batch, d, n_heads, n_kv, head_dim,
                                      (double)theta, k_cache, v_cache, max_len, static_cast<float *>(ws), S, o,
-                                     static_cast<cudaStream_t>(stream));
+                                     early, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "attention launch");
   return ok();
+}
+
+}  // namespace
+
+extern "C" {
+
+wq_status wq_attn_decode(const float *qkv, const void *x, const int32_t *lens, int batch, int d, int n_heads, int n_kv,
+                         int head_dim, float theta, void *k_cache, void *v_cache, int max_len, void *o, void *ws,
+                         size_t ws_bytes, void *stream) {
+  return attn_decode_impl(qkv, x, lens, batch, d, n_heads, n_kv, head_dim, theta, k_cache, v_cache, max_len, o, ws,
+                          ws_bytes, false, stream);
 }
 
 }  // extern "C"
@@ -1293,8 +1309,9 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
   uint8_t *w8 = static_cast<uint8_t *>(ws);
   if ((st = wq_down_w4(x, batch, &Ly.qkv, nullptr, w8 + W.qkv, WQ_F32, w8 + W.proj_qkv, W.n_qkv, stream)) != WQ_OK)
     return fail(st, "qkv projection: %s", g_last_error.c_str());
-  if ((st = wq_attn_decode(reinterpret_cast<const float *>(w8 + W.qkv), x, lens, batch, d, H, Hkv, hd, Ly.rope_theta,
-                           k_cache, v_cache, max_len, w8 + W.o, w8 + W.attn, W.n_attn, stream)) != WQ_OK)
+  // x, lens and the caches come from before the projection, whose launches wait first
+  if ((st = attn_decode_impl(reinterpret_cast<const float *>(w8 + W.qkv), x, lens, batch, d, H, Hkv, hd, Ly.rope_theta,
+                           k_cache, v_cache, max_len, w8 + W.o, w8 + W.attn, W.n_attn, true, stream)) != WQ_OK)
     return fail(st, "attention: %s", g_last_error.c_str());
   const wq_mlp_layer &M = Ly.mlp;
   // Decode sizes: the output projection's epilogue also writes the MLP
