@@ -1612,6 +1612,7 @@ wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe
   a.partials = reinterpret_cast<float *>(w8 + W.part_gu);
   a.counters = reinterpret_cast<unsigned *>(w8 + W.cnt_gu);
   a.slot_expert = idx;
+  a.slot_logits = logits;
   a.n_experts = E;
   a.slot_div = k;
   e = launch_gemv_slots(X.gate.bits == 4 ? kGateUpW4 : kGateUpW2, W.gu, a, S, s, true);

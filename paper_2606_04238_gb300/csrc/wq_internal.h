@@ -87,6 +87,8 @@ struct GemvArgs {
   // row s; tp, partials and counters hold one region per slot.
   const int *slot_expert;    // [slots], written by the routing kernel
   int n_experts, slot_div;
+  const float *slot_logits;  // not null: router logits [tokens][n_experts], complete before the previous launch let
+                             // this one start; slot s finds its expert itself (choice s % slot_div of token s / slot_div)
   int slot_expert_ready;     // the routing kernel completed before this launch can start (not the previous launch)
   // buffer sizes in bytes (checked by the debug build, WQ_DEBUG_CHECKS)
   size_t nb_codes[2], nb_meta[2], nb_lora_b[2], nb_act, nb_tp, nb_res, nb_out, nb_an, nb_tp_out, nb_part, nb_cnt;

@@ -13,7 +13,6 @@
 //      and one expert each) -> h per slot;
 //   3. the down dequant-GEMV over the slots -> y_j per slot in fp32;
 //   4. moe_combine_kernel: y[t] = bf16(x[t] + sum_j w_j y_j), j in order.
-#include <climits>
 #include <cstdint>
 
 #include <cuda_bf16.h>
@@ -21,12 +20,12 @@
 
 #include "wq_internal.h"
 #include "wq_ptx.cuh"
+#include "wq_route.cuh"
 
 namespace wq {
 
 namespace {
 
-constexpr int kMoeMaxExperts = 256;
 constexpr int kMoeMaxTopK = 16;
 constexpr int kPrepWarps = 8;  // tiles of 16 features a CTA of moe_prep_kernel takes
 
@@ -37,12 +36,6 @@ __device__ __forceinline__ void unpack8(const uint4 v, float (&f)[8]) {
     f[2 * i] = __uint_as_float(w[i] << 16);
     f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
   }
-}
-
-// (logit, expert) a ranks before (logit, expert) b: the larger logit first,
-// the lower expert index among equal logits.
-__device__ __forceinline__ bool ranks_before(float la, int ea, float lb, int eb) {
-  return la > lb || (la == lb && ea < eb);
 }
 
 // grid (ceil(ntp / 8), slots), 256 threads.  Every CTA routes its own token
@@ -56,40 +49,16 @@ __global__ void __launch_bounds__(kPrepWarps * 32) moe_prep_kernel(const __nv_bf
   __shared__ float w_s[kMoeMaxTopK];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slot = blockIdx.y, t = slot / top_k, j = slot % top_k;
+  // x and the logits may come from the previous launch.  The gate/up launch may
+  // start only now: it reads the logits without a wait of its own.
+  pdl_wait();
   pdl_launch_dependents();
-  pdl_wait();  // x and the logits may come from the previous launch
   if (warp == 0) {
-    // lane l holds experts l, l + 32, ..: taken ones are marked by clearing their bit
-    constexpr int PER = kMoeMaxExperts / 32;
-    float lg[PER];
-    uint32_t live = 0u;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = lane + 32 * i;
-      lg[i] = e < E ? __ldcg(logits + (size_t)t * E + e) : 0.f;
-      if (e < E) live |= 1u << i;
-    }
+    RouteKeys keys;
+    route_load(keys, logits + (size_t)t * E, E, lane);
     float sel_l[kMoeMaxTopK];
-    for (int c = 0; c < top_k; ++c) {
-      float bl = 0.f;
-      int be = INT_MAX;
-#pragma unroll
-      for (int i = 0; i < PER; ++i)
-        if (((live >> i) & 1u) && (be == INT_MAX || ranks_before(lg[i], lane + 32 * i, bl, be))) {
-          bl = lg[i];
-          be = lane + 32 * i;
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ol = __shfl_xor_sync(0xffffffffu, bl, o);
-        const int oe = __shfl_xor_sync(0xffffffffu, be, o);
-        if (oe != INT_MAX && (be == INT_MAX || ranks_before(ol, oe, bl, be))) {
-          bl = ol;
-          be = oe;
-        }
-      }
-      if (be != INT_MAX && (be & 31) == lane) live &= ~(1u << (be >> 5));
-      sel_l[c] = bl;  // top_k <= kMoeMaxTopK (checked by the launcher)
+    for (int c = 0; c < top_k; ++c) {  // top_k <= kMoeMaxTopK (checked by the launcher)
+      const int be = route_next(keys, lane, sel_l[c]);
       if (lane == 0) sel_s[c] = be;
     }
     if (lane == 0) {

@@ -194,3 +194,17 @@ def test_decoder_workspace_of_several_batches(wq):
         y0 = wq.decoder_layer_forward(x, lens, layer, kc, vc)
         assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), b
     assert wq.device_status() == 0
+
+
+@pytest.mark.parametrize("m,E,k", [(1, 256, 12), (3, 33, 4), (12, 2, 1)])
+def test_slots_find_their_experts(wq, m, E, k):
+    """At most 12 slots: the gate/up launch and the routing launch rank the experts
+    alike -- ties, signed zeros, negative and extreme logits."""
+    from tests.test_gpu_moe import _build, _check_block
+    d, inter, group = 64, 32, 32
+    layer, ents = _build(wq, d, inter, E, k, group, 8, 700 + E)
+    x = synth.activations((m, d), 17 + m)
+    lg = np.random.default_rng(40 + E).integers(-3, 2, (m, E)).astype(np.float32)  # many ties
+    lg[:, ::3] *= -0.0
+    lg[0, E // 2], lg[0, -1], lg[0, 0] = 3e38, 1e-40, -3e38
+    _check_block(wq, layer, ents, x, torch.from_numpy(lg), group, f"slots m={m} E={E} k={k}", 2.0)
