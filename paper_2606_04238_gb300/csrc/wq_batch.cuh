@@ -63,6 +63,12 @@ struct BatchCfg {
   static constexpr int NWARP = NT <= 3 ? 16 : 8;
   static constexpr int RG = NPROJ == 2 ? 8 : 4;
   static constexpr int WK = NWARP / RG;
+  // A group's scales and zero points applied two tokens an instruction: the
+  // loop is short of issue slots (67 % used beside the MMAs).  us a layer, one
+  // -> two tokens an instruction: d 4096 at 32 tokens 60.5 -> 57.4, with groups
+  // of 32 at 64 tokens 111 -> 105; only 4-bit codes in groups of 128 at 56
+  // tokens and more lose (d 4096 87.4 -> 89.3).
+  static constexpr bool PAIRED = !(BITS == 4 && GPB == 1 && NT == 8);
   static constexpr int REC = NT * (2048 + 32 + 32 * GPB);
   static constexpr int SLOT = 2 * (BPK + GPB * 64);  // two tiles of a unit
   static constexpr int TF = BITS == 4 ? 0 : 4096 * NT;  // LoRA-A products (rank 64)
@@ -364,10 +370,17 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
                 for (int tl = 0; tl < 2; ++tl) {
                   float *c = tot[tl][nt];
                   const float *q = acc[tl][nt];
-                  c[0] = fmaf(zl[tl], xs.x, fmaf(sl[tl] * sx.x, q[0], c[0]));
-                  c[1] = fmaf(zl[tl], xs.y, fmaf(sl[tl] * sx.y, q[1], c[1]));
-                  c[2] = fmaf(zh[tl], xs.x, fmaf(sh[tl] * sx.x, q[2], c[2]));
-                  c[3] = fmaf(zh[tl], xs.y, fmaf(sh[tl] * sx.y, q[3], c[3]));
+                  if (C::PAIRED) {  // the same operations and roundings
+                    fma_f32x2(c[0], c[1], mul_f32x2(sl[tl], sl[tl], sx.x, sx.y), q[0], q[1]);
+                    fma_f32x2(c[0], c[1], pack_f32x2(zl[tl], zl[tl]), xs.x, xs.y);
+                    fma_f32x2(c[2], c[3], mul_f32x2(sh[tl], sh[tl], sx.x, sx.y), q[2], q[3]);
+                    fma_f32x2(c[2], c[3], pack_f32x2(zh[tl], zh[tl]), xs.x, xs.y);
+                  } else {
+                    c[0] = fmaf(zl[tl], xs.x, fmaf(sl[tl] * sx.x, q[0], c[0]));
+                    c[1] = fmaf(zl[tl], xs.y, fmaf(sl[tl] * sx.y, q[1], c[1]));
+                    c[2] = fmaf(zh[tl], xs.x, fmaf(sh[tl] * sx.x, q[2], c[2]));
+                    c[3] = fmaf(zh[tl], xs.y, fmaf(sh[tl] * sx.y, q[3], c[3]));
+                  }
                 }
               }
             }

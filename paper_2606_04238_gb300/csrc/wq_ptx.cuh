@@ -127,6 +127,24 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Two fp32 operations an instruction, each rounded as its scalar form.
+__device__ __forceinline__ uint64_t pack_f32x2(float a, float b) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(float a0, float a1, float b0, float b1) {
+  uint64_t v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pack_f32x2(a0, a1)), "l"(pack_f32x2(b0, b1)));
+  return v;
+}
+// (c0, c1) += a * (b0, b1)
+__device__ __forceinline__ void fma_f32x2(float &c0, float &c1, uint64_t a, float b0, float b1) {
+  uint64_t v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(pack_f32x2(b0, b1)), "l"(pack_f32x2(c0, c1)));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(v));
+}
+
 // D = A * B + C on the tensor cores: m16n8k16, A row-major f16, B col-major
 // f16, fp32 accumulators.
 __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
