@@ -1485,7 +1485,8 @@ bool moe_ws(int m, const wq_moe_layer &L, unsigned flags, MoeWs *W) {
     W->rs = off;     off = up256(off + segs * W->nt * 32);
     W->tf = off;     off = up256(off + segs * batch_tfrag_bytes(W->nt, r));
     W->ys = off;     off = up256(off + (size_t)S * d * 4);
-    W->part = off;   off = up256(off + batch_scratch_floats(W->nt, 2, sms) * 4);
+    const int occ = batch_routed_occ(W->nt, segs * std::max(KBd, KBi), sms);
+    W->part = off;   off = up256(off + batch_scratch_floats(W->nt, 2, sms * occ) * 4);
     W->total = off;
     return true;
   }

@@ -331,12 +331,12 @@ cudaError_t launch_batch_routed(GemvKind kind, const BatchArgs &a, int max_segs,
   int sms = 0;
   cudaError_t e = batch_sms(&sms);
   if (e != cudaSuccess) return e;
-  const long long W = (long long)max_segs * ((a.N + kBatchRows - 1) / kBatchRows) * ((a.K + 127) / 128);
-  const int ctas = (int)std::max(1LL, std::min((long long)sms, W / 2));
+  const long long T = (long long)max_segs * ((a.N + kBatchRows - 1) / kBatchRows), W = T * ((a.K + 127) / 128);
+  const int occ = batch_routed_occ(nt, T, sms), ctas = (int)std::max(1LL, std::min((long long)sms * occ, W / 2));
   switch (kind) {
-    case kGateUpW2: return launch_batch_routed_gu2(a, nt, ctas, s);
-    case kGateUpW4: return launch_batch_routed_gu4(a, nt, ctas, s);
-    case kDownW4: return launch_batch_routed_dn4(a, nt, ctas, s);
+    case kGateUpW2: return launch_batch_routed_gu2(a, nt, ctas, occ, s);
+    case kGateUpW4: return launch_batch_routed_gu4(a, nt, ctas, occ, s);
+    case kDownW4: return launch_batch_routed_dn4(a, nt, ctas, occ, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -13,7 +13,7 @@
 // fragment of 256 weights costs 4 ANDs and is used for all tokens.
 //
 // Work split: row blocks of 128 rows x 128-feature blocks are the units;
-// gridDim.x CTAs (one an SM) take equal contiguous ranges of them (row block
+// gridDim.x CTAs (one an SM; OCC = 2 for some routed launches) take equal contiguous ranges of them (row block
 // major), so every SM has the same work for any shape.  A unit is computed by
 // RG warps of two row tiles each (gate/up: tile w of gate and tile w of up;
 // down: two neighbouring tiles), so each activation fragment is used twice;
@@ -53,14 +53,15 @@ constexpr int kBatchRows = 128;            // rows of a row block
 constexpr int kHsStride = kBatchRows + 8;  // halves a token of the staged h
 constexpr int kYsStride = kBatchRows + 4;  // floats a token of the staged y
 
-template <int BITS, int NPROJ, int GROUP, int NT>
+template <int BITS, int NPROJ, int GROUP, int NT, int OCC = 1>
 struct BatchCfg {
   static constexpr int BPK = BITS * 256;  // code bytes per (row tile, block)
   static constexpr int GPB = 128 / GROUP;
   // Few tokens leave a warp few independent MMAs (2 NT) between dependent
   // phases: 16 warps of at most 128 registers; the accumulators of more
   // tokens need 8 warps of up to 255.
-  static constexpr int NWARP = NT <= 3 ? 16 : 8;
+  static constexpr int NWARP = NT <= 3 && OCC == 1 ? 16 : 8;
+  static constexpr int MAXSMEM = OCC == 2 ? 115712 : 232448;
   static constexpr int RG = NPROJ == 2 ? 8 : 4;
   static constexpr int WK = NWARP / RG;
   // A group's scales and zero points applied two tokens an instruction: the
@@ -75,7 +76,7 @@ struct BatchCfg {
   static constexpr int STG_SUM = (WK - 1) * RG * 2 * NT * 512;
   static constexpr int STG_OUT = NPROJ == 2 ? NT * 8 * kHsStride * 2 : NT * 8 * kYsStride * 4;
   static constexpr int STG = std::max(STG_SUM, STG_OUT);
-  static constexpr int LIMIT = 232448 - 256 - NT * 32 - TF - STG;
+  static constexpr int LIMIT = MAXSMEM - 256 - NT * 32 - TF - STG;
   static constexpr int RXR = LIMIT - 4 * WK * REC >= 5 * NWARP * SLOT ? 4 : 3;  // rounds of WK records in the ring
   static constexpr int RX = RXR * WK, LEAD = RXR - 2;
   static constexpr int D = std::min(64 / NWARP, (LIMIT - RX * REC) / (NWARP * SLOT));
@@ -86,7 +87,7 @@ struct BatchCfg {
   static constexpr int OFF_STG = OFF_RS + NT * 32;
   static constexpr int OFF_BAR = OFF_STG + STG;
   static constexpr int SMEM = OFF_BAR + (2 * RX + 1) * 8 + 16;
-  static_assert(SMEM <= 232448, "batched-decode shared memory");
+  static_assert(SMEM <= MAXSMEM, "batched-decode shared memory");
   static constexpr int SLOT_F4 = RG * 2 * NT * 32;  // float4s of a part
 };
 
@@ -131,10 +132,10 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED>
-__global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 1)
+template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED, int OCC>
+__global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP * 32, OCC)
     batch_kernel(const __grid_constant__ BatchArgs a) {
-  using C = BatchCfg<BITS, NPROJ, GROUP, NT>;
+  using C = BatchCfg<BITS, NPROJ, GROUP, NT, OCC>;
   constexpr int BPK = C::BPK, GPB = C::GPB, WK = C::WK, RG = C::RG, D = C::D, RX = C::RX, GS = GROUP / 16;
   constexpr int NTHREADS = C::NWARP * 32;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -617,10 +618,10 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT>::NWARP * 32, 
   }
 }
 
-template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED = false>
+template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED = false, int OCC = 1>
 cudaError_t launch_batch_t(const BatchArgs &a, int ctas, cudaStream_t s) {
-  using C = BatchCfg<BITS, NPROJ, GROUP, NT>;
-  auto kern = batch_kernel<BITS, NPROJ, GROUP, NT, ROUTED>;
+  using C = BatchCfg<BITS, NPROJ, GROUP, NT, OCC>;
+  auto kern = batch_kernel<BITS, NPROJ, GROUP, NT, ROUTED, OCC>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -660,7 +661,12 @@ cudaError_t launch_batch_g(const BatchArgs &a, int nt, int ctas, cudaStream_t s)
 }
 
 template <int BITS, int NPROJ, int GROUP>
-cudaError_t launch_batch_routed_n(const BatchArgs &a, int nt, int ctas, cudaStream_t s) {
+cudaError_t launch_batch_routed_n(const BatchArgs &a, int nt, int ctas, int occ, cudaStream_t s) {
+  if (occ == 2) {
+    if (nt == 1) return launch_batch_t<BITS, NPROJ, GROUP, 1, true, 2>(a, ctas, s);
+    if (nt == 2) return launch_batch_t<BITS, NPROJ, GROUP, 2, true, 2>(a, ctas, s);
+    return cudaErrorInvalidValue;
+  }
   switch (nt) {
     case 1: return launch_batch_t<BITS, NPROJ, GROUP, 1, true>(a, ctas, s);
     case 2: return launch_batch_t<BITS, NPROJ, GROUP, 2, true>(a, ctas, s);
@@ -670,11 +676,11 @@ cudaError_t launch_batch_routed_n(const BatchArgs &a, int nt, int ctas, cudaStre
 }
 
 template <int BITS, int NPROJ>
-cudaError_t launch_batch_routed_g(const BatchArgs &a, int nt, int ctas, cudaStream_t s) {
+cudaError_t launch_batch_routed_g(const BatchArgs &a, int nt, int ctas, int occ, cudaStream_t s) {
   switch (a.group) {
-    case 32: return launch_batch_routed_n<BITS, NPROJ, 32>(a, nt, ctas, s);
-    case 64: return launch_batch_routed_n<BITS, NPROJ, 64>(a, nt, ctas, s);
-    case 128: return launch_batch_routed_n<BITS, NPROJ, 128>(a, nt, ctas, s);
+    case 32: return launch_batch_routed_n<BITS, NPROJ, 32>(a, nt, ctas, occ, s);
+    case 64: return launch_batch_routed_n<BITS, NPROJ, 64>(a, nt, ctas, occ, s);
+    case 128: return launch_batch_routed_n<BITS, NPROJ, 128>(a, nt, ctas, occ, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -45,6 +45,18 @@ inline int batch_max_segs(int slots, int experts, int nt) {
   return (slots < experts ? slots : experts) + slots / (8 * nt);
 }
 
+// CTAs an SM of a routed launch over `tiles` row blocks (of all segments at
+// most).  A CTA of many row blocks finishes several, each finish a latency chain
+// of one set of warps: with a second CTA of 8 warps the other computes
+// meanwhile; with few row blocks twice the CTAs mean twice the split ones.
+// Measured (us a block, one CTA vs two; row blocks an SM): 64 experts of 2048 x
+// 768, 2.8: 61.4 vs 56.9; GPT-OSS-20B shape, 2.7: 65.6 vs 66.7, 3.3: 73.0 vs 72.2,
+// 6: 123 vs 118.4; 8 experts of 4096 x 4096, 2.1: 68.1 vs 70.0, 2.9: 95.3 vs 94.8;
+// 8 experts of 2048 x 2048, 1.1: 36.6 vs 40.2.
+inline int batch_routed_occ(int nt, long long tiles, int num_sms) {
+  return nt <= 2 && 4 * tiles >= 11LL * num_sms ? 2 : 1;
+}
+
 struct BatchArgs {
   const uint8_t *panel;      // [ceil(K / 128)] records
   int M, N, K, group;
@@ -96,12 +108,12 @@ cudaError_t read_batch_status(int *status);
 
 // One translation unit per kind.
 cudaError_t launch_batch_gu2(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
-cudaError_t launch_batch_routed_gu2(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_gu2(const BatchArgs &a, int nt, int ctas, int occ, cudaStream_t s);
 cudaError_t launch_batch_gu3(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
 cudaError_t launch_batch_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
-cudaError_t launch_batch_routed_gu4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_gu4(const BatchArgs &a, int nt, int ctas, int occ, cudaStream_t s);
 cudaError_t launch_batch_dn4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
-cudaError_t launch_batch_routed_dn4(const BatchArgs &a, int nt, int ctas, cudaStream_t s);
+cudaError_t launch_batch_routed_dn4(const BatchArgs &a, int nt, int ctas, int occ, cudaStream_t s);
 cudaError_t read_batch_status_gu2(int *status);
 cudaError_t read_batch_status_gu3(int *status);
 cudaError_t read_batch_status_gu4(int *status);

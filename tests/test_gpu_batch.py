@@ -208,3 +208,36 @@ def test_slots_find_their_experts(wq, m, E, k):
     lg[:, ::3] *= -0.0
     lg[0, E // 2], lg[0, -1], lg[0, 0] = 3e38, 1e-40, -3e38
     _check_block(wq, layer, ents, x, torch.from_numpy(lg), group, f"slots m={m} E={E} k={k}", 2.0)
+
+
+@pytest.mark.parametrize("m,k", [(40, 3), (64, 6)])
+def test_routed_batch_of_two_ctas_an_sm(wq, m, k):
+    """Row blocks enough for two CTAs an SM (of 128 rows: 27 gate/up and 28 down ones an
+    expert), with one and two token tiles a segment; sampled slots."""
+    d, inter, E, group, r = 3488, 3424, 33, 32, 8
+    n = lambda rows, cols, bits, s: wq.pack(torch.randn((rows, cols), device="cuda",
+                                                        generator=torch.Generator("cuda").manual_seed(s)) * 0.02, group, bits)
+    _, bg, bu = synth.lora(d, E * inter, r, 5)
+    a_all = synth.weights((E * 2 * r, d), 6, std=0.01).to(torch.bfloat16)
+    g, u, dn = n(E * inter, d, 2, 1), n(E * inter, d, 2, 2), n(E * d, inter, 4, 3)
+    layer = wq.MoELayer(wq.MLPLayer(g, u, dn, lora_a=a_all.cuda(), lora_b_gate=bg.cuda(), lora_b_up=bu.cuda(),
+                                    lora_scale=2.0), E, k)
+    x = synth.activations((m, d), 8).cuda()
+    lg = torch.from_numpy(np.random.default_rng(9).standard_normal((m, E)).astype(np.float32)).cuda()
+    y, idx, wt, hs, ys = wq.moe_forward(x, lg, layer, with_slots=True)
+    # the slots one by one on the single-expert calls
+    sub = lambda q, e, rows: wq.QWeight(q.codes.view(E, -1)[e].contiguous(), q.meta.view(E, -1)[e].contiguous(),
+                                        rows, q.k, q.group, q.bits)
+    for s in range(0, m * k, 17):
+        e, t = int(idx.view(-1)[s]), s // k
+        h1 = wq.gateup_w2_lora(x[t:t + 1], sub(g, e, inter), sub(u, e, inter),
+                               a_all.cuda()[e * 2 * r:(e + 1) * 2 * r].contiguous(),
+                               bg.cuda()[e * inter:(e + 1) * inter].contiguous(),
+                               bu.cuda()[e * inter:(e + 1) * inter].contiguous(), lora_scale=2.0, prenorm=True)
+        y1 = wq.down_w4(hs[s:s + 1].contiguous(), sub(dn, e, d), out_f32=True)
+        # both are fp32 sums of exact products: one bf16 rounding apart at most, 1e-4 of the largest for fp32
+        dh = (hs[s].float() - h1[0].float()).abs()
+        assert (dh <= h1[0].float().abs() * 2.0 ** -7 + 1e-5).all() and (dh == 0).float().mean() > 0.97, s
+        assert ((ys[s] - y1[0]).abs() <= 1e-4 * y1.abs().max()).all(), s
+    torch.cuda.synchronize()
+    assert wq.device_status() == 0
