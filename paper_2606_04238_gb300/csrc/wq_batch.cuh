@@ -30,8 +30,8 @@
 //
 // Measured (GB300, us a layer of an MLP stack at W2 g128, the swapped-operand
 // tcgen05 launch or the GEMV chain before -> this): d 4096 / inter 14336 at 9,
-// 24, 64 tokens 102.7 -> 41.1, 104.1 -> 48.8, 110.8 -> 89.8; d 2560 / inter
-// 9728 35.3 -> 26.7, 62.7 -> 31.5, 75.7 -> 52.0.  At 24 tokens of the d 4096
+// 24, 64 tokens 102.7 -> 39.6, 104.1 -> 47.3, 110.8 -> 87.5; d 2560 / inter
+// 9728 35.3 -> 26.5, 62.7 -> 30.8, 75.7 -> 51.3.  At 24 tokens of the d 4096
 // shape a gate/up launch takes ~24 us, 15 of them in the main loop, which keeps
 // the mma.sync pipe (8 cycles an instruction) ~62 % busy; the rest is the
 // launch's start (~2 us), the exchange of split parts (~2 us) and the finish.
@@ -230,30 +230,29 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
   uint64_t *sfull = full + wk * RXR, *sempty = empty + wk * RXR;
   uint8_t *xring = smem + wk * RXR * C::REC;
   const int nset = (n - wk + WK - 1) / WK;  // units of this set (n >= wk or 0)
-  int rkb = kb0 + wk, rtile = tile0;        // block (and row block) of the next record
-  int rj = 0, rst = 0, rph = 1;             // its index, stage, and the parity its stage's `empty` was last completed with
+  // (The bookkeeping is the producing warp's alone, every RG rounds: done by
+  // every warp each round it took 3 % of a d 4096 layer at 24 tokens.)
   int issued = -1;                          // the last record this warp copied
-  auto produce = [&](int turn) {
-    if (rj < nset && turn == rg && elect_one()) {
-      while (rkb >= U) rkb -= U, ++rtile;
+  int rj = rg, rleft = rg - LEAD;           // the next record it copies, and the rounds until then
+  auto produce = [&]() {
+    if (rj < nset && elect_one()) {
+      const int at = kb0 + wk + rj * WK, rtile = tile0 + at / U, rkb = at % U;
       const uint8_t *panel = a.panel + (ROUTED ? (size_t)(rtile / RB) * U * C::REC : 0);
-      if (rj < RXR || wait(&sempty[rst], rph)) {
+      const int rst = rj % RXR;
+      if (rj < RXR || wait(&sempty[rst], (rj / RXR - 1) & 1)) {
         mbar_arrive_expect_tx(&sfull[rst], (uint32_t)C::REC);
         bulk_g2s(xring + rst * C::REC, panel + (size_t)rkb * C::REC, (uint32_t)C::REC, &sfull[rst]);
         issued = rj;
       }
     }
-    ++rj;
-    rkb += WK;
-    while (rkb >= U) rkb -= U, ++rtile;
-    if (++rst == RXR) rst = 0, rph ^= 1;
+    rj += RG;
+    rleft += RG;
   };
 #pragma unroll 1
   for (int j = 0; j < D; ++j) issue();
   pdl_wait();
   pdl_launch_dependents();
-#pragma unroll
-  for (int q = 0; q < LEAD; ++q) produce(q);
+  if (rg < LEAD) produce();
   if (NPROJ == 2 && !ROUTED && warp == LEAD && elect_one()) {
     const uint32_t tfb = BITS != 4 && a.tfrag != nullptr ? 2u * ((a.r + 15) / 16) * NT * 512u : 0u;
     const uint32_t rsb = a.rs != nullptr ? NT * 32u : 0u;
@@ -264,7 +263,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
   __syncwarp();
 
   float tot[2][NT][4];
-  int i = wk, cslot = 0, st = 0, ph = 0, turn = LEAD % RG;  // this warp's next unit, its code slot, record stage and phase
+  int i = wk, cslot = 0, st = 0, ph = 0;  // this warp's next unit, its code slot, record stage and phase
   for (int i0 = 0, tile = tile0, ub = kb0; i0 < n;) {
     const int len = min(U - ub, n - i0);
     if (NPROJ == 2 && a.tfrag != nullptr && wk == 0 && lane < a.r / 4) {
@@ -283,8 +282,10 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
 #pragma unroll
         for (int q = 0; q < 4; ++q) tot[tl][nt][q] = 0.f;
     for (; i < i0 + len; i += WK) {
-      produce(turn);
-      if (++turn == RG) turn = 0;
+      if (--rleft < 0) {
+        produce();
+        __syncwarp();
+      }
       cp_async_wait_group<D - 1>();
       __syncwarp();
       if (wait(&sfull[st], ph)) {
