@@ -444,10 +444,14 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnOcc) attn_split_kernel(
 }
 
 // o[b][h * HD + e] = bf16( sum_s O_s 2^(M_s - M) / sum_s L_s 2^(M_s - M) ).
-// grid B * H, 8 warps: warp w merges the splits w, w + 8, .. in order (its
-// own max first), lane l the features l * HD/32 ..; then the warps' results
-// are merged in warp order -- a fixed order, so the result is deterministic.
-template <int HD>
+// grid B * H, 8 warps: warp w merges the splits w, w + 8, .. in order, CU at a
+// time (their loads, rows of HD + 2 floats, in one round trip beside the
+// length's, then their max; a decoder layer of one sequence of 8192 positions,
+// 57 splits, 46.2 -> 43.7 us against a pass for the max first; CU 1 up to 8
+// splits, where the seven empty places cost 1 %), lane l the features l * HD/32
+// ..; then the warps' results are merged in warp order -- a fixed order, so the
+// result is deterministic.
+template <int HD, int CU>
 __global__ void __launch_bounds__(kCombWarps * 32) attn_combine_kernel(const float *part, const int *lens, int H, int S,
                                                                        int max_len, __nv_bfloat16 *o) {
   constexpr int E = HD / 32;
@@ -456,23 +460,42 @@ __global__ void __launch_bounds__(kCombWarps * 32) attn_combine_kernel(const flo
   pdl_wait();
   pdl_launch_dependents();
   const int pos = lens[bh / H];
-  if (pos < 0 || pos >= max_len) return;  // skipped by the split kernel
-  const float *pt = part + (size_t)bh * S * (HD + 2);
-  float M = -INFINITY;
-#pragma unroll 8
-  for (int s = warp; s < S; s += kCombWarps) M = fmaxf(M, pt[(size_t)s * (HD + 2) + HD]);
-  float L = 0.f, O[E];
+  const float *pt = part + (size_t)bh * S * (HD + 2) + lane * E;
+  float M = -INFINITY, L = 0.f, O[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) O[e] = 0.f;
-#pragma unroll 4
-  for (int s = warp; s < S; s += kCombWarps) {
-    const float *ps = pt + (size_t)s * (HD + 2);
-    const float ms = ps[HD];
-    const float f = ms == -INFINITY ? 0.f : exp2f(ms - M);
-    L = fmaf(ps[HD + 1], f, L);
+  for (int s0 = warp; s0 < S; s0 += CU * kCombWarps) {
+    float2 ml[CU], ov[CU][E / 2];
+    float mn = M;
 #pragma unroll
-    for (int e = 0; e < E; ++e) O[e] = fmaf(ps[lane * E + e], f, O[e]);
+    for (int u = 0; u < CU; ++u) {
+      const int s = s0 + u * kCombWarps;
+      const float *ps = pt + (size_t)s * (HD + 2);
+      ml[u] = s < S ? *reinterpret_cast<const float2 *>(ps + HD - lane * E) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int e = 0; e < E / 2; ++e)
+        ov[u][e] = s < S ? *reinterpret_cast<const float2 *>(ps + 2 * e) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < CU; ++u) mn = fmaxf(mn, ml[u].x);
+    const float f0 = M == -INFINITY ? 0.f : exp2f(M - mn);
+    M = mn;
+    L *= f0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) O[e] *= f0;
+#pragma unroll
+    for (int u = 0; u < CU; ++u) {
+      if (s0 + u * kCombWarps >= S) break;
+      const float f = ml[u].x == -INFINITY ? 0.f : exp2f(ml[u].x - M);
+      L = fmaf(ml[u].y, f, L);
+#pragma unroll
+      for (int e = 0; e < E / 2; ++e) {
+        O[2 * e] = fmaf(ov[u][e].x, f, O[2 * e]);
+        O[2 * e + 1] = fmaf(ov[u][e].y, f, O[2 * e + 1]);
+      }
+    }
   }
+  if (pos < 0 || pos >= max_len) return;  // skipped by the split kernel
   if (lane == 0) {
     wm[warp] = M;
     wl[warp] = L;
@@ -524,7 +547,8 @@ cudaError_t launch_attn_t(const float *qkv, const __nv_bfloat16 *x, const int *l
   cfg.gridDim = dim3(B * H);
   cfg.blockDim = dim3(kCombWarps * 32);
   cfg.dynamicSmemBytes = 0;
-  return cudaLaunchKernelEx(&cfg, attn_combine_kernel<HD>, (const float *)part, lens, H, S, max_len, o);
+  return cudaLaunchKernelEx(&cfg, S <= kCombWarps ? attn_combine_kernel<HD, 1> : attn_combine_kernel<HD, 8>,
+                            (const float *)part, lens, H, S, max_len, o);
 }
 
 }  // namespace
