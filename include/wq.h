@@ -382,7 +382,7 @@ typedef struct {
  *   expert_idx (int32 [m, top_k]), expert_w (fp32 [m, top_k]), h_slots
  *   (bf16 [m top_k, inter]) and y_slots (fp32 [m top_k, d]): optional device
  *   outputs of steps 1-2, slot t*top_k + j (NULL: kept in the workspace).
- * Up to 12 slots, four launches on `stream` (routing with the tile partials,
+ * Few slots (up to 12, more of small experts), four launches on `stream` (routing with the tile partials,
  * gate/up and down over the slots, combine); above, five (routing and grouping
  * of the slots by expert, the groups' inputs, gate/up and down over the groups,
  * combine).  Only the selected experts' weights are read.

@@ -124,18 +124,27 @@ int gemv_prefer_tokens(int d) { return d >= 4096 ? 8 : kGemvPreferTokens; }
 //     1 token 48.2 vs 41.4; d 2560 W4 5 tokens 22.7 vs 23.8, 6 tokens 24.6 vs
 //     23.9 (W3 g32 5 tokens 27.4 vs 27.4); at 9 tokens 35.3 vs 26.7, and above
 //     64 tokens each weight's expansion for tcgen05 is shared by 128 and more.
+//   Down matrices of few rows and less than 16M weights are split into many parts
+//   a row block: 1024 x 8192 at 9 / 16 tokens 10.9 / 12.7 vs 15.5 / 15.1, 2048 x
+//   6144 at 12 / 16 13.4 / 14.9 vs 16.6 / 16.8, 512 x 2048 at 12 / 16 8.8 / 10.9 vs
+//   9.8 / 9.8, but 2560 x 4096 at 9 13.6 vs 12.5; stacks of such layers: d 1024 /
+//   inter 8192 at 9 / 12 / 16 21.9 / 24.8 / 28.6 vs 26.4 / 26.5 / 26.0, d 512 / 2048
+//   15.9 / 15.8 / 19.3 vs 16.3 / 16.3 / 15.6, but d 256 / 768 at 9 13.8 vs 11.5, d
+//   2048 / 2048 at 9 20.4 vs 20.2.
 int gateup_batch_above(const wq_qweight &gate) {
   const long long w = 2LL * gate.n * gate.k;
   return w >= 100000000 ? 0 : w >= 30000000 ? 1 : 8;
 }
 int down_batch_above(const wq_qweight &down) {
   const long long w = (long long)down.n * down.k;
+  if (w < 16000000 && down.n < 2560) return down.k <= 2048 ? 12 : 16;
   return w >= 80000000 ? 0 : w >= 50000000 ? 2 : 8;
 }
 int layer_batch_above(const wq_mlp_layer &l) {
   const long long w = (long long)l.gate.n * l.gate.k;
   if (w >= 80000000) return 0;
   if (w >= 50000000) return l.gate.bits == 2 ? 1 : 0;
+  if (w >= 1000000 && w < 16000000 && l.gate.k < 1536) return 12;
   return w >= 20000000 && l.gate.bits != 2 ? 5 : 8;
 }
 // A stack takes them when every layer does.
@@ -962,7 +971,7 @@ StackRoute stack_route(int m, const wq_mlp_layer *layers, int n_layers, unsigned
   for (int l = 0; l < n_layers; ++l) {
     const wq_mlp_layer &Ly = layers[l];
     const bool next_tp = l + 1 < n_layers && ((flags & WQ_PRENORM) || layers[l + 1].r > 0);
-    if (m > 8) continue;  // the batched-decode launches take every shape
+    if (m > 8 && batch) continue;  // the batched-decode launches take every shape
     GemvPlan pl;
     if (!plan_gemv(gateup_kind(Ly.gate.bits), Ly.gate.n, Ly.gate.k, m, Ly.gate.group, Ly.r, num_sms(), &pl) ||
         (Ly.down.bits == 4 && !plan_gemv(kDownW4, Ly.down.n, Ly.down.k, m, Ly.down.group,
@@ -1056,7 +1065,7 @@ wq_status mlp_forward_impl(const void *x, int m, const wq_mlp_layer *layers, int
     }
     return ok();
   }
-  if (m <= kBatchMaxTokens && (m > 8 || route == kRouteGemmChain)) {
+  if (m <= kBatchMaxTokens && (route == kRouteGemmChain || (m > 8 && stack_takes_batch(m, layers, n_layers)))) {
     // batched-decode chain: per layer the panel of x with its RMSNorm scales
     // and LoRA-A products, gate/up (which leaves the panel of h), down
     const void *cur = x;
@@ -1177,7 +1186,7 @@ wq_status wq_mlp_forward_info(int m, const wq_mlp_layer *layers, int n_layers, u
   if (route == kRouteGemvChain) {
     const wq_mlp_layer &L0 = layers[0];
     const GemvKind kind = gateup_kind(L0.gate.bits);
-    if (m > 8) {  // the batched-decode launches have no GEMV plan; gate/up leaves the down launch's panel
+    if (m > 8 && stack_takes_batch(m, layers, n_layers)) {  // the batched-decode launches have no GEMV plan; gate/up leaves the down launch's panel
       info[13] = L0.down.bits == 4 ? 1 : 0;
       return ok();
     }
@@ -1328,7 +1337,7 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
     const int r_o = need_tp ? M.r : 0;
     const bool batched = gu_ok && stack_takes_batch(batch, &M, 1);
     GemvPlan pl;
-    const bool gemv = gu_ok && !batched && batch <= 8 && (r_o == 0 || d % 8 == 0) &&
+    const bool gemv = gu_ok && !batched && batch <= kGemvPreferTokens && (r_o == 0 || d % 8 == 0) &&
                       plan_gemv(kind, inter, d, batch, M.gate.group, M.r, num_sms(), &pl) &&
                       plan_gemv(kDownW4, d, inter, batch, M.down.group, 0, num_sms(), &pl) &&
                       plan_gemv(kDownW4, d, H * hd, batch, Ly.o.group, r_o, num_sms(), &pl);
@@ -1390,7 +1399,7 @@ namespace {
 // the split-K partials.  Each slot's launches are planned as one token on
 // its share of the SMs (all slots of a launch run side by side).
 //
-// More slots than kMoeBatchAbove are grouped by expert instead and run on the
+// Many slots (moe_grouped) are grouped by expert instead and run on the
 // batched-decode kernels: segments of up to 8 nt slots of one expert, whose
 // weights are then read once a segment, not once a slot.
 //
@@ -1404,12 +1413,24 @@ struct MoeWs {
   size_t route, panel, hpanel, rs, tf, part, cnt_bu, cnt_bd;
 };
 
-// Measured (GPT-OSS-20B shape, 32 experts top-4, us a block, slots vs grouped):
-// 8 slots 45.8 vs 48.4, 12 slots 60.8 vs 58.5, 16 slots 77 vs 69, 128 slots
-// 487 vs 128, 256 slots 942 vs 172; 8 experts top-2 of width 2048: 8 slots 25.5
-// vs 34.7, 16 slots 43 vs 37, 128 slots 247 vs 61.  Grouping costs one launch
-// more and the routing's single CTA.
-constexpr int kMoeBatchAbove = 12;
+// Grouping costs one launch more and the routing's single CTA, about 10 us; a slot
+// costs ~0.45 us for a million weights of an expert's matrix, a distinct expert
+// of the grouped launches ~0.4 (about 1.3 E S / (E + S) of E experts get one of S
+// slots).  Measured (us a block, slots vs grouped): GPT-OSS-20B shape (8.3M, 32
+// experts) 12 slots 60.8 vs 58.5, 16 slots 77 vs 69, 128 slots 487 vs 128; 8
+// experts of 2048 x 2048 14 slots 45.7 vs 36.1; 8 of 1024 x 1024 28 slots 27.0 vs
+// 28.7, 40 slots 36.5 vs 32.6; 16 of 2048 x 1024 16 slots 27.3 vs 34.9, 28 slots
+// 45.8 vs 36.5; 32 of 512 x 512 40 slots 22.1 vs 33.0.
+bool moe_grouped(int slots, int experts, int d, int inter) {
+  const double w = 1e-6 * d * inter;
+  return slots > 12 && w * slots * (0.45 - 0.52 * experts / (experts + slots)) > 11.0;
+}
+// The most slots a layer's slots path takes (the rule above is monotone in them).
+int moe_most_slots(int experts, int top_k, int d, int inter) {
+  int m = kMaxTokens;
+  while (m > 1 && moe_grouped(m * top_k, experts, d, inter)) --m;
+  return m * top_k;
+}
 
 // Token tiles a segment by the mean number of slots an expert gets: with most
 // experts' slots in one segment each weight is streamed once.
@@ -1455,11 +1476,11 @@ wq_status moe_check(int m, const wq_moe_layer *layer) {
   return WQ_OK;
 }
 
-// The counter block every MoE layout starts with (up to kMoeBatchAbove slots).
-size_t moe_slot_counters(int d, int inter, MoeWs *W) {
+// The counter block every MoE layout of a layer starts with.
+size_t moe_slot_counters(int most, int d, int inter, MoeWs *W) {
   size_t off = 0;
-  W->cnt_gu = off; off = up256(off + (size_t)kMoeBatchAbove * ((inter + 15) / 16) * 4);
-  W->cnt_dn = off; off = up256(off + (size_t)kMoeBatchAbove * ((d + 15) / 16) * 4);
+  W->cnt_gu = off; off = up256(off + (size_t)most * ((inter + 15) / 16) * 4);
+  W->cnt_dn = off; off = up256(off + (size_t)most * ((d + 15) / 16) * 4);
   return off;
 }
 
@@ -1468,13 +1489,14 @@ bool moe_ws(int m, const wq_moe_layer &L, unsigned flags, MoeWs *W) {
   const int E = L.n_experts, S = m * L.top_k, d = X.gate.k, inter = X.gate.n / E, r = X.r;
   const GemvKind kgu = X.gate.bits == 4 ? kGateUpW4 : kGateUpW2;
   *W = MoeWs{};
-  if (S > kMoeBatchAbove) {
+  const int most = moe_most_slots(E, L.top_k, d, inter);
+  if (moe_grouped(S, E, d, inter)) {
     const int sms = num_sms();
     if (sms <= 0) return false;
     W->nt = moe_batch_nt(S, E);
     W->max_segs = batch_max_segs(S, E, W->nt);
     const size_t segs = W->max_segs, KBd = (d + 127) / 128, KBi = (inter + 127) / 128;
-    size_t off = moe_slot_counters(d, inter, W);
+    size_t off = moe_slot_counters(most, d, inter, W);
     W->cnt_bu = off; off = up256(off + segs * KBi * 4);
     W->cnt_bd = off; off = up256(off + segs * KBd * 4);
     W->idx = off;    off = up256(off + (size_t)S * 4);
@@ -1493,7 +1515,7 @@ bool moe_ws(int m, const wq_moe_layer &L, unsigned flags, MoeWs *W) {
   if (!moe_plan(kgu, inter, d, X.gate.group, r, S, &W->gu) || !moe_plan(kDownW4, d, inter, X.down.group, 0, S, &W->dn))
     return false;
   const bool need_tp = (flags & WQ_PRENORM) || r > 0;
-  size_t off = moe_slot_counters(d, inter, W);
+  size_t off = moe_slot_counters(most, d, inter, W);
   W->idx = off;     off = up256(off + (size_t)S * 4);
   W->w = off;       off = up256(off + (size_t)S * 4);
   W->tp = off;      off = up256(off + (need_tp ? (size_t)S * (d / 16) * WQ_TP_STRIDE(r) * 4 : 0));

@@ -393,22 +393,14 @@ __device__ __forceinline__ void gemm_silu16(float *g, const float (&u)[16], floa
 // sectors) instead of 16 bytes of 32; the residual is read the same way.
 template <bool GATEUP>
 __device__ __forceinline__ void gemm_emit32(const GemmArgs &a, int mw, int nb, float (&v)[32], int lane) {
-  if ((a.N & 7) != 0 || (!GATEUP && a.out_f32)) {  // ragged rows, or fp32 output: a token a lane
+  const bool f32 = !GATEUP && a.out_f32;
+  const size_t row = (size_t)(mw + lane) * a.N + nb;
+  if ((a.N & 7) != 0) {  // ragged rows: a token a lane
     if (mw + lane >= a.M) return;
-    const size_t row = (size_t)(mw + lane) * a.N + nb;
-    const bool f32 = !GATEUP && a.out_f32;
     if (!GATEUP && a.residual) {
 #pragma unroll
       for (int e = 0; e < 32; ++e)
         if (nb + e < a.N) v[e] += __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(a.residual)[row + e]);
-    }
-    if (f32 && (a.N & 7) == 0) {
-#pragma unroll
-      for (int e = 0; e < 32; e += 4)
-        if (nb + e < a.N)
-          *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row + e) =
-              make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-      return;
     }
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
@@ -437,6 +429,15 @@ __device__ __forceinline__ void gemm_emit32(const GemmArgs &a, int mw, int nb, f
       for (int e = 0; e < 8; ++e)
         v[8 * i + e] += __uint_as_float(e & 1 ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16));
     }
+  }
+  if (f32) {  // 128 contiguous bytes a lane
+    if (mw + lane >= a.M) return;
+#pragma unroll
+    for (int e = 0; e < 32; e += 4)
+      if (nb + e < a.N)
+        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) + row + e) =
+            make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+    return;
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)

@@ -2,7 +2,7 @@
 // block (sm_103a).  Sec. 5 analyses an MoE model whose router activates a
 // few experts per token, so a decode step reads only those experts' weights.
 //
-// Up to a dozen slots a step is four launches joined by programmatic dependent
+// With few slots a step is four launches joined by programmatic dependent
 // launch (above, wq_batch.cu groups the slots by expert and only the combine
 // is used from here):
 //   1. moe_prep_kernel: per token, the top_k experts by router logit and

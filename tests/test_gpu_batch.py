@@ -69,7 +69,7 @@ def test_batch_gateup(wq, bits, d, inter, group, r, ms):
 
 DOWN = [
     # d, inter, group, token counts
-    (16, 128, 128, (9,)),
+    (16, 128, 128, (9, 13)),
     (202, 1056, 32, (12, 64)),        # rows no multiple of 4; ragged feature block
     (130, 20480, 128, (17, 63)),      # 2 row blocks, 160 blocks: about 76 parts each
     (2560, 704, 64, (32, 33)),
@@ -129,14 +129,14 @@ def test_batch_stack_hands_down_the_panel(wq, bits, group, group_down, r, m):
 
 
 @pytest.mark.parametrize("m,E,k,r,skew", [
-    (7, 8, 2, 8, 0.0),      # 14 slots, segments of up to 8
+    (30, 16, 2, 8, 0.0),    # 60 slots, segments of up to 8
     (33, 8, 2, 24, 0.0),    # 66 slots, segments of up to 16; rank 24
     (64, 4, 3, 0, 0.0),     # 192 slots, segments of up to 32
-    (24, 32, 1, 8, 9.0),    # every token takes expert 0: three segments, 31 experts unread
+    (64, 32, 1, 8, 9.0),    # every token takes expert 0: eight segments, 31 experts unread
 ])
 def test_routed_batch(wq, m, E, k, r, skew):
     from tests.test_gpu_moe import _build, _check_block
-    d, inter, group = 352, 224, 32  # ragged feature blocks and row blocks
+    d, inter, group = 1120, 992, 32  # ragged feature blocks and row blocks
     layer, ents = _build(wq, d, inter, E, k, group, r, 300 + m)
     x = synth.activations((m, d), 11 + m)
     lg = np.random.default_rng(5 + m).standard_normal((m, E)).astype(np.float32)
