@@ -1230,7 +1230,11 @@ cudaError_t num_sms_cached(int *sms) {
 // -> 103 us, d 5120 at 1500 228 -> 216), and for gate/up, whose parts are twice
 // as large, a main loop about a tenth slower (d 4096 at 700 tokens 159 -> 152
 // with it, at 512 tokens 110 -> 116, d 5120 at 3001 658 -> 695; d 2560 at 65
-// tokens, half the SMs without it, 39 -> 34).  One CTA per tile otherwise.
+// tokens, half the SMs without it, 39 -> 34).  Where gate/up tiles of 256 tokens
+// fill one wave at most, the parts of two halves weigh more (~15; at 160 tokens
+// without it -> with it d 2560 x inter 9728 39.1 -> 41.1, d 1600 x 4352 29.9 ->
+// 37.5, but d 4096 x 6144 54.9 -> 51.1, d 5120 x 2048 80 -> 52).  One CTA per
+// tile otherwise.
 struct GemmSched {
   int mt, T, U, P;
   bool sk;
@@ -1243,7 +1247,8 @@ GemmSched gemm_schedule(int M, int N, int K, int nproj, int r, int sms, int rows
   const long long W = (long long)g.T * g.U;
   const long long waves = (g.T + sms - 1) / sms, P = std::max(1LL, std::min((long long)sms, W / 4));
   const double share = (double)W / P;  // units a CTA
-  g.sk = W >= 8 && waves * g.U > (nproj == 2 ? 1.25 * share + 6 : share + 8);
+  const double cost = nproj == 2 ? std::max(14., 1.25 * share + (g.mt == 2 && waves == 1 ? 15 : 6)) : share + 8;
+  g.sk = W >= 8 && waves * g.U > cost;
   g.P = g.sk ? (int)P : g.T;
   return g;
 }
