@@ -129,7 +129,8 @@ int gemv_prefer_tokens(int d) { return d >= 4096 ? 8 : kGemvPreferTokens; }
 //   6144 at 12 / 16 13.4 / 14.9 vs 16.6 / 16.8, 512 x 2048 at 12 / 16 8.8 / 10.9 vs
 //   9.8 / 9.8, but 2560 x 4096 at 9 13.6 vs 12.5; stacks of such layers: d 1024 /
 //   inter 8192 at 9 / 12 / 16 21.9 / 24.8 / 28.6 vs 26.4 / 26.5 / 26.0, d 512 / 2048
-//   15.9 / 15.8 / 19.3 vs 16.3 / 16.3 / 15.6, but d 256 / 768 at 9 13.8 vs 11.5, d
+//   15.9 / 15.8 / 19.3 vs 16.3 / 16.3 / 15.6, d 2688 / 1344 W3 g32 at 12 21.5 vs 25.8,
+//   but d 256 / 768 at 9 13.8 vs 11.5, d
 //   2048 / 2048 at 9 20.4 vs 20.2.
 int gateup_batch_above(const wq_qweight &gate) {
   const long long w = 2LL * gate.n * gate.k;
@@ -144,7 +145,7 @@ int layer_batch_above(const wq_mlp_layer &l) {
   const long long w = (long long)l.gate.n * l.gate.k;
   if (w >= 80000000) return 0;
   if (w >= 50000000) return l.gate.bits == 2 ? 1 : 0;
-  if (w >= 1000000 && w < 16000000 && l.gate.k < 1536) return 12;
+  if (w >= 1000000 && (w < 6000000 || (w < 16000000 && l.gate.k < 1536))) return 12;
   return w >= 20000000 && l.gate.bits != 2 ? 5 : 8;
 }
 // A stack takes them when every layer does.
