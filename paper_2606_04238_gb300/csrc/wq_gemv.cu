@@ -584,9 +584,6 @@ __device__ __forceinline__ void qgemv_body(const GemvArgs &a, const GemvPlan &p)
         // per group: ctot += s * (sx * sum_k code * x' - z * sum_k x) for the
         // chains (c0, c1) of the group, the affine dequantization s (q - z)
         // with x' = x / sx (sx of the chain's half)
-        // (two tokens an instruction: a stack at one token, d 2560, groups of 32,
-        // 2- and 3-bit gate/up 20.9 -> 20.3 and 22.2 -> 21.5 us a layer, groups of
-        // 128 17.3 -> 17.2)
         auto group_epi = [&](const int gl, const int c0, const int c1) {
           float2 xs[NT];
 #pragma unroll
@@ -610,16 +607,22 @@ __device__ __forceinline__ void qgemv_body(const GemvArgs &a, const GemvPlan &p)
                 float *ct = ctot[pj][j][nt];
                 const float2 sa = scv[c0][nt];
                 const float *ga = acc[c0][pj][j][nt];
-                fma_f32x2(ct[0], ct[1], mul_f32x2(s_lo, s_lo, sa.x, sa.y), ga[0], ga[1]);
-                fma_f32x2(ct[2], ct[3], mul_f32x2(s_hi, s_hi, sa.x, sa.y), ga[2], ga[3]);
+                ct[0] = fmaf(s_lo * sa.x, ga[0], ct[0]);
+                ct[1] = fmaf(s_lo * sa.y, ga[1], ct[1]);
+                ct[2] = fmaf(s_hi * sa.x, ga[2], ct[2]);
+                ct[3] = fmaf(s_hi * sa.y, ga[3], ct[3]);
                 if (c1 != c0) {
                   const float2 sb = scv[c1][nt];
                   const float *gb = acc[c1][pj][j][nt];
-                  fma_f32x2(ct[0], ct[1], mul_f32x2(s_lo, s_lo, sb.x, sb.y), gb[0], gb[1]);
-                  fma_f32x2(ct[2], ct[3], mul_f32x2(s_hi, s_hi, sb.x, sb.y), gb[2], gb[3]);
+                  ct[0] = fmaf(s_lo * sb.x, gb[0], ct[0]);
+                  ct[1] = fmaf(s_lo * sb.y, gb[1], ct[1]);
+                  ct[2] = fmaf(s_hi * sb.x, gb[2], ct[2]);
+                  ct[3] = fmaf(s_hi * sb.y, gb[3], ct[3]);
                 }
-                fma_f32x2(ct[0], ct[1], pack_f32x2(zs_lo, zs_lo), xs[nt].x, xs[nt].y);
-                fma_f32x2(ct[2], ct[3], pack_f32x2(zs_hi, zs_hi), xs[nt].x, xs[nt].y);
+                ct[0] = fmaf(zs_lo, xs[nt].x, ct[0]);
+                ct[1] = fmaf(zs_lo, xs[nt].y, ct[1]);
+                ct[2] = fmaf(zs_hi, xs[nt].x, ct[2]);
+                ct[3] = fmaf(zs_hi, xs[nt].y, ct[3]);
               }
             }
         };
