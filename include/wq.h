@@ -22,8 +22,8 @@
  *   - Supported: group in {32, 64, 128}; in-features a multiple of the group
  *     (WQ_ERR_SHAPE otherwise); 1 <= m <= 16384 tokens (m == 0 is a no-op);
  *     LoRA rank r a multiple of 8, r <= 64 (r == 0: no adapter).
- *   - Three paths behind the same calls.  Up to 8 tokens the dequant-GEMV
- *     kernels; up to 64 tokens (for large matrices already from one to three
+ *   - Three paths behind the same calls.  Up to 8 tokens (12 or 16 for small
+ *     matrices) the dequant-GEMV kernels; up to 64 tokens (for large matrices already from one to three
  *     tokens on, and for a layer shape the GEMV kernels have no launch
  *     configuration for) the batched-decode kernels -- both form exact products
  *     of the codes and binary16 activations on the mma.sync tensor-core path
@@ -295,7 +295,8 @@ wq_status wq_down_bf16(const void *h, int m, const void *wd, int d, int inter, c
  *     input statistics) with programmatic dependent launch, each down launch
  *     also producing the next layer's RMSNorm and LoRA-A partial sums;
  *   - the batched chain above 16 tokens (8 for d >= 4096; fewer where a layer's
- *     matrices have 50M weights and more): the dequant-GEMM above 64 tokens.  From 9 to 64 tokens both chains run the batched-decode
+ *     matrices have 50M weights and more): the dequant-GEMM above 64 tokens.
+ *     From 9 (small layers 13) to 64 tokens both chains run the batched-decode
  *     kernels: per layer the activation panel of x with its RMSNorm scales and
  *     LoRA-A products, gate/up (which leaves the panel of h), down.
  * Every route can be captured into a CUDA graph.
@@ -382,8 +383,9 @@ typedef struct {
  *   expert_idx (int32 [m, top_k]), expert_w (fp32 [m, top_k]), h_slots
  *   (bf16 [m top_k, inter]) and y_slots (fp32 [m top_k, d]): optional device
  *   outputs of steps 1-2, slot t*top_k + j (NULL: kept in the workspace).
- * Few slots (up to 12, more of small experts), four launches on `stream` (routing with the tile partials,
- * gate/up and down over the slots, combine); above, five (routing and grouping
+ * Few slots (up to 12, more of small experts): four launches on `stream`
+ * (routing with the tile partials, gate/up and down over the slots, combine);
+ * above, five (routing and grouping
  * of the slots by expert, the groups' inputs, gate/up and down over the groups,
  * combine).  Only the selected experts' weights are read.
  * Workspace: wq_moe_workspace_bytes for this layer, token count and flags,
