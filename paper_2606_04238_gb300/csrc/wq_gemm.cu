@@ -485,10 +485,13 @@ __device__ __forceinline__ void gemm_emit_tmem(const GemmArgs &a, uint32_t taddr
 // one that it never waited for.  With two, the barrier's next phase belongs to
 // a use that cannot begin before this one, and its previous phase has completed
 // before the group's last stage.
+// acc_full is the MMAs' completion of a part, acc_empty the 16 dequantizing warps'
+// reads of its accumulators: the next part's first MMA, for whose B tile one
+// group of 8 suffices, starts them anew.
 template <class C>
 struct GemmSmem {
   uint8_t *base;
-  uint64_t *raw_full, *raw_empty, *a_full, *a_empty, *b_full, *b_empty, *acc_full;
+  uint64_t *raw_full, *raw_empty, *a_full, *a_empty, *b_full, *b_empty, *acc_full, *acc_empty;
   uint32_t *tmem_s;
   volatile int *abort_s;
   __device__ explicit GemmSmem(uint8_t *smem_raw) {
@@ -501,7 +504,8 @@ struct GemmSmem {
     b_full = a_empty + C::SA;
     b_empty = b_full + C::SB;
     acc_full = b_empty + 2 * C::SB;
-    tmem_s = reinterpret_cast<uint32_t *>(acc_full + 2);
+    acc_empty = acc_full + 1;
+    tmem_s = reinterpret_cast<uint32_t *>(acc_empty + 1);
     abort_s = reinterpret_cast<volatile int *>(tmem_s + 1);
   }
   // thread 0: barrier initialisation; the MMA warp: TMEM allocation
@@ -522,6 +526,7 @@ struct GemmSmem {
         mbar_init(&b_empty[2 * s + 1], 1);
       }
       mbar_init(acc_full, 1);
+      mbar_init(acc_empty, kDeqWarps);
       *abort_s = 0;
       fence_barrier_init();
     }
@@ -782,11 +787,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
     }
   } else if (warp == kMmaWarp) {
     if (elect_one()) {
-      int gs = 0;
+      int gs = 0, part = 0;
       bool ok = true;
       WQ_FOR_EACH_PART {
         if (!ok) break;
         const int mth = halves(tile_m0(tile));
+        // the previous part's accumulators are read
+        if (part > 0 && !wait(sm.acc_empty, (part - 1) & 1)) ok = false;
+        ++part;
+        if (!ok) break;
         for (int it = 0; it < nit; ++it, ++gs) {
           const int sa = gs % SA, sb = gs % SB;
           if (!wait(&sm.a_full[sa], (gs / SA) & 1) || !wait(&sm.b_full[sb], (gs / SB) & 1)) {
@@ -805,7 +814,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
     __syncwarp();
   } else {
     // dequantization, then each part's epilogue; a warp that met a timeout
-    // skips its work but still passes the epilogue's named barriers
+    // skips its work but still arrives for every part
     const int hb = warp / kDeqGroup, dt = tid & (kDeqGroup * 32 - 1);
     int gs = 0, gr = 0, part = 0;
     bool ok = true;
@@ -836,9 +845,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
       ++part;
       tc_fence_after();
       gemm_part_epilogue<BITS, NPROJ, GROUP, EXACT, TALL>(a, tmem, tile, ub, ue, U, g0, have);
-      // the next part's MMAs overwrite the accumulators only after this warp's
-      // b_full arrival, which follows its TMEM reads
+      // every lane's TMEM reads are done: the next part may overwrite them
       tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sm.acc_empty);
     }
   }
 #undef WQ_FOR_EACH_PART
