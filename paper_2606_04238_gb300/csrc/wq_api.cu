@@ -203,6 +203,17 @@ size_t counter_block(int d, int inter, WsLayout *L) {
   return off;
 }
 
+// The layout with its counter block (`block` bytes) at offset `counters` and the
+// rest of it from offset `body` on.
+WsLayout move_layout(WsLayout L, size_t block, size_t counters, size_t body) {
+  for (size_t *o : {&L.cnt1, &L.cnt2, &L.sctr, &L.bcnt}) *o += counters;
+  for (size_t *o : {&L.tp, &L.xa, &L.xb, &L.h, &L.hq, &L.hsc, &L.hxs, &L.part1, &L.part2, &L.x16, &L.rs, &L.ta, &L.h16,
+                    &L.hsx, &L.sk_part, &L.bpx, &L.bph, &L.brs, &L.btf, &L.bpart, &L.sxw, &L.stp, &L.shg, &L.spart,
+                    &L.sxc, &L.total})
+    *o += body - block;
+  return L;
+}
+
 // The dequant-GEMM buffers from offset `off`: binary16 copies of the GEMM
 // inputs, RMSNorm scales, the LoRA-A products and the stream-K scratch.
 bool gemm_layout(int m, int d, int inter, size_t off, WsLayout *L) {
@@ -621,6 +632,29 @@ wq_status check_gateup_pair(const wq_qweight *gate, const wq_qweight *up, int bi
   return WQ_OK;
 }
 
+// wq_down_w4 without its workspace: the arguments (m == 0 is ok), then the launches.
+wq_status check_down_args(const void *h, int m, const wq_qweight *down, const void *residual, const void *y, int y_dtype) {
+  wq_status st = check_tokens(m);
+  if (st != WQ_OK) return st;
+  if ((st = check_qweight(down, 4, "down")) != WQ_OK) return st;
+  if (y_dtype != WQ_BF16 && y_dtype != WQ_F32) return fail(WQ_ERR_ARG, "y_dtype %d not WQ_BF16 or WQ_F32", y_dtype);
+  if (m == 0) return ok();
+  if (!h || !y) return fail(WQ_ERR_ARG, "null h or y");
+  if (!aligned16(h) || !aligned16(y) || (residual && !aligned16(residual)))
+    return fail(WQ_ERR_ALIGN, "h, y or residual not 16-byte aligned");
+  return ok();
+}
+wq_status run_down_any(const void *h, int m, const wq_qweight *down, const void *residual, void *y, int y_dtype,
+                       const WsLayout &L, uint8_t *ws, cudaStream_t s) {
+  wq_status st = WQ_OK;
+  switch (down_path(m, down, 0)) {
+    case Path::kGemm: st = run_down_gemm(h, m, down, residual, y, y_dtype == WQ_F32, L, ws, s); break;
+    case Path::kBatch: st = run_down_batch(h, m, down, residual, y, y_dtype == WQ_F32, L, ws, s); break;
+    case Path::kGemv: st = run_down(h, m, down, residual, y, y_dtype == WQ_F32, nullptr, 0, nullptr, L, ws, s); break;
+  }
+  return st == WQ_OK ? ok() : st;
+}
+
 wq_status gateup_entry(GemvKind kind, const void *x, int m, const wq_qweight *gate, const wq_qweight *up,
                        const void *lora_a, const void *bg, const void *bu, int r, float lora_scale, unsigned flags,
                        void *h, void *ws, size_t ws_bytes, void *stream) {
@@ -838,24 +872,11 @@ wq_status wq_gateup_w4(const void *x, int m, const wq_qweight *gate, const wq_qw
 
 wq_status wq_down_w4(const void *h, int m, const wq_qweight *down, const void *residual, void *y, int y_dtype, void *ws,
                      size_t ws_bytes, void *stream) {
-  wq_status st = check_tokens(m);
-  if (st != WQ_OK) return st;
-  if ((st = check_qweight(down, 4, "down")) != WQ_OK) return st;
-  if (y_dtype != WQ_BF16 && y_dtype != WQ_F32) return fail(WQ_ERR_ARG, "y_dtype %d not WQ_BF16 or WQ_F32", y_dtype);
-  if (m == 0) return ok();
-  if (!h || !y) return fail(WQ_ERR_ARG, "null h or y");
-  if (!aligned16(h) || !aligned16(y) || (residual && !aligned16(residual)))
-    return fail(WQ_ERR_ALIGN, "h, y or residual not 16-byte aligned");
+  wq_status st = check_down_args(h, m, down, residual, y, y_dtype);
+  if (st != WQ_OK || m == 0) return st;
   WsLayout L;
   if ((st = check_ws(ws, ws_bytes, m, down->n, down->k, &L)) != WQ_OK) return st;
-  uint8_t *w8 = static_cast<uint8_t *>(ws);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  switch (down_path(m, down, 0)) {
-    case Path::kGemm: st = run_down_gemm(h, m, down, residual, y, y_dtype == WQ_F32, L, w8, s); break;
-    case Path::kBatch: st = run_down_batch(h, m, down, residual, y, y_dtype == WQ_F32, L, w8, s); break;
-    case Path::kGemv: st = run_down(h, m, down, residual, y, y_dtype == WQ_F32, nullptr, 0, nullptr, L, w8, s); break;
-  }
-  return st == WQ_OK ? ok() : st;
+  return run_down_any(h, m, down, residual, y, y_dtype, L, static_cast<uint8_t *>(ws), static_cast<cudaStream_t>(stream));
 }
 
 wq_status wq_down_bf16(const void *h, int m, const void *wd, int d, int inter, const void *residual, void *y,
@@ -1256,12 +1277,16 @@ wq_status wq_attn_decode(const float *qkv, const void *x, const int32_t *lens, i
 
 namespace {
 
-// Regions of a decoder layer's workspace: the MLP's, the two projections'
-// (each with its own arrival counters), the attention partials, then the
-// intermediates qkv (fp32), o, x1 and h (bf16).
+// Regions of a decoder layer's workspace: the two projections' arrival
+// counters and the MLP's region, which starts with its own, so that every
+// counter lies at the same offset for all batch sizes (zero once, left at zero
+// by every call) and one workspace serves them all; then the rest of the
+// projections', the attention partials and the intermediates qkv (fp32), o, x1
+// and h (bf16).
 struct DecoderWs {
-  size_t mlp, proj_qkv, proj_o, attn, qkv, o, x1, h, total;
-  size_t n_mlp, n_qkv, n_o, n_attn;
+  size_t cnt_qkv, cnt_o, mlp, proj_qkv, proj_o, attn, qkv, o, x1, h, total;
+  size_t b_qkv, b_o;  // sizes of the projections' counter blocks
+  size_t n_mlp, n_attn;
 };
 
 bool decoder_ws(int batch, const wq_decoder_layer &Ly, int max_len, DecoderWs *W) {
@@ -1269,14 +1294,18 @@ bool decoder_ws(int batch, const wq_decoder_layer &Ly, int max_len, DecoderWs *W
   const int H = Ly.n_heads, Hkv = Ly.n_kv, hd = Ly.head_dim;
   const int nqkv = (H + 2 * Hkv) * hd;
   W->n_mlp = wq_workspace_bytes(batch, d, inter, Ly.mlp.r);
-  W->n_qkv = wq_workspace_bytes(batch, nqkv, d, 0);
-  W->n_o = wq_workspace_bytes(batch, d, H * hd, 0);
+  const size_t n_qkv = wq_workspace_bytes(batch, nqkv, d, 0), n_o = wq_workspace_bytes(batch, d, H * hd, 0);
   W->n_attn = wq_attn_workspace_bytes(batch, H, Hkv, hd, max_len);
-  if (!W->n_mlp || !W->n_qkv || !W->n_o || !W->n_attn) return false;
+  if (!W->n_mlp || !n_qkv || !n_o || !W->n_attn) return false;
+  WsLayout L;
+  W->b_qkv = counter_block(nqkv, d, &L);
+  W->b_o = counter_block(d, H * hd, &L);
   size_t off = 0;
+  W->cnt_qkv = off;  off = up256(off + W->b_qkv);
+  W->cnt_o = off;    off = up256(off + W->b_o);
   W->mlp = off;      off = up256(off + W->n_mlp);
-  W->proj_qkv = off; off = up256(off + W->n_qkv);
-  W->proj_o = off;   off = up256(off + W->n_o);
+  W->proj_qkv = off; off = up256(off + n_qkv - W->b_qkv);
+  W->proj_o = off;   off = up256(off + n_o - W->b_o);
   W->attn = off;     off = up256(off + W->n_attn);
   W->qkv = off;      off = up256(off + (size_t)batch * nqkv * 4);
   W->o = off;        off = up256(off + (size_t)batch * H * hd * 2);
@@ -1284,6 +1313,17 @@ bool decoder_ws(int batch, const wq_decoder_layer &Ly, int max_len, DecoderWs *W
   W->h = off;        off = up256(off + (size_t)batch * inter * 2);
   W->total = off;
   return true;
+}
+
+// A projection of a decoder layer, its layout relative to the layer's workspace.
+wq_status decoder_projection(const char *name, const void *h, int m, const wq_qweight *q, const void *residual, void *y,
+                             int y_dtype, size_t block, size_t counters, size_t body, uint8_t *ws, cudaStream_t s) {
+  wq_status st = check_down_args(h, m, q, residual, y, y_dtype);
+  if (st == WQ_OK && !aligned16(ws)) st = fail(WQ_ERR_ALIGN, "workspace not 16-byte aligned");
+  WsLayout L;
+  if (st == WQ_OK && !ws_layout(m, q->n, q->k, &L)) st = fail(WQ_ERR_CUDA, "cannot query the current device");
+  if (st == WQ_OK) st = run_down_any(h, m, q, residual, y, y_dtype, move_layout(L, block, counters, body), ws, s);
+  return st == WQ_OK ? st : fail(st, "%s projection: %s", name, g_last_error.c_str());
 }
 
 }  // namespace
@@ -1317,8 +1357,10 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
   if (!ws || ws_bytes < W.total)
     return fail(WQ_ERR_WORKSPACE, "decoder workspace of %zu bytes, %zu needed", ws_bytes, W.total);
   uint8_t *w8 = static_cast<uint8_t *>(ws);
-  if ((st = wq_down_w4(x, batch, &Ly.qkv, nullptr, w8 + W.qkv, WQ_F32, w8 + W.proj_qkv, W.n_qkv, stream)) != WQ_OK)
-    return fail(st, "qkv projection: %s", g_last_error.c_str());
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if ((st = decoder_projection("qkv", x, batch, &Ly.qkv, nullptr, w8 + W.qkv, WQ_F32, W.b_qkv, W.cnt_qkv, W.proj_qkv, w8,
+                               s)) != WQ_OK)
+    return st;
   // x, lens and the caches come from before the projection, whose launches wait first
   if ((st = attn_decode_impl(reinterpret_cast<const float *>(w8 + W.qkv), x, lens, batch, d, H, Hkv, hd, Ly.rope_theta,
                            k_cache, v_cache, max_len, w8 + W.o, w8 + W.attn, W.n_attn, true, stream)) != WQ_OK)
@@ -1346,12 +1388,11 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
       if (!y) return fail(WQ_ERR_ARG, "null y");
       if (!aligned16(y)) return fail(WQ_ERR_ALIGN, "y not 16-byte aligned");
       WsLayout Lm, Lo;
-      if ((st = check_ws(w8 + W.mlp, W.n_mlp, batch, d, inter, &Lm)) != WQ_OK ||
-          (st = check_ws(w8 + W.proj_o, W.n_o, batch, d, H * hd, &Lo)) != WQ_OK)
-        return st;
-      cudaStream_t s = static_cast<cudaStream_t>(stream);
+      if ((st = check_ws(w8 + W.mlp, W.n_mlp, batch, d, inter, &Lm)) != WQ_OK) return st;
+      if (!ws_layout(batch, d, H * hd, &Lo)) return fail(WQ_ERR_CUDA, "cannot query the current device");
+      Lo = move_layout(Lo, W.b_o, W.cnt_o, W.proj_o);
       if (batched) {
-        if ((st = run_down_batch(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, 0, Lo, w8 + W.proj_o, s)) != WQ_OK)
+        if ((st = run_down_batch(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, 0, Lo, w8, s)) != WQ_OK)
           return fail(st, "output projection: %s", g_last_error.c_str());
         if ((st = run_gateup_batch(kind, w8 + W.x1, batch, &M.gate, &M.up, M.lora_a, M.lora_b_gate, M.lora_b_up, M.r,
                                    M.lora_scale, flags, nullptr, &M.down, Lm, w8 + W.mlp, s)) != WQ_OK)
@@ -1362,7 +1403,7 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
       }
       float *tp = need_tp ? reinterpret_cast<float *>(w8 + W.mlp + Lm.tp) : nullptr;
       if ((st = run_down(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, 0, need_tp ? M.lora_a : nullptr, r_o, tp, Lo,
-                         w8 + W.proj_o, s)) != WQ_OK)
+                         w8, s)) != WQ_OK)
         return fail(st, "output projection: %s", g_last_error.c_str());
       const bool panel = chain_panel_ok(kind, batch, M.gate, M.r, M.down, 0);
       if ((st = run_gateup(kind, w8 + W.x1, batch, &M.gate, &M.up, M.lora_a, M.lora_b_gate, M.lora_b_up, M.r,
@@ -1374,8 +1415,9 @@ wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens
       return ok();
     }
   }
-  if ((st = wq_down_w4(w8 + W.o, batch, &Ly.o, x, w8 + W.x1, WQ_BF16, w8 + W.proj_o, W.n_o, stream)) != WQ_OK)
-    return fail(st, "output projection: %s", g_last_error.c_str());
+  if ((st = decoder_projection("output", w8 + W.o, batch, &Ly.o, x, w8 + W.x1, WQ_BF16, W.b_o, W.cnt_o, W.proj_o, w8, s)) !=
+      WQ_OK)
+    return st;
   if (M.gate.bits == 3)
     st = wq_gateup_w3_lora(w8 + W.x1, batch, &M.gate, &M.up, M.lora_a, M.lora_b_gate, M.lora_b_up, M.r, M.lora_scale,
                            flags, w8 + W.h, w8 + W.mlp, W.n_mlp, stream);

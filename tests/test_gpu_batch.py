@@ -180,7 +180,7 @@ def test_moe_workspace_of_several_token_counts(wq):
 
 
 def test_decoder_workspace_of_several_batches(wq):
-    """The projections' counters lie elsewhere in a decoder workspace for every batch."""
+    """One workspace for the largest batch serves smaller ones in between."""
     d, inter, H, kv, hd, max_len = 512, 896, 4, 2, 128, 64
     mk = lambda n, kk, bits, s: upload_packed(*_q((n, kk), 64, bits, s), 64, bits)
     layer = wq.DecoderLayer(mk((H + 2 * kv) * hd, d, 4, 1), mk(d, H * hd, 4, 2),
@@ -190,6 +190,33 @@ def test_decoder_workspace_of_several_batches(wq):
         x = synth.activations((b, d), 80 + i).cuda()
         lens = torch.full((b,), 10 + i, dtype=torch.int32, device="cuda")
         kc, vc = (synth.activations((b, kv, max_len, hd), 90 + j).cuda() for j in range(2))
+        y = wq.decoder_layer_forward(x, lens, layer, kc, vc, ws=ws).clone()
+        y0 = wq.decoder_layer_forward(x, lens, layer, kc, vc)
+        assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), b
+    assert wq.device_status() == 0
+
+
+@pytest.mark.parametrize("d,inter,H,group,big,split", [
+    (5120, 17408, 40, 32, 25, (8, 7)),  # q/k/v and output projection of a batch of 8 and 7
+    (1024, 8192, 40, 64, 17, (12, 11)),  # output projection of a batch of 12 and 11
+])
+def test_decoder_workspace_of_several_batches_with_split_projections(wq, d, inter, H, group, big, split):
+    """The same where a GEMV launch of the projections splits its rows over feature
+    panels, whose arrival counters have to be zero when it starts: a larger batch
+    fills the workspace's buffers before."""
+    kv, hd, max_len = 8, 128, 64
+    nqkv = (H + 2 * kv) * hd
+    for b in split:
+        assert wq.plan_info(wq.KIND_DOWN_W4, d, H * hd, b, group)["panels"] > 1
+    gen = torch.Generator("cuda").manual_seed(5)
+    mk = lambda n, kk, bits: wq.pack(torch.randn((n, kk), device="cuda", generator=gen) * 0.02, group, bits)
+    layer = wq.DecoderLayer(mk(nqkv, d, 4), mk(d, H * hd, 4),
+                            wq.MLPLayer(mk(inter, d, 2), mk(inter, d, 2), mk(d, inter, 4)), H, kv, hd, 1e6)
+    ws = wq.decoder_workspace(big, layer, max_len)
+    for i, b in enumerate((big, split[0], big, split[1])):
+        x = synth.activations((b, d), 180 + i).cuda()
+        lens = torch.full((b,), 10 + i, dtype=torch.int32, device="cuda")
+        kc, vc = (synth.activations((b, kv, max_len, hd), 190 + j).cuda() for j in range(2))
         y = wq.decoder_layer_forward(x, lens, layer, kc, vc, ws=ws).clone()
         y0 = wq.decoder_layer_forward(x, lens, layer, kc, vc)
         assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), b
