@@ -18,7 +18,7 @@ __device__ __forceinline__ uint32_t word4(const uint4 &v, int q) { return q == 0
 
 // CTAs 0 .. nt * row_tiles - 1 (row_tiles > 0): 8 tokens x 16 rows of A_cat
 // over all features: t = lora_scale * x A^T on bf16 mma.sync (exact products,
-// fp32 sums), stored as two bf16 parts in the gate/up launch's fragment order;
+// fp32 sums), stored as three bf16 parts in the gate/up launch's fragment order;
 // row tile 0 also the tokens' RMSNorm scales.  The 16 warps take interleaved
 // chunks of 32 features and their sums are added in warp order.  A lane loads
 // 8 consecutive features of a row and feeds them to two k-steps in the same
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __nv_bfl
   if (ROUTED) {
     if (seg >= __ldcg(&route->n_segs)) return;
     sg = __ldcg(&route->seg[seg]);
-    if (r2 > 0) lora_a += (size_t)sg.x * r2 * K, tfrag += (size_t)seg * 2 * ((r + 15) / 16) * nt_total * 512;
+    if (r2 > 0) lora_a += (size_t)sg.x * r2 * K, tfrag += (size_t)seg * 2 * ((r + 15) / 16) * nt_total * kTfragBytes;
     if (rs != nullptr) rs += seg * nt_total * 8;
   }
   const int row = xrow(sg, nt * 8 + g);
@@ -136,19 +136,24 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __nv_bfl
     if (j < r2) {
       v *= lora_scale;
       const int p = j >= r ? 1 : 0, rho = j - p * r, RK = (r + 15) / 16, c = rho & 15;
-      const size_t at = ((((size_t)p * RK + (rho >> 4)) * nt_total + nt) * 32 + 4 * ml + ((c & 7) >> 1)) * 16 +
-                        (c >> 3) * 4 + (c & 1) * 2;
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v), lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-      *reinterpret_cast<__nv_bfloat16 *>(tfrag + at) = hi;
-      *reinterpret_cast<__nv_bfloat16 *>(tfrag + at + 8) = lo;
+      uint8_t *frag = tfrag + (((size_t)p * RK + (rho >> 4)) * nt_total + nt) * kTfragBytes;
+      const int ln = 4 * ml + ((c & 7) >> 1), e = (c >> 3) * 4 + (c & 1) * 2;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+      const float rest = v - __bfloat162float(hi);
+      const __nv_bfloat16 mid = __float2bfloat16_rn(rest);
+      *reinterpret_cast<__nv_bfloat16 *>(frag + ln * 16 + e) = hi;
+      *reinterpret_cast<__nv_bfloat16 *>(frag + ln * 16 + 8 + e) = mid;
+      *reinterpret_cast<__nv_bfloat16 *>(frag + 512 + ln * 8 + e) = __float2bfloat16_rn(rest - __bfloat162float(mid));
     }
   }
   // ranks r .. 16 RK - 1 multiply zero rows of B: zeros, not leftovers
   if (jt == 0 && r2 > 0 && (r & 15) != 0 && tid >= 128 && tid < 256) {
     const int i = tid - 128, p = i >> 6, c = 8 + ((i >> 3) & 7), ml = i & 7, RK = (r + 15) / 16;
-    const size_t at = ((((size_t)p * RK + RK - 1) * nt_total + nt) * 32 + 4 * ml + ((c & 7) >> 1)) * 16 + 4 + (c & 1) * 2;
-    *reinterpret_cast<uint16_t *>(tfrag + at) = 0;
-    *reinterpret_cast<uint16_t *>(tfrag + at + 8) = 0;
+    uint8_t *frag = tfrag + (((size_t)p * RK + RK - 1) * nt_total + nt) * kTfragBytes;
+    const int ln = 4 * ml + ((c & 7) >> 1), e = 4 + (c & 1) * 2;
+    *reinterpret_cast<uint16_t *>(frag + ln * 16 + e) = 0;
+    *reinterpret_cast<uint16_t *>(frag + ln * 16 + 8 + e) = 0;
+    *reinterpret_cast<uint16_t *>(frag + 512 + ln * 8 + e) = 0;
   }
   if (jt == 0 && rs != nullptr && tid >= 256 && tid < 264) {
     const int ml = tid - 256;
@@ -367,7 +372,7 @@ size_t batch_scratch_floats(int nt, int nproj, int num_sms) {
   return (size_t)num_sms * 2 * (nproj == 2 ? 8 : 4) * 2 * nt * 32 * 4;
 }
 
-size_t batch_tfrag_bytes(int nt, int r) { return (size_t)2 * ((r + 15) / 16) * nt * 512; }
+size_t batch_tfrag_bytes(int nt, int r) { return (size_t)2 * ((r + 15) / 16) * nt * kTfragBytes; }
 
 cudaError_t read_batch_status(int *status) {
   cudaError_t (*const read[4])(int *) = {read_batch_status_gu2, read_batch_status_gu3, read_batch_status_gu4,

@@ -72,7 +72,7 @@ struct BatchCfg {
   static constexpr bool PAIRED = !(BITS == 4 && GPB == 1 && NT == 8);
   static constexpr int REC = NT * (2048 + 32 + 32 * GPB);
   static constexpr int SLOT = 2 * (BPK + GPB * 64);  // two tiles of a unit
-  static constexpr int TF = BITS == 4 ? 0 : 4096 * NT;  // LoRA-A products (rank 64)
+  static constexpr int TF = BITS == 4 || OCC == 2 ? 0 : 8 * NT * (int)kTfragBytes;  // LoRA-A products (rank 64; routed: from L2)
   static constexpr int STG_SUM = (WK - 1) * RG * 2 * NT * 512;
   static constexpr int STG_OUT = NPROJ == 2 ? NT * 8 * kHsStride * 2 : NT * 8 * kYsStride * 4;
   static constexpr int STG = std::max(STG_SUM, STG_OUT);
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
   pdl_launch_dependents();
   if (rg < LEAD) produce();
   if (NPROJ == 2 && !ROUTED && warp == LEAD && elect_one()) {
-    const uint32_t tfb = BITS != 4 && a.tfrag != nullptr ? 2u * ((a.r + 15) / 16) * NT * 512u : 0u;
+    const uint32_t tfb = BITS != 4 && a.tfrag != nullptr ? 2u * ((a.r + 15) / 16) * NT * kTfragBytes : 0u;
     const uint32_t rsb = a.rs != nullptr ? NT * 32u : 0u;
     mbar_arrive_expect_tx(aux, tfb + rsb);
     if (tfb) bulk_g2s(smem + C::OFF_TF, a.tfrag, tfb, aux);
@@ -480,41 +480,88 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
     auto orow = [&](int m) -> size_t { return ROUTED ? (size_t)__ldcg(&a.route->list[sg.z + m]) : (size_t)m; };
     if (NPROJ == 2) {
       if (!ROUTED) wait(aux, 0);
-      // Eq. 1's unmerged adapter: tot += B t, t as two bf16 parts
+      // Eq. 1's unmerged adapter: tot += B t, t as three bf16 parts (all 24 bits),
+      // the smallest first, summed on their own before they join the total
       if (BITS != 4 && a.tfrag != nullptr) {
         const int RK = (a.r + 15) / 16;
-        auto load_b = [&](int kk, uint32_t (&bf)[2][4]) {
+        auto load_b = [&](int p, int kk, uint32_t (&bf)[4]) {
 #pragma unroll
-          for (int p = 0; p < 2; ++p)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int row = n0 + rg * 16 + g + 8 * (q & 1), col = kk * 16 + 2 * t + 8 * (q >> 1);
-              const size_t at = (ROUTED ? (size_t)sg.x * a.N + row : (size_t)row) * a.r + col;
-              bf[p][q] = row < a.N && col < a.r
-                             ? __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(a.lora_b[p]) + at * 2))
-                             : 0u;
-            }
+          for (int q = 0; q < 4; ++q) {
+            const int row = n0 + rg * 16 + g + 8 * (q & 1), col = kk * 16 + 2 * t + 8 * (q >> 1);
+            const size_t at = (ROUTED ? (size_t)sg.x * a.N + row : (size_t)row) * a.r + col;
+            bf[q] = row < a.N && col < a.r
+                        ? __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(a.lora_b[p]) + at * 2))
+                        : 0u;
+          }
         };
-        uint32_t bf[2][4];
-        load_b(0, bf);
-        for (int kk = 0; kk < RK; ++kk) {
-          uint32_t bn[2][4] = {};
-          if (kk + 1 < RK) load_b(kk + 1, bn);
+        // the fragments of a rank step: from shared memory, or (routed) from L2 a step ahead
+        auto load_t = [&](int p, int kk, uint4 (&tv)[NT], uint2 (&tl)[NT]) {
 #pragma unroll
-          for (int p = 0; p < 2; ++p)
+          for (int nt = 0; nt < NT; ++nt) {
+            const uint32_t at = ((p * RK + kk) * NT + nt) * kTfragBytes;
+            if (ROUTED) {
+              const uint8_t *src = a.tfrag + (size_t)seg * (2 * RK * NT * kTfragBytes) + at;
+              tv[nt] = __ldcg(reinterpret_cast<const uint4 *>(src) + lane);
+              tl[nt] = __ldcg(reinterpret_cast<const uint2 *>(src + 512) + lane);
+            } else {
+              tv[nt] = lds128(smem + C::OFF_TF + at + lane * 16);
+              tl[nt] = lds64(smem + C::OFF_TF + at + 512 + lane * 8);
+            }
+          }
+        };
+        // PP projections at a time: both where their registers allow (d 4096 in
+        // groups of 32 at 5 tokens 38.4 -> 38.1 us a layer against one at a time; two
+        // parts of t in place of three took 37.9)
+        constexpr int PP = NT <= (ROUTED ? 1 : 2) ? 2 : 1;
+        uint32_t bf[PP][4], bn[PP][4] = {};
+        uint4 tv[PP][NT], tvn[PP][NT] = {};
+        uint2 tl[PP][NT], tln[PP][NT] = {};
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              const uint32_t at = (((p * RK + kk) * NT + nt) * 32 + lane) * 16;
-              const uint4 tv = ROUTED ? __ldcg(reinterpret_cast<const uint4 *>(
-                                            a.tfrag + (size_t)seg * (2 * RK * NT * 512) + at))
-                                      : lds128(smem + C::OFF_TF + at);
-              mma_bf16_16816(tot[p][nt], bf[p], tv.x, tv.y);
-              mma_bf16_16816(tot[p][nt], bf[p], tv.z, tv.w);
+        for (int q = 0; q < PP; ++q) {
+          load_b(q, 0, bf[q]);
+          if (ROUTED) load_t(q, 0, tv[q], tl[q]);
+        }
+#pragma unroll
+        for (int p0 = 0; p0 < 2; p0 += PP) {
+          float ad[PP][NT][4] = {};
+#pragma unroll 1
+          for (int kk = 0; kk < RK; ++kk) {
+            const bool same = kk + 1 < RK;
+            if (same || p0 + PP < 2) {
+#pragma unroll
+              for (int q = 0; q < PP; ++q) {
+                load_b(same ? p0 + q : 1, same ? kk + 1 : 0, bn[q]);
+                if (ROUTED) load_t(same ? p0 + q : 1, same ? kk + 1 : 0, tvn[q], tln[q]);
+              }
             }
 #pragma unroll
-          for (int p = 0; p < 2; ++p)
+            for (int q = 0; q < PP; ++q)
+              if (!ROUTED) load_t(p0 + q, kk, tv[q], tl[q]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) bf[p][q] = bn[p][q];
+            for (int part = 2; part >= 0; --part)
+#pragma unroll
+              for (int q = 0; q < PP; ++q)
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) {
+                  const uint4 v = tv[q][nt];
+                  const uint2 w = part == 2 ? tl[q][nt] : part == 1 ? make_uint2(v.z, v.w) : make_uint2(v.x, v.y);
+                  mma_bf16_16816(ad[q][nt], bf[q], w.x, w.y);
+                }
+#pragma unroll
+            for (int q = 0; q < PP; ++q) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) bf[q][e] = bn[q][e];
+#pragma unroll
+              for (int nt = 0; nt < NT; ++nt)
+                if (ROUTED) tv[q][nt] = tvn[q][nt], tl[q][nt] = tln[q][nt];
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < PP; ++q)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) tot[p0 + q][nt][e] += ad[q][nt][e];
         }
       }
       // h = SiLU(rs g) rs u, staged as bf16 [token][128 rows]

@@ -57,14 +57,19 @@ inline int batch_routed_occ(int nt, long long tiles, int num_sms) {
   return nt <= 2 && 4 * tiles >= 11LL * num_sms ? 2 : 1;
 }
 
+// A fragment of the LoRA-A products t in three bf16 parts whose sum is the fp32
+// value: [32 lanes][16 bytes] the high and the middle part, then [32 lanes][8
+// bytes] the low one.
+constexpr uint32_t kTfragBytes = 768;
+
 struct BatchArgs {
   const uint8_t *panel;      // [ceil(K / 128)] records
   int M, N, K, group;
   const uint32_t *codes[2];  // gate, up; or down
   const uint16_t *meta[2];
-  // gate/up: lora_scale * x A^T as bf16 high and low parts, m16n8k16 B
-  // fragments [projection][ceil(r / 16)][NT][32 lanes][16 bytes] (null: no
-  // adapter); LoRA-B bf16 [N][r]; RMSNorm scale per token (null: 1)
+  // gate/up: lora_scale * x A^T, m16n8k16 B fragments [projection][ceil(r / 16)]
+  // [NT] of kTfragBytes (null: no adapter); LoRA-B bf16 [N][r]; RMSNorm scale
+  // per token (null: 1)
   const uint8_t *tfrag;
   int r;
   const void *lora_b[2];

@@ -164,6 +164,59 @@ def test_batch_stack_of_a_large_layer(wq, bits, m):
     check_bf16(y, ref, f"large layer y bits={bits} m={m}")
 
 
+def _cancelling_adapter(d, inter, r, gen):
+    """Weights of value zero and an adapter whose large products cancel: the rows of A
+    come in pairs whose products with x differ by x[0] (x and A are integers, so every
+    fp32 sum is exact), and B subtracts one from the other.  Returns (gate, up, A, Bg, Bu)."""
+    pairs = gen.integers(1, 128, (r, d)).astype(np.float32)  # row 2 i of gate, then of up
+    a = np.repeat(pairs.reshape(r, 1, d), 2, 1).reshape(2 * r, d)
+    a[1::2, 0] += 1
+    b = [np.tile(np.array([-1, 1], np.float32) * (1 + i), (inter, r // 2)) / 16 for i in range(2)]
+    z = (np.zeros((inter, d), np.uint8), np.full((inter, d // 64), 0x3C00, np.uint16), np.zeros((inter, d // 64), np.uint16))
+    return z, *(torch.from_numpy(v).to(torch.bfloat16) for v in (a, *b))
+
+
+@pytest.mark.parametrize("bits,d,inter,r,m", [(2, 256, 144, 8, 9), (2, 512, 768, 32, 24), (3, 256, 200, 64, 33),
+                                              (2, 1024, 400, 16, 64)])
+def test_adapter_products_are_kept_in_fp32(wq, bits, d, inter, r, m):
+    """t = x A^T of 2^20 and more whose differences are 1 to 64: with fewer than 24 bits
+    in t the difference is lost.  Exact sums, so h is the exact value rounded twice at
+    most (fp32 SiLU, bf16)."""
+    gen = np.random.default_rng(d + r)
+    z, a, bg, bu = _cancelling_adapter(d, inter, r, gen)
+    q = upload_packed(*z, 64, bits)
+    x = gen.integers(64, 128, (m, d)).astype(np.float32)
+    x[:, 0] = gen.integers(1, 65, m)
+    fn = wq.gateup_w2_lora if bits == 2 else wq.gateup_w3_lora
+    h = fn(torch.from_numpy(x).to(torch.bfloat16).cuda(), q, q, a.cuda(), bg.cuda(), bu.cuda(), lora_scale=0.25)
+    g = x[:, :1].astype(np.float64) * 0.25 * (r / 2) / 16  # r / 2 pairs of weight 1 / 16
+    ref = np.broadcast_to(g / (1 + np.exp(-g)) * (2 * g), (m, inter))
+    got = h.float().cpu().numpy().astype(np.float64)
+    # half a bf16 unit and 16 fp32 ones for the SiLU's exponential and quotient
+    assert (np.abs(got - ref) <= np.abs(ref) * (2.0 ** -8 + 2.0 ** -20)).all(), np.abs(got / ref - 1).max()
+
+
+@pytest.mark.parametrize("m,E,k,r", [(16, 4, 2, 8), (40, 8, 4, 24)])
+def test_grouped_expert_adapter_products_are_kept_in_fp32(wq, m, E, k, r):
+    d, inter = 2048, 1024
+    gen = np.random.default_rng(m + E)
+    z, a, bg, bu = _cancelling_adapter(d, inter, r, gen)
+    st = lambda t: torch.cat([t] * E).contiguous().cuda()
+    zz = upload_packed(*(np.concatenate([v] * E) for v in z), 64, 2)
+    down = wq.pack(torch.randn((E * d, inter), device="cuda", generator=torch.Generator("cuda").manual_seed(1)) * 0.02, 64, 4)
+    layer = wq.MoELayer(wq.MLPLayer(zz, zz, down, lora_a=st(a), lora_b_gate=st(bg), lora_b_up=st(bu), lora_scale=0.25),
+                        E, k)
+    x = gen.integers(8, 16, (m, d)).astype(np.float32)
+    x[:, 0] = gen.integers(1, 65, m)
+    lg = torch.from_numpy(gen.standard_normal((m, E)).astype(np.float32)).cuda()
+    _, _, _, hs, _ = wq.moe_forward(torch.from_numpy(x).to(torch.bfloat16).cuda(), lg, layer, prenorm=False,
+                                    with_slots=True)
+    g = np.repeat(x[:, :1].astype(np.float64), k, 0) * 0.25 * (r / 2) / 16
+    ref = np.broadcast_to(g / (1 + np.exp(-g)) * (2 * g), hs.shape)
+    got = hs.float().cpu().numpy().astype(np.float64)
+    assert (np.abs(got - ref) <= np.abs(ref) * (2.0 ** -8 + 2.0 ** -20)).all(), np.abs(got / ref - 1).max()
+
+
 def test_moe_workspace_of_several_token_counts(wq):
     """One workspace for the largest token count serves smaller ones in between,
     on the slots' and the grouped launches."""
