@@ -7,7 +7,7 @@
 // binary16 subnormal code * 4^c * 2^-24 (c its bit-position class, cancelled
 // by the activation's scale), mma.sync m16n8k16 multiplies it exactly with
 // binary16 activations and sums in fp32, and per quantization group
-//   tot += s * (sx * sum code x') - s z * sum x
+//   tot += s sx * (sum code x' - z * sum x')
 // is the affine dequantization s (q - z).  The tcgen05 path has to write every
 // dequantized weight to shared memory first, whatever the token count; here a
 // fragment of 256 weights costs 4 ANDs and is used for all tokens.
@@ -70,6 +70,12 @@ struct BatchCfg {
   // of 32 at 64 tokens 111 -> 105; only 4-bit codes in groups of 128 at 56
   // tokens and more lose (d 4096 87.4 -> 89.3).
   static constexpr bool PAIRED = !(BITS == 4 && GPB == 1 && NT == 8);
+  // mma.sync truncates its sums: a down launch of up to 16 tokens adds a group of
+  // 128 from two chains of 4, as the GEMV kernels that small matrices take do (d
+  // 5120 x 17408 at 4 tokens of mean 0.5: error 1.6e-6 of the result with one
+  // chain of 8, 5.8e-7 with two, 7.5e-7 on the GEMV kernels; above 16 tokens the
+  // tcgen05 launch that was faster before had 1.05e-5, one chain has 1.65e-6).
+  static constexpr bool SPLIT = NPROJ == 1 && GROUP == 128 && NT <= 2;
   static constexpr int REC = NT * (2048 + 32 + 32 * GPB);
   static constexpr int SLOT = 2 * (BPK + GPB * 64);  // two tiles of a unit
   static constexpr int TF = BITS == 4 || OCC == 2 ? 0 : 8 * NT * (int)kTfragBytes;  // LoRA-A products (rank 64; routed: from L2)
@@ -119,7 +125,7 @@ __device__ __forceinline__ void batch_panel_token(uint8_t *rec, int nt_total, in
   float gs = (f[0] + f[1]) + (f[2] + f[3]);
   const int lpg = group >> 2;  // lanes of a group
   for (int o = 1; o < lpg; o <<= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
-  if (lane % lpg == 0) sx[(1 + lane / lpg) * nt_total * 8 + m] = gs;
+  if (lane % lpg == 0) sx[(1 + lane / lpg) * nt_total * 8 + m] = gs * batch_exp2i(e - 24);
   if (lane == 0) sx[m] = batch_exp2i(24 - e);
 }
 
@@ -307,7 +313,7 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
             wd[tl][NW - 4] = w1.x; wd[tl][NW - 3] = w1.y; wd[tl][NW - 2] = w1.z; wd[tl][NW - 1] = w1.w;
           }
         }
-        float acc[2][NT][4];
+        float acc[2][NT][4], acc2[2][NT][4];  // acc2: C::SPLIT's second half of the block
 #pragma unroll
         for (int kp = 0; kp < 4; ++kp) {
           uint4 b[NT];
@@ -347,13 +353,17 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
 #pragma unroll
               for (int tl = 0; tl < 2; ++tl) {
                 const uint32_t b0 = hf ? b[nt].z : b[nt].x, b1 = hf ? b[nt].w : b[nt].y;
-                if (ks % GS == 0)
-                  mma_f16_16816_zc(acc[tl][nt], af[tl], b0, b1);
+                float(&c)[4] = C::SPLIT && ks >= 4 ? acc2[tl][nt] : acc[tl][nt];
+                if (ks % (C::SPLIT ? 4 : GS) == 0)
+                  mma_f16_16816_zc(c, af[tl], b0, b1);
                 else
-                  mma_f16_16816(acc[tl][nt], af[tl], b0, b1);
+                  mma_f16_16816(c, af[tl], b0, b1);
               }
             if ((ks + 1) % GS == 0) {
-              // the group's share: tot += s (sx sum q x') - s z sum x
+              // the group's share, tot += s sx (sum q x' - z sum x'): the difference
+              // first, rounded once (sx is a power of two).  Added to tot one by one the
+              // two terms round at their own size, which for activations of one sign is
+              // many times the difference's.
               const int gl = ks / GS;
               float sl[2], sh[2], zl[2], zh[2];
 #pragma unroll
@@ -361,8 +371,8 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
                 const uint2 sz = lds64(cw + 2 * BPK + (tl * GPB + gl) * 64 + g * 8);
                 sl[tl] = batch_half(sz.x);
                 sh[tl] = batch_half(sz.x >> 16);
-                zl[tl] = -sl[tl] * batch_half(sz.y);
-                zh[tl] = -sh[tl] * batch_half(sz.y >> 16);
+                zl[tl] = -batch_half(sz.y);
+                zh[tl] = -batch_half(sz.y >> 16);
               }
 #pragma unroll
               for (int nt = 0; nt < NT; ++nt) {
@@ -371,17 +381,21 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
 #pragma unroll
                 for (int tl = 0; tl < 2; ++tl) {
                   float *c = tot[tl][nt];
-                  const float *q = acc[tl][nt];
+                  float *q = acc[tl][nt];
+                  if (C::SPLIT)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) q[e] += acc2[tl][nt][e];
                   if (C::PAIRED) {  // the same operations and roundings
-                    fma_f32x2(c[0], c[1], mul_f32x2(sl[tl], sl[tl], sx.x, sx.y), q[0], q[1]);
-                    fma_f32x2(c[0], c[1], pack_f32x2(zl[tl], zl[tl]), xs.x, xs.y);
-                    fma_f32x2(c[2], c[3], mul_f32x2(sh[tl], sh[tl], sx.x, sx.y), q[2], q[3]);
-                    fma_f32x2(c[2], c[3], pack_f32x2(zh[tl], zh[tl]), xs.x, xs.y);
+                    const uint64_t sx2 = pack_f32x2(sx.x, sx.y), xs2 = pack_f32x2(xs.x, xs.y);
+                    const uint64_t dl = fma_f32x2(pack_f32x2(zl[tl], zl[tl]), xs2, pack_f32x2(q[0], q[1]));
+                    const uint64_t dh = fma_f32x2(pack_f32x2(zh[tl], zh[tl]), xs2, pack_f32x2(q[2], q[3]));
+                    unpack_f32x2(fma_f32x2(mul_f32x2(pack_f32x2(sl[tl], sl[tl]), sx2), dl, pack_f32x2(c[0], c[1])), c[0], c[1]);
+                    unpack_f32x2(fma_f32x2(mul_f32x2(pack_f32x2(sh[tl], sh[tl]), sx2), dh, pack_f32x2(c[2], c[3])), c[2], c[3]);
                   } else {
-                    c[0] = fmaf(zl[tl], xs.x, fmaf(sl[tl] * sx.x, q[0], c[0]));
-                    c[1] = fmaf(zl[tl], xs.y, fmaf(sl[tl] * sx.y, q[1], c[1]));
-                    c[2] = fmaf(zh[tl], xs.x, fmaf(sh[tl] * sx.x, q[2], c[2]));
-                    c[3] = fmaf(zh[tl], xs.y, fmaf(sh[tl] * sx.y, q[3], c[3]));
+                    c[0] = fmaf(sl[tl] * sx.x, fmaf(zl[tl], xs.x, q[0]), c[0]);
+                    c[1] = fmaf(sl[tl] * sx.y, fmaf(zl[tl], xs.y, q[1]), c[1]);
+                    c[2] = fmaf(sh[tl] * sx.x, fmaf(zh[tl], xs.x, q[2]), c[2]);
+                    c[3] = fmaf(sh[tl] * sx.y, fmaf(zh[tl], xs.y, q[3]), c[3]);
                   }
                 }
               }

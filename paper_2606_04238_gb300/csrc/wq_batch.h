@@ -27,7 +27,7 @@ inline int batch_nt(int m) {
 //                                codes) or 16^-c (4-bit) for the bit-position
 //                                class c of the codes they meet
 //   [NT * 8] fp32                2^(24 - e) per token
-//   [128 / group][NT * 8] fp32   sums of x over each quantization group
+//   [128 / group][NT * 8] fp32   sums of x 2^(e - 24) over each quantization group
 inline __host__ __device__ uint32_t batch_rec_bytes(int nt, int group) {
   return (uint32_t)nt * (2048u + 32u + 32u * (128u / (uint32_t)group));
 }

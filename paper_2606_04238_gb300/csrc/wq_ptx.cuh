@@ -133,16 +133,19 @@ __device__ __forceinline__ uint64_t pack_f32x2(float a, float b) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
   return v;
 }
-__device__ __forceinline__ uint64_t mul_f32x2(float a0, float a1, float b0, float b1) {
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
   uint64_t v;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pack_f32x2(a0, a1)), "l"(pack_f32x2(b0, b1)));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
   return v;
 }
-// (c0, c1) += a * (b0, b1)
-__device__ __forceinline__ void fma_f32x2(float &c0, float &c1, uint64_t a, float b0, float b1) {
+// a * b + c
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t v;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(pack_f32x2(b0, b1)), "l"(pack_f32x2(c0, c1)));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(v));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
 
 // D = A * B + C on the tensor cores: m16n8k16, A row-major f16, B col-major
