@@ -41,8 +41,9 @@
 // warps an SM keep ~190 KB in flight.  Measured (GB300, cold, us, lanes' dot
 // products with 8 warps a CTA and two CTAs an SM before -> this): 16 sequences of 512
 // to 2048 positions, 32 / 8 heads of 128: 39.1 -> 24.4 for 84 MB of cache rows;
-// one of 8192: 17.5 -> 14.7 for 34 MB.  Share of bf16 outputs off the exact
-// rounding 0.00026 -> 0.00024 at 8192 positions, 0.00026 -> 0.00019 at 2048.
+// one of 8192: 17.5 -> 14.7 for 34 MB; the kept roundings of the scores (below) took
+// 0.6 and 0.2 us of it back.  Share of bf16 outputs off the exact rounding 0.00027
+// -> 0.00022 at 8192 positions, 0.00024 -> 0.00019 at 512 to 2048.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -329,23 +330,36 @@ __global__ void __launch_bounds__(kAttnWarps * 32, kAttnOcc) attn_split_kernel(
         __syncwarp();
       }
       const uint32_t krow = smem_addr(cur) + lrow * (HD * 2), vrow = krow + kPos * HD * 2;
-      // Each MMA starts from zero and is added in fp32 here (likewise for P V):
-      // the tensor core's own accumulation truncates, which showed as twice the
-      // outputs off the exact rounding.
-      float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+      // The tensor core's own accumulation truncates, which showed as twice the
+      // outputs off the exact rounding, so Q's first parts start every MMA from zero
+      // and are added in fp32 here (likewise P V); the other two, 2^-8 and 2^-16 of
+      // them, accumulate.  The first parts' sums are added pairwise, then with what
+      // each addition rounds away kept (Knuth's two-sum).  Scores of deviation 6 (in
+      // units of log 2), outputs off the exact rounding: added one by one 0.00052,
+      // this 0.00033, lanes' dot products 0.00038.
+      float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f}, pair[2] = {0.f, 0.f};
+      float hi[2] = {0.f, 0.f}, rest[2] = {0.f, 0.f};
 #pragma unroll
       for (int ks = 0; ks < HD / 16; ++ks) {
         uint32_t ka[4];
         ldmatrix_x4(ka, krow + (((2 * ks + lchk) ^ (lrow & 7)) << 4));
-        float t0[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_bf16_16816(t0, ka, qb[ks][0][0], qb[ks][0][1]);
+        d0[0] = d0[2] = 0.f;
+        mma_bf16_16816(d0, ka, qb[ks][0][0], qb[ks][0][1]);
         mma_bf16_16816(d1, ka, qb[ks][1][0], qb[ks][1][1]);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) d0[e] += t0[e];
+        for (int i = 0; i < 2; ++i) {
+          if (ks % 2 == 0) {
+            pair[i] = d0[2 * i];
+          } else {
+            const float v = pair[i] + d0[2 * i], sum = __fadd_rn(hi[i], v), bb = __fsub_rn(sum, hi[i]);
+            if (ks > 1) rest[i] = __fadd_rn(rest[i], __fadd_rn(__fsub_rn(hi[i], __fsub_rn(sum, bb)), __fsub_rn(v, bb)));
+            hi[i] = ks > 1 ? sum : v;
+          }
+        }
       }
       // scores of positions c0 + gr, c0 + gr + 8 with head h0 + tc
-      const float s0 = c0 + gr < p1 ? (d0[0] + d0[1]) + d1[0] : -INFINITY;
-      const float s1 = c0 + gr + 8 < p1 ? (d0[2] + d0[3]) + d1[2] : -INFINITY;
+      const float s0 = c0 + gr < p1 ? hi[0] + ((d0[1] + d1[0]) + rest[0]) : -INFINITY;
+      const float s1 = c0 + gr + 8 < p1 ? hi[1] + ((d0[3] + d1[2]) + rest[1]) : -INFINITY;
       float mc = fmaxf(s0, s1);
       mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 4));
       mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, 8));
