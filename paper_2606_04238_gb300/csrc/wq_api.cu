@@ -764,10 +764,13 @@ size_t wq_workspace_bytes(int m, int d, int inter, int r) {
   const SizeMemo<size_t, 4>::Key key{m, d, inter, num_sms()};
   size_t most = 0;  // enough for every token count up to m
   if (memo.find(key, &most)) return most;
-  if (m > kMaxTokens) {
+  // The stream-K scratch comes and goes with the split, which is the same for all
+  // token counts of a number of tiles (of 128 tokens, from 129 on of 256): the
+  // largest count of each.
+  for (int mm = std::min(m, 128); mm > kMaxTokens; mm = mm == m ? 0 : std::min(m, mm < 256 ? 256 : mm + 256)) {
     WsLayout L;
-    if (!ws_layout(m, d, inter, &L)) return 0;  // grows with m
-    most = L.total;
+    if (!make_ws_layout(mm, d, inter, &L, false)) return 0;
+    most = std::max(most, L.total);
   }
   for (int mm = 1; mm <= std::min(m, kMaxTokens); ++mm) {
     WsLayout L;

@@ -249,3 +249,21 @@ def test_gemm_down_tall_tiles(wq, d, inter, group, m):
     for got, r, what in ((y, res, "residual"), (y0, None, "plain")):
         ref, _ = orc.down(synth.bf16_bits(h)[rows], qd, group, None if r is None else synth.bf16_bits(r)[rows])
         check_bf16(got[torch.from_numpy(rows).cuda()], ref, f"tall {what} d={d} I={inter} m={m}", min_exact=MIN_EXACT)
+
+
+@pytest.mark.parametrize("d,inter", [(2560, 9728), (4096, 2560)])
+def test_workspace_of_several_token_counts(wq, d, inter):
+    """One workspace for the largest count serves smaller ones in between, also where
+    the split of the work needs scratch at the smaller count only."""
+    gen = torch.Generator("cuda").manual_seed(d)
+    mk = lambda n, k, bits: wq.pack(torch.randn((n, k), device="cuda", generator=gen) * 0.02, 128, bits)
+    layer = wq.MLPLayer(mk(inter, d, 2), mk(inter, d, 2), mk(d, inter, 4))
+    ws = wq.workspace(1400, d, inter, 0)
+    for i, m in enumerate((1400, 512, 130, 128, 65, 24, 300, 1, 9)):
+        x = synth.activations((m, d), 300 + i).cuda()
+        y, y0 = wq.mlp_forward(x, [layer], ws=ws).clone(), wq.mlp_forward(x, [layer])
+        assert torch.equal(y.view(torch.int16), y0.view(torch.int16)), m
+    small = wq.workspace(129, d, inter, 0)
+    x = synth.activations((128, d), 1).cuda()
+    assert torch.equal(wq.mlp_forward(x, [layer], ws=small), wq.mlp_forward(x, [layer]))
+    assert wq.device_status() == 0
