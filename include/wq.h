@@ -324,7 +324,8 @@ wq_status wq_mlp_forward(const void *x, int m, const wq_mlp_layer *layers, int n
  *            the device status (wq_device_status).
  *   caches:  bf16 [batch, n_kv, max_len, head_dim].  o: bf16 [batch, n_heads head_dim].
  *   Supported: head_dim 64 or 128, n_heads a multiple of n_kv, n_heads / n_kv <= 8.
- *   Workspace: wq_attn_workspace_bytes (split partial results, no zeroing needed).
+ *   Workspace: wq_attn_workspace_bytes for up to `batch` sequences (split partial
+ *   results, no zeroing needed).
  */
 size_t wq_attn_workspace_bytes(int batch, int n_heads, int n_kv, int head_dim, int max_len);
 wq_status wq_attn_decode(const float *qkv, const void *x, const int32_t *lens, int batch, int d, int n_heads,
@@ -346,7 +347,8 @@ typedef struct {
  *   y = the MLP block on x1 (as wq_gateup_* then wq_down_w4 with residual x1;
  *   flags as for wq_mlp_forward, WQ_PRENORM for the MLP's RMSNorm).
  * Five calls on `stream`; the caches gain position lens[b] (lens is not changed).
- * Workspace: wq_decoder_workspace_bytes, zero-filled before first use (wq_workspace_init).
+ * Workspace: wq_decoder_workspace_bytes for up to `batch` sequences, zero-filled
+ * before first use (wq_workspace_init).
  */
 size_t wq_decoder_workspace_bytes(int batch, const wq_decoder_layer *layer, int max_len);
 wq_status wq_decoder_layer_forward(const void *x, int batch, const int32_t *lens, const wq_decoder_layer *layer,

@@ -1229,11 +1229,21 @@ wq_status wq_mlp_forward_info(int m, const wq_mlp_layer *layers, int n_layers, u
   return ok();
 }
 
+}  // extern "C"
+
+namespace {
+// Partial results of `parts` (sequence, split) pairs.
+size_t attn_ws_bytes(long long parts, int n_heads, int head_dim) {
+  return up256((size_t)parts * n_heads * (head_dim + 2) * 4);
+}
+}  // namespace
+
+extern "C" {
+
 size_t wq_attn_workspace_bytes(int batch, int n_heads, int n_kv, int head_dim, int max_len) {
   const int sms = num_sms();
   if (batch <= 0 || n_heads <= 0 || n_kv <= 0 || head_dim <= 0 || max_len <= 0 || sms <= 0) return 0;
-  const int S = attn_splits(batch, n_kv, max_len, sms);
-  return up256((size_t)batch * n_heads * S * (head_dim + 2) * 4);
+  return attn_ws_bytes(attn_most_parts(batch, n_kv, max_len, sms), n_heads, head_dim);
 }
 
 }  // extern "C"
@@ -1254,10 +1264,11 @@ wq_status attn_decode_impl(const float *qkv, const void *x, const int32_t *lens,
   if (!aligned16(qkv) || !aligned16(x) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(o) ||
       !aligned16(ws))
     return fail(WQ_ERR_ALIGN, "qkv, x, caches, o or workspace not 16-byte aligned");
-  if (ws_bytes < wq_attn_workspace_bytes(batch, n_heads, n_kv, head_dim, max_len))
-    return fail(WQ_ERR_WORKSPACE, "attention workspace of %zu bytes, %zu needed", ws_bytes,
-                wq_attn_workspace_bytes(batch, n_heads, n_kv, head_dim, max_len));
-  const int S = attn_splits(batch, n_kv, max_len, num_sms());
+  const int sms = num_sms();
+  if (sms <= 0) return fail(WQ_ERR_CUDA, "cannot query the current device");
+  const int S = attn_splits(batch, n_kv, max_len, sms);
+  const size_t need = attn_ws_bytes((long long)batch * S, n_heads, head_dim);
+  if (ws_bytes < need) return fail(WQ_ERR_WORKSPACE, "attention workspace of %zu bytes, %zu needed", ws_bytes, need);
   cudaError_t e = launch_attn_decode(qkv, x, reinterpret_cast<const int *>(lens), batch, d, n_heads, n_kv, head_dim,
                                      (double)theta, k_cache, v_cache, max_len, static_cast<float *>(ws), S, o,
                                      early, static_cast<cudaStream_t>(stream));

@@ -536,6 +536,11 @@ int attn_splits(int B, int Hkv, int max_len, int num_sms) {
   return std::max(1, std::min(want, (max_len + 63) / 64));
 }
 
+long long attn_most_parts(int B, int Hkv, int max_len, int num_sms) {
+  // b splits(b) is b, or at most the CTAs held (and 64 positions a split)
+  return std::min(std::max((long long)B, (long long)kAttnOcc * num_sms / Hkv), (long long)B * ((max_len + 63) / 64));
+}
+
 namespace {
 
 template <int HD>

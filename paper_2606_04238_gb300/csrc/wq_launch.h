@@ -30,6 +30,8 @@ cudaError_t launch_attn_decode(const float *qkv, const void *x, const int *lens,
                                bool early, cudaStream_t s);
 // Context splits of a launch (S above).
 int attn_splits(int B, int Hkv, int max_len, int num_sms);
+// The most (sequence, split) pairs of a launch of up to B sequences.
+long long attn_most_parts(int B, int Hkv, int max_len, int num_sms);
 // Reads and clears the attention kernels' device status word.
 cudaError_t read_attn_status(int *status);
 

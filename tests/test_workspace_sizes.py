@@ -53,3 +53,18 @@ def run(tmp_path_factory):
 @pytest.mark.parametrize("d,inter", [(2560, 9728), (5120, 17408), (4096, 14336), (4096, 2560), (512, 896)])
 def test_layer_workspace_grows_with_the_tokens(run, d, inter):
     run(f"grows((m, L.wq_workspace_bytes(m, {d}, {inter}, 16)) for m in [*range(1, 1030), *range(1030, 4200, 13), 16384])")
+
+
+@pytest.mark.parametrize("heads,kv,hd,max_len", [(32, 8, 128, 8192), (16, 4, 64, 2048), (8, 1, 64, 100000)])
+def test_attention_workspace_grows_with_the_batch(run, heads, kv, hd, max_len):
+    run(f"grows((b, L.wq_attn_workspace_bytes(b, {heads}, {kv}, {hd}, {max_len})) for b in range(1, 1200))")
+
+
+@pytest.mark.parametrize("d,inter,heads,kv,hd,max_len", [(2560, 9728, 32, 8, 128, 8192), (512, 896, 8, 1, 64, 100000),
+                                                         (1024, 1024, 32, 8, 128, 32768)])
+def test_decoder_workspace_grows_with_the_batch(run, d, inter, heads, kv, hd, max_len):
+    run(f"""
+mlp = wq._MLPLayer(q({inter}, {d}, 128, 2), q({inter}, {d}, 128, 2), q({d}, {inter}, 128, 4), None, None, None, 0, 1.0)
+layer = wq._DecoderLayer(q({(heads + 2 * kv) * hd}, {d}, 128, 4), q({d}, {heads * hd}, 64, 4), mlp, {heads}, {kv}, {hd}, 1e6)
+grows((b, L.wq_decoder_workspace_bytes(b, ctypes.byref(layer), {max_len})) for b in range(1, 300))
+""")
