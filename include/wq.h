@@ -390,8 +390,8 @@ typedef struct {
  * above, five (routing and grouping
  * of the slots by expert, the groups' inputs, gate/up and down over the groups,
  * combine).  Only the selected experts' weights are read.
- * Workspace: wq_moe_workspace_bytes for this layer, token count and flags,
- * zero-filled before first use (wq_workspace_init).
+ * Workspace: wq_moe_workspace_bytes for this layer, up to m tokens and these
+ * flags, zero-filled before first use (wq_workspace_init).
  */
 size_t wq_moe_workspace_bytes(int m, const wq_moe_layer *layer, unsigned flags);
 wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe_layer *layer, unsigned flags,

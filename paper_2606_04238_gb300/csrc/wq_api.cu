@@ -1590,8 +1590,19 @@ extern "C" {
 
 size_t wq_moe_workspace_bytes(int m, const wq_moe_layer *layer, unsigned flags) {
   if (m <= 0 || moe_check(m, layer) != WQ_OK) return 0;
+  const wq_mlp_layer &X = layer->experts;
+  static SizeMemo<size_t, 11> memo;
+  const SizeMemo<size_t, 11>::Key key{m, layer->n_experts, layer->top_k, X.gate.n, X.gate.k, X.gate.bits, X.gate.group,
+                                      X.down.group, X.r, flags & WQ_PRENORM ? 1 : 0, num_sms()};
+  size_t most = 0;  // enough for every token count up to m
+  if (memo.find(key, &most)) return most;
   MoeWs W;
-  return moe_ws(m, *layer, flags, &W) ? W.total : 0;
+  if (!moe_ws(m, *layer, flags, &W)) return 0;
+  most = W.total;
+  for (int mm = 1; mm < m; ++mm)
+    if (moe_ws(mm, *layer, flags, &W)) most = std::max(most, W.total);
+  memo.put(key, most);
+  return most;
 }
 
 wq_status wq_moe_forward(const void *x, int m, const float *logits, const wq_moe_layer *layer, unsigned flags,

@@ -68,3 +68,14 @@ mlp = wq._MLPLayer(q({inter}, {d}, 128, 2), q({inter}, {d}, 128, 2), q({d}, {int
 layer = wq._DecoderLayer(q({(heads + 2 * kv) * hd}, {d}, 128, 4), q({d}, {heads * hd}, 64, 4), mlp, {heads}, {kv}, {hd}, 1e6)
 grows((b, L.wq_decoder_workspace_bytes(b, ctypes.byref(layer), {max_len})) for b in range(1, 300))
 """)
+
+
+@pytest.mark.parametrize("d,inter,experts,top_k,group", [(4096, 4096, 8, 2, 128), (2880, 2880, 32, 4, 64),
+                                                         (2048, 1024, 16, 4, 64)])
+def test_moe_workspace_grows_with_the_tokens(run, d, inter, experts, top_k, group):
+    run(f"""
+gu, dn = q({experts * inter}, {d}, {group}, 2), q({experts * d}, {inter}, {group}, 4)
+layer = wq._MoELayer(wq._MLPLayer(gu, gu, dn, 256, 256, 256, 16, 1.0), {experts}, {top_k})
+for flags in (0, wq.WQ_PRENORM):
+    grows((m, L.wq_moe_workspace_bytes(m, ctypes.byref(layer), flags)) for m in range(1, 65))
+""")
