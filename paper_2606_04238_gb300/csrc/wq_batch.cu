@@ -7,6 +7,7 @@
 // GPT-OSS-20B shape, top 4 of 32: 494 -> 127 us a block, of which gate/up ~70
 // and down ~40; its 334 MB of packed experts take 49 us at the copy rate).
 #include "wq_batch.cuh"
+#include "wq_route.cuh"
 
 namespace wq {
 namespace {
@@ -166,9 +167,6 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __nv_bfl
 
 constexpr int kRouteThreads = 1024;
 
-// (logit, expert) a ranks before b: the larger logit, the lower index among equal ones.
-__device__ __forceinline__ bool route_before(float la, int ea, float lb, int eb) { return la > lb || (la == lb && ea < eb); }
-
 // One CTA.  Warp t: the top_k experts of token t by logit and the softmax of
 // the selected logits (fp32, the largest subtracted).  Then the slots of each
 // expert in slot order (one warp an expert, ballots over the slots), cut into
@@ -176,45 +174,22 @@ __device__ __forceinline__ bool route_before(float la, int ea, float lb, int eb)
 __global__ void __launch_bounds__(kRouteThreads) batch_route_kernel(const float *logits, int m, int E, int top_k,
                                                                     int tok, int *idx_out, float *w_out,
                                                                     BatchRoute *route) {
-  __shared__ int idx_s[kRouteMaxSlots], count_s[256], first_s[256], seg_s[256];
+  __shared__ int idx_s[kRouteMaxSlots], count_s[kMoeMaxExperts], first_s[kMoeMaxExperts], seg_s[kMoeMaxExperts];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kRouteThreads / 32;
   pdl_wait();
   pdl_launch_dependents();
   for (int t = warp; t < m; t += nw) {
-    // lane l holds experts l, l + 32, ..: taken ones are marked by clearing their bit
-    float lg[8];
-    uint32_t live = 0u;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int e = lane + 32 * i;
-      lg[i] = e < E ? __ldcg(logits + (size_t)t * E + e) : 0.f;
-      if (e < E) live |= 1u << i;
-    }
+    RouteKeys keys;
+    route_load(keys, logits + (size_t)t * E, E, lane);
     float first = 0.f, mine = 0.f, sum = 0.f;  // lane c: choice c
     int mine_e = 0;
     for (int c = 0; c < top_k; ++c) {
-      float bl = 0.f;
-      int be = 0x7fffffff;
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (((live >> i) & 1u) && (be == 0x7fffffff || route_before(lg[i], lane + 32 * i, bl, be))) {
-          bl = lg[i];
-          be = lane + 32 * i;
-        }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ol = __shfl_xor_sync(0xffffffffu, bl, o);
-        const int oe = __shfl_xor_sync(0xffffffffu, be, o);
-        if (oe != 0x7fffffff && (be == 0x7fffffff || route_before(ol, oe, bl, be))) {
-          bl = ol;
-          be = oe;
-        }
-      }
-      if ((be & 31) == lane) live &= ~(1u << (be >> 5));
-      if (c == 0) first = bl;
-      const float ex = expf(bl - first);
+      float l;
+      const int e = route_next(keys, lane, l);
+      if (c == 0) first = l;
+      const float ex = expf(l - first);
       sum += ex;
-      if (lane == c) mine = ex, mine_e = be;
+      if (lane == c) mine = ex, mine_e = e;
     }
     if (lane < top_k) {
       idx_s[t * top_k + lane] = mine_e;
@@ -307,7 +282,7 @@ cudaError_t launch_batch_prep(const void *x, int M, int K, int bits, int group, 
 
 cudaError_t launch_batch_route(const float *logits, int m, int E, int top_k, int nt, int *idx, float *w,
                                BatchRoute *route, cudaStream_t s) {
-  if (m <= 0 || E <= 0 || E > 256 || top_k <= 0 || top_k > 16 || top_k > E || m * top_k > kRouteMaxSlots)
+  if (m <= 0 || E <= 0 || E > kMoeMaxExperts || top_k <= 0 || top_k > 16 || top_k > E || m * top_k > kRouteMaxSlots)
     return cudaErrorInvalidValue;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = batch_config(dim3(1), dim3(kRouteThreads), s, attr);

@@ -1,7 +1,8 @@
 // wq_route.cuh -- a token's experts by router logit, one warp: the larger logit
-// first, the lower expert index among equal ones.  Shared by the routing launch
-// and the gate/up launch over the slots, which finds its own expert so that it
-// need not wait for the former.
+// first, the lower expert index among equal ones.  A NaN ranks by its sign, above
+// every number or below, so the order is total.  Shared by the routing launches of
+// the slots and of the grouped experts, and by the gate/up launch over the slots,
+// which finds its own expert so that it need not wait for the former.
 #pragma once
 
 #include <cstdint>

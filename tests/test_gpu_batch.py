@@ -342,3 +342,31 @@ def test_routed_batch_of_two_ctas_an_sm(wq, m, k):
         assert ((ys[s] - y1[0]).abs() <= 1e-4 * y1.abs().max()).all(), s
     torch.cuda.synchronize()
     assert wq.device_status() == 0
+
+
+@pytest.mark.parametrize("E,k", [(8, 4), (33, 5)])
+def test_grouped_experts_rank_as_the_slots_do(wq, E, k):
+    """Enough slots that they are grouped: ties, signed zeros, extreme logits, and NaNs of
+    one token, of all of a token's logits and unselected ones.  The choices are those
+    of the slots' launches, and a NaN weight makes its own token NaN only."""
+    d, inter, group, m = 2048, 2048, 64, 24
+    n = lambda rows, cols, bits, s: wq.pack(torch.randn((rows, cols), device="cuda",
+                                                        generator=torch.Generator("cuda").manual_seed(s)) * 0.02, group, bits)
+    layer = wq.MoELayer(wq.MLPLayer(n(E * inter, d, 2, 1), n(E * inter, d, 2, 2), n(E * d, inter, 4, 3)), E, k)
+    x = synth.activations((m, d), 8).cuda()
+    lg = np.random.default_rng(E).integers(-3, 2, (m, E)).astype(np.float32)  # many ties
+    lg[:, ::3] *= -0.0
+    lg[0, E // 2], lg[0, -1], lg[0, 0] = 3e38, 1e-40, -3e38
+    nan = np.uint32(0x7FC00000).view(np.float32)
+    lg[5, 2], lg[9, :], lg[11, 1] = nan, nan, -nan
+    t = torch.from_numpy(lg).cuda()
+    y, idx, wt, _, _ = wq.moe_forward(x, t, layer, with_slots=True)
+    for i in range(m):
+        _, i1, w1, _, _ = wq.moe_forward(x[i:i + 1], t[i:i + 1].clone(), layer, with_slots=True)
+        assert torch.equal(idx[i], i1[0]) and torch.equal(wt[i].isnan(), w1[0].isnan()), i
+        e = idx[i].tolist()
+        assert len(set(e)) == k and min(e) >= 0 and max(e) < E, i
+    bad = torch.zeros(m, dtype=torch.bool, device="cuda")
+    bad[[5, 9]] = True
+    assert torch.equal(y.isnan().all(1), bad) and torch.equal(y.isnan().any(1), bad)
+    assert wq.device_status() == 0
