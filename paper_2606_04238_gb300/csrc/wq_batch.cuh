@@ -24,7 +24,10 @@
 //
 // The codes are private to a warp: it keeps D units in flight in its own
 // shared-memory ring with cp.async, issued before the wait on the previous
-// launch.  The activation records are shared by a set's warps, which take
+// launch.  That hides little between gate/up and down, whose CTAs do not fit on
+// an SM together (registers and shared memory): a CTA starts once the SM's last
+// one has left.  Beside an input launch, which leaves SMs free, the codes are
+// under way before it ends.  The activation records are shared by a set's warps, which take
 // turns at issuing their bulk copies LEAD rounds ahead, onto mbarriers
 // (bounded waits).
 //

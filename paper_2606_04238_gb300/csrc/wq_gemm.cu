@@ -543,7 +543,7 @@ struct GemmSmem {
 template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmArgs a, const __grid_constant__ GemmMaps tm) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
-  constexpr int SA = C::SA, SB = C::SB, R = C::R, GPB = C::GPB;
+  constexpr int SA = C::SA, SB = C::SB, R = C::R;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   GemmSmem<C> sm(smem_raw);
   uint8_t *smem = sm.base;
@@ -707,7 +707,7 @@ template <int BITS, int NPROJ, int GROUP, bool EXACT, bool TALL>
 __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_constant__ GemmArgs a,
                                                                    const __grid_constant__ GemmMaps tm) {
   using C = GemmCfg<BITS, NPROJ, GROUP, EXACT>;
-  constexpr int SA = C::SA, SB = C::SB, R = C::R, GPB = C::GPB;
+  constexpr int SA = C::SA, SB = C::SB, R = C::R;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   GemmSmem<C> sm(smem_raw);
   uint8_t *smem = sm.base;
@@ -1176,9 +1176,9 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 // Tensor maps of a launch (zero fill outside every tensor):
-//   activations [M][lda] binary16, boxes of 8 features x 128 tokens;
-//   codes [RT][KB * BPK / 128][128 B], boxes of one block of 8 row tiles;
-//   scales/zeros [RT][KB * GPB][64 B], boxes of one block of 8 row tiles.
+//   activations [M][lda] binary16, boxes of 64 features x 128 tokens;
+//   codes [RT][KB * BPK / 128][128 B], boxes of a 2-bit block or half a 4-bit one of 8 row tiles;
+//   scales/zeros [RT][KB * GPB][64 B], boxes of the groups that those codes have.
 cudaError_t make_maps(const GemmArgs &a, int nproj, int bits, GemmMaps *m) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
@@ -1372,20 +1372,6 @@ cudaError_t read_gemm_status(int *status) {
   e = cudaMemcpyToSymbol(g_gemm_status, &zero, sizeof(int));
   *status = v;
   return e;
-}
-
-int gemm_stages(GemvKind kind, int group) {
-  switch (kind * 3 + (group == 32 ? 0 : group == 64 ? 1 : 2)) {
-    case 0: return GemmCfg<2, 2, 32, false>::SA;
-    case 1: return GemmCfg<2, 2, 64, false>::SA;
-    case 2: return GemmCfg<2, 2, 128, false>::SA;
-    case 3: return GemmCfg<4, 2, 32, false>::SA;
-    case 4: return GemmCfg<4, 2, 64, false>::SA;
-    case 5: return GemmCfg<4, 2, 128, false>::SA;
-    case 6: return GemmCfg<4, 1, 32, false>::SA;
-    case 7: return GemmCfg<4, 1, 64, false>::SA;
-    default: return GemmCfg<4, 1, 128, false>::SA;
-  }
 }
 
 }  // namespace wq

@@ -130,7 +130,6 @@ cudaError_t launch_to_f16(const void *x, int M, int K, int lda16, uint16_t *x16,
 // Stream-K scratch a GEMM launch of this shape can need: fp32 partial sums
 // (num_sms: the device's SM count).
 size_t gemm_scratch_floats(int M, int N, int K, int nproj, int num_sms);
-int gemm_stages(GemvKind kind, int group);  // depth of the activation-tile ring
 // Reads and clears the GEMM kernels' device status word.
 cudaError_t read_gemm_status(int *status);
 
