@@ -163,6 +163,17 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
+def route_name(wq, m, layers, table):
+    """The kernels a stack of `layers` runs on at m tokens."""
+    info = wq.mlp_forward_info(m, layers, table=table)
+    if info["route"] == wq.ROUTE_STACK:
+        return "single-launch stack kernel"
+    # from 9 to 64 tokens both chains run the batched-decode kernels unless there is a GEMV plan
+    if info["route"] == wq.ROUTE_GEMV_CHAIN and info["gateup"]["ctas"] > 0:
+        return "GEMV launch chain"
+    return "batched-decode chain" if m <= 64 else "dequant-GEMM chain"
+
+
 # --------------------------------------------------------------------------- byte model
 def algorithmic_bytes(cfg, m, bits_gu=2, lora=True):
     """Bytes one decode step must move: packed codes, fp16 scales/zeros, LoRA
@@ -397,8 +408,7 @@ def run_gpu(args):
            "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
            "dtype": "w2/w4 codes x f16 mma, f32 accumulate, bf16 activations", "data": "synthetic",
            "config": stack_config(cfg, n_layers, m, ws_),
-           "route": ("launch chain", "dequant-GEMM chain", "single-launch stack kernel")[
-               wq.mlp_forward_info(m, layers, table=table)["route"]],
+           "route": route_name(wq, m, layers, table),
            "gpu_launches": launches_per_step * steps, "clocks": clocks, "e2e": e2e,
            "stack_gbs": n_layers * (gu_bytes + dn_bytes) / (ms_step / 1e3) / 1e9}
 
@@ -532,8 +542,7 @@ def run_sweep(wq, synth, dev, steps, warmup, sweep=SWEEP):
             gu, dn = algorithmic_bytes(cfg, m)
             gbs = cfg.layers * (gu + dn) / t_step / 1e9
             out["rows"].append({"config": name, "layers": cfg.layers, "m": m,
-                                "route": ("launch chain", "dequant-GEMM chain", "single-launch stack kernel")[
-                                    wq.mlp_forward_info(m, layers, table=table)["route"]],
+                                "route": route_name(wq, m, layers, table),
                                 "tokens_per_s": m / t_step,
                                 "us_per_step": t_step * 1e6, "us_per_layer": t_step * 1e6 / cfg.layers,
                                 "stack_gbs": gbs, "frac_of_hbm": gbs / peak, "clocks": clocks})
@@ -703,8 +712,7 @@ def run_quant_settings(wq, synth, dev, cfg, n_layers, m, x, y, ws, steps, warmup
         rows.append({"gate_up": f"W{bits} g{g}" + (" + LoRA r" + str(cfg.r) if lora else ""),
                      "tokens_per_s": m / t, "us_per_layer": t * 1e6 / n_layers, "gb_per_step": gb,
                      "frac_of_hbm": gb / t / peak,
-                     "route": ("launch chain", "dequant-GEMM chain", "single-launch stack kernel")[
-                         wq.mlp_forward_info(m, layers, table=table)["route"]]})
+                     "route": route_name(wq, m, layers, table)})
         del layers, table, gr
         torch.cuda.empty_cache()
     return {"workload": f"{cfg.name}_stack_{n_layers}L_m{m}", "down": f"W4 g{cfg.group_down}", "rows": rows}

@@ -2,7 +2,7 @@
 projection in BF16) as a stack through wq_mlp_forward: 2-bit gate/up with the
 adapters, the dense bf16 down, the residual stream in bf16.  Each layer is
 checked teacher-forced against the oracle (gate/up on the GPU's input, the
-bf16 down on the GPU's h), on the launch chain and on the GEMM chain, and a
+bf16 down on the GPU's h), on the launch chain and on the batched chain, and a
 stack that mixes 4-bit and bf16 down layers."""
 import numpy as np
 import pytest
@@ -51,7 +51,7 @@ def _check(wq, layers, ents, group, m, d, what):
     _, states, h_states = wq.mlp_forward_states(x, layers, prenorm=True, with_h=True)
     torch.cuda.synchronize()
     assert wq.device_status() == 0
-    exact = 0.97 if wq.mlp_forward_info(m, layers)["route"] != wq.ROUTE_GEMM_CHAIN else 0.6
+    exact = 0.97 if m <= 64 else 0.6  # exact products; binary16 weights above
     prev = synth.bf16_bits(x.cpu())
     for l, ent in enumerate(ents):
         h_ref, _ = orc.gateup(prev, ent["g"], ent["u"], group, ent["a"], ent["bg"], ent["bu"], lora_scale=2.0, prenorm=True)

@@ -105,7 +105,7 @@ def test_gemm_down_w4(wq, d, inter, group, m, residual):
 @pytest.mark.parametrize("m", [100, 300])
 def test_gemm_stack_matches_oracle(wq, m):
     """wq_mlp_forward above the decode limit: the GEMM chain (inputs kernel,
-    gate/up handing h in binary16 to down) vs the oracle, teacher-forced per
+    gate/up, the binary16 copy of h, down) vs the oracle, teacher-forced per
     layer through the single-layer calls, and end to end."""
     cfg = synth.CONFIGS["small_d256_i768"]
     n_layers = 3
@@ -169,10 +169,10 @@ def test_gemm_two_token_halves(wq, m):
     check_f32(y32, ref, f"GEMM y(f32) (two halves) m={m}")
 
 
-def test_planless_decode_shape_takes_gemm(wq):
+def test_planless_decode_shape_takes_batched(wq):
     """64 tokens of the 14B-shaped layer (d=5120, inter=17408): the decode
-    GEMV kernels have no launch configuration at this size, so the calls (and
-    the stack) take the dequant-GEMM path under the same results contract."""
+    GEMV kernels have no launch configuration at this size; the calls (and the
+    stack) take the batched-decode launches, exact products and fp32 sums."""
     cfg = synth.CONFIGS["dense_14b"]
     m = 64
     wg, wu, wd = synth.layer_weights(cfg, 0)
@@ -194,9 +194,9 @@ def test_planless_decode_shape_takes_gemm(wq):
     xb = synth.bf16_bits(x)
     ref_h, hb = orc.gateup(xb, qg, qu, cfg.group_gu, synth.bf16_bits(a), synth.bf16_bits(bg), synth.bf16_bits(bu),
                            lora_scale=cfg.lora_scale, prenorm=True)
-    check_bf16(h, ref_h, "14B gate/up m=64", min_exact=MIN_EXACT)
+    check_bf16(h, ref_h, "14B gate/up m=64")
     ref_y, _ = orc.down(synth.bf16_bits(h.cpu()), qd, cfg.group_down, xb)  # teacher-forced on the GPU's h
-    check_bf16(y, ref_y, "14B stack m=64", min_exact=MIN_EXACT)
+    check_bf16(y, ref_y, "14B stack m=64")
 
 
 @pytest.mark.parametrize("m", [65, 200])

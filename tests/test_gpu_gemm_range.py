@@ -1,11 +1,11 @@
-"""The batched dequant-GEMM path on activations far from unit scale.
+"""The batched-decode launches and the dequant-GEMM on activations far from unit scale.
 
-The tcgen05 path multiplies binary16 copies of the activations.  Each token
-is scaled by an exact power of two before the narrowing (its largest |x| put
-in [16, 32)) and the epilogue undoes it, so tokens of any magnitude keep the
-precision of unit-scale ones: here tokens span 1e-6 .. 1e5 (gate/up with
-and without the RMSNorm, down with bf16 and fp32 output; 24 tokens on the
-swapped-operand launch, 65 and 512 on the token-tile ones) and a stack
+Both multiply binary16 copies of the activations.  The tcgen05 path scales each
+token by an exact power of two before the narrowing (its largest |x| put in [16,
+32)), the batched-decode one each token's block of 128 features, and the epilogue
+undoes it, so tokens of any magnitude keep the precision of unit-scale ones: here
+tokens span 1e-6 .. 1e5 (gate/up with and without the RMSNorm, down with bf16 and
+fp32 output; 24 tokens on the batched-decode launches, 65 and 512 on tcgen05) and a stack
 without the RMSNorm whose h reaches ~1e6 (past the binary16 maximum 65504).
 Every token is checked against the oracle with its own bound.
 """
@@ -19,7 +19,9 @@ from tests.gpu_util import check_bf16, check_f32, upload_packed
 
 pytestmark = pytest.mark.gpu
 
-MIN_EXACT = 0.6  # the GEMM path's share of outputs equal to the oracle's own bf16 rounding
+# share of outputs equal to the oracle's own bf16 rounding: exact products to 64 tokens, binary16 weights above
+def _min_exact(m):
+    return 0.97 if m <= 64 else 0.6
 
 
 @pytest.fixture(scope="module")
@@ -42,12 +44,12 @@ def _wide(m, n, seed, lo=-6.0, hi=5.0):
     return (x * torch.pow(10.0, k)).to(torch.bfloat16)
 
 
-def _per_token(got, ref, what, min_exact=MIN_EXACT, f32=False):
+def _per_token(got, ref, what, f32=False):
     for i in range(ref.shape[0]):
         if f32:
             check_f32(got[i:i + 1], ref[i:i + 1], f"{what} token {i}")
         else:
-            check_bf16(got[i:i + 1], ref[i:i + 1], f"{what} token {i}", min_exact=min_exact)
+            check_bf16(got[i:i + 1], ref[i:i + 1], f"{what} token {i}", min_exact=_min_exact(ref.shape[0]))
 
 
 @pytest.mark.parametrize("m", [24, 65, 512])

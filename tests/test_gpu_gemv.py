@@ -4,7 +4,8 @@ MLP with 2-bit gate/up and 4-bit down), through the C ABI.
 Shapes span several row tiles and feature blocks, ragged row and feature
 tails, every supported group size and both panel modes (one CTA per row
 block, and split panels finished by the last-arriving CTA).  The GEMV kernels
-take 1..16 tokens; the 17/33/64-token cases here take the dequant-GEMM path.
+take small layers to 8 tokens (down matrices to 12 or 16); the cases of more
+tokens here take the batched-decode launches.
 """
 import numpy as np
 import pytest
@@ -80,9 +81,8 @@ def test_gateup_w2_lora(wq, d, inter, group, r, m, prenorm):
 
 @pytest.mark.parametrize("m", [17, 33, 64])
 def test_gateup_w2_many_tokens(wq, m):
-    """Above 16 tokens the call takes the dequant-GEMM path (weights rounded
-    once to binary16): the bound is unchanged, the share of outputs equal to
-    the oracle's own bf16 rounding is that path's (0.6)."""
+    """Above 8 tokens the call takes the batched-decode launches: exact products as
+    here, the same bound and share of outputs equal to the oracle's rounding."""
     d, inter, group, r = 512, 384, 64, 16
     L = _layer(d, inter, group, 64, r, seed=5)
     x = synth.activations((m, d), 7)
@@ -91,7 +91,7 @@ def test_gateup_w2_many_tokens(wq, m):
     h = wq.gateup_w2_lora(x.cuda(), g, u, a, bg, bu, lora_scale=2.0, prenorm=True)
     torch.cuda.synchronize()
     ref, _ = orc.gateup(synth.bf16_bits(x), L["g"], L["u"], group, *_orc_lora(L), lora_scale=2.0, prenorm=True)
-    check_bf16(h, ref, f"h m={m}", min_exact=0.6)
+    check_bf16(h, ref, f"h m={m}")
 
 
 @pytest.mark.parametrize("d,inter,group", [(256, 768, 64), (384, 200, 32), (512, 1000, 128)])

@@ -98,7 +98,7 @@ def test_merge_full_size_qwen3_4b_gate(wq):
 
 @pytest.mark.parametrize("m", [1, 8, 40])
 def test_merged_layer_forward(wq, m):
-    """A merged layer on the decode (m <= 16) and GEMM (m > 16) paths, r = 0,
+    """A merged layer on the GEMV kernels (1, 8 tokens) and the batched-decode ones, r = 0,
     vs the oracle's gate/up on the oracle's merged codes."""
     d, inter, group, r = 512, 1000, 128, 16
     rng = np.random.default_rng(77)
@@ -116,7 +116,7 @@ def test_merged_layer_forward(wq, m):
     gm = orc.quantize(orc.merge_lora(*g0, group, synth.bf16_bits(bg), synth.bf16_bits(a[:r]), 2.0), group, 2)[:3]
     um = orc.quantize(orc.merge_lora(*u0, group, synth.bf16_bits(bu), synth.bf16_bits(a[r:]), 2.0), group, 2)[:3]
     ref, _ = orc.gateup(synth.bf16_bits(x), gm, um, group, prenorm=True)
-    check_bf16(h, ref, f"merged h m={m}", min_exact=0.6 if m > 16 else 0.97)
+    check_bf16(h, ref, f"merged h m={m}")
 
 
 def test_merge_argument_errors(wq):

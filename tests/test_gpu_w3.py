@@ -5,7 +5,7 @@ The kernels read a 3-bit code as the 2-bit low plane plus one bit of the
 second plane shifted next to it, so a mistake in the plane layout, the shift
 or the mask shows as a wrong product.  Shapes: ragged rows and feature
 blocks, every group size (g32 is the paper's INT3 setting), 1..64 tokens
-(3-bit codes stay on the dequant-GEMV kernels at every token count), with
+(the GEMV kernels, above 8 tokens the batched-decode ones), with
 and without the RMSNorm and the adapter; a two-layer stack teacher-forced
 per layer; the Qwen3-4B shape at g32.
 """

@@ -78,8 +78,8 @@ def test_noalloc_rejects_a_layer_beyond_its_scratch():
 
 
 def test_noalloc_rejects_more_than_16_tokens():
-    """Above 16 tokens the workspace entry point takes the dequant-GEMM path;
-    the built-in scratch only serves the decode path, so the call refuses."""
+    """The built-in scratch only serves the GEMV kernels, whose limit here is 16
+    tokens, so the call refuses more."""
     import __graft_entry__
     __graft_entry__.build()
     from paper_2606_04238_gb300 import wq
