@@ -44,12 +44,12 @@ def _wide(m, n, seed, lo=-6.0, hi=5.0):
     return (x * torch.pow(10.0, k)).to(torch.bfloat16)
 
 
-def _per_token(got, ref, what, f32=False):
+def _per_token(got, ref, what, f32=False, min_exact=None):
     for i in range(ref.shape[0]):
         if f32:
             check_f32(got[i:i + 1], ref[i:i + 1], f"{what} token {i}")
         else:
-            check_bf16(got[i:i + 1], ref[i:i + 1], f"{what} token {i}", min_exact=_min_exact(ref.shape[0]))
+            check_bf16(got[i:i + 1], ref[i:i + 1], f"{what} token {i}", min_exact=min_exact or _min_exact(ref.shape[0]))
 
 
 @pytest.mark.parametrize("m", [24, 65, 512])
@@ -66,7 +66,9 @@ def test_gateup_wide_range(wq, m, prenorm):
     ref, _ = orc.gateup(synth.bf16_bits(x), qg, qu, group, synth.bf16_bits(a), synth.bf16_bits(bg),
                         synth.bf16_bits(bu), lora_scale=2.0, prenorm=prenorm)
     assert np.isfinite(h.float().cpu().numpy()).all()
-    _per_token(h, ref, f"gate/up m={m} prenorm={prenorm}")
+    # without the RMSNorm |g| reaches hundreds, and for negative g the relative error of
+    # h ~ e^g is g's absolute one: a hundred times that of a sum
+    _per_token(h, ref, f"gate/up m={m} prenorm={prenorm}", min_exact=None if prenorm or m > 64 else 0.9)
 
 
 @pytest.mark.parametrize("m", [24, 65, 512])
