@@ -675,13 +675,13 @@ __global__ void __launch_bounds__(BatchCfg<BITS, NPROJ, GROUP, NT, OCC>::NWARP *
       }
     }
   }
-  // no CTA ends with a copy into its shared memory in flight: one whose parts are
-  // all finished by others has not waited for the LoRA-A products and scales
   cp_async_wait_all();
   __syncwarp();
-  if (NPROJ == 2 && !ROUTED && warp == LEAD && elect_one() && !mbar_wait(aux, 0)) atomicExch(&g_batch_status, -6);
   // the records were waited for where they are used, unless a timeout came before
   if (*abort_s && elect_one() && issued >= 0) mbar_wait(&sfull[issued % RXR], (issued / RXR) & 1);
+  // no CTA ends with a copy into its shared memory in flight: one whose parts are
+  // all finished by others has not waited for the LoRA-A products and scales
+  if (NPROJ == 2 && !ROUTED && tid == 0 && !mbar_wait(aux, 0)) atomicExch(&g_batch_status, -6);
 }
 
 template <int BITS, int NPROJ, int GROUP, int NT, bool ROUTED = false, int OCC = 1>
