@@ -70,9 +70,10 @@ struct BatchCfg {
   // A group's scales and zero points applied two tokens an instruction: the
   // loop is short of issue slots (67 % used beside the MMAs).  us a layer, one
   // -> two tokens an instruction: d 4096 at 32 tokens 60.5 -> 57.4, with groups
-  // of 32 at 64 tokens 111 -> 105; only 4-bit codes in groups of 128 at 56
-  // tokens and more lose (d 4096 87.4 -> 89.3).
-  static constexpr bool PAIRED = !(BITS == 4 && GPB == 1 && NT == 8);
+  // of 32 at 64 tokens 111 -> 105; only 4-bit gate/up in groups of 128 at 56
+  // tokens and more loses (d 2560 W4 at 64 tokens 51.1 with one token in gate/up
+  // and two in down, 51.6 with one in both, 51.9 with two).
+  static constexpr bool PAIRED = !(BITS == 4 && GPB == 1 && NT == 8 && NPROJ == 2);
   // mma.sync truncates its sums: a down launch of up to 16 tokens adds a group of
   // 128 from two chains of 4, as the GEMV kernels that small matrices take do (d
   // 5120 x 17408 at 4 tokens of mean 0.5: error 1.6e-6 of the result with one
