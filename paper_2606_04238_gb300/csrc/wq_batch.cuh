@@ -32,9 +32,9 @@
 // (bounded waits).
 //
 // Measured (GB300, us a layer of an MLP stack at W2 g128, the swapped-operand
-// tcgen05 launch or the GEMV chain before -> this): d 4096 / inter 14336 at 9,
-// 24, 64 tokens 102.7 -> 39.6, 104.1 -> 47.3, 110.8 -> 87.5; d 2560 / inter
-// 9728 35.3 -> 26.5, 62.7 -> 30.8, 75.7 -> 51.3.  At 24 tokens of the d 4096
+// tcgen05 launch or the GEMV chain before -> this): d 4096 / inter 14336 at 16,
+// 24, 64 tokens 102.2 -> 39.1, 104.1 -> 47.6, 110.4 -> 88.8; d 2560 / inter 9728
+// at 16, 32, 64 47.2 -> 25.8, 61.9 -> 35.0, 74.5 -> 51.8.  At 24 tokens of the d 4096
 // shape a gate/up launch takes ~24 us, 15 of them in the main loop, which keeps
 // the mma.sync pipe (8 cycles an instruction) ~62 % busy; the rest is the
 // launch's start (~2 us), the exchange of split parts (~2 us) and the finish.

@@ -40,8 +40,8 @@
 // clocks where its MMAs need 1024, a tile ~4400 before its first MMA and ~7800
 // for its epilogue, half of them the 2 x 32768 exponentials and reciprocals.
 // Measured with 256-row down tiles, the reduction kernel, 3 B tiles and the
-// sector-wide stores: the d 5120 layer at 512 tokens 212 us, the d 2560 layer at
-// 3001 tokens 364 us.
+// sector-wide stores: the d 5120 layer at 512 tokens 209 us, the d 2560 layer at
+// 3001 tokens 357 us.
 // Stages are handed over with mbarriers; every wait is bounded (a timeout
 // sets the device status word and the CTA skips the rest of its work).
 #include <algorithm>
