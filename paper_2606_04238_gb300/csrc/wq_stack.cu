@@ -395,8 +395,6 @@ __global__ void __launch_bounds__(kSThreads, 1) stack_kernel(const __grid_consta
   }
   const unsigned long long base = base_s[0];
   unsigned long long gen = 0;
-  const int KBd = (a.inter + 127) / 128;
-  (void)KBd;
   const int nsg = (p.KBg + p.kps - 1) / p.kps;
   const int nsd = dn_stage_count(p, sh);
   int q = 0;  // stage sequence position
@@ -1035,7 +1033,8 @@ cudaError_t stack_layer_maps(const void *gate_codes, const void *up_codes, const
                              const void *down_codes, const void *down_meta, int d, int inter, int bits_gu, int group,
                              const StackPlan &p, CUtensorMap out[6]) {
   const uint64_t BPK = bits_gu == 2 ? 512 : 1024, GPB = 128 / group, GPH = group == 32 ? 2 : 1;
-  const uint64_t RTg = (uint64_t)inter / 16, KBg = (uint64_t)d / 128, RTd = (uint64_t)d / 16, KBd = (uint64_t)inter / 128;
+  const uint64_t RTg = (uint64_t)inter / 16, KBg = (uint64_t)d / 128, RTd = (uint64_t)d / 16;
+  const uint64_t KBd = ((uint64_t)inter + 127) / 128;  // the packed rows end with a whole block, also where inter does not
   const uint64_t NGd = KBd * 128 / group;
   cudaError_t e;
   if ((e = encode3(gate_codes, 128, KBg * BPK / 128, RTg, (uint32_t)(p.kps * BPK / 128), p.Tbox, &out[0])) != cudaSuccess ||

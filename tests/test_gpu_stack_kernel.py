@@ -105,6 +105,14 @@ def test_mid_stack_kernel_every_group(wq):
         _check(wq, layers, ents, group, 5, True, f"mid g{group}")
 
 
+@pytest.mark.parametrize("d,inter,group,r,m,bits", [(512, 704, 32, 16, 2, 2), (1024, 192, 64, 8, 7, 2),
+                                                    (256, 2496, 64, 0, 3, 4)])
+def test_stack_kernel_ragged_intermediate_size(wq, d, inter, group, r, m, bits):
+    # the down rows' last 128-feature block is half full
+    layers, ents = _layers(wq, d, inter, group, r, 2, bits_gu=bits, seed=13)
+    _check(wq, layers, ents, group, m, True, f"ragged inter={inter} g{group}")
+
+
 def test_stack_longer_than_one_launch(wq):
     # 70 layers: two launches (64 + 6), the second starting from the first's output
     layers, ents = _layers(wq, 256, 768, 64, 8, 70, seed=9)
