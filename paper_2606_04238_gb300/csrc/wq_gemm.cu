@@ -120,6 +120,14 @@ struct GemmCfg {
 
 __device__ __forceinline__ void gemm_timeout() { atomicExch(&g_gemm_status, -6); }
 
+// After a timeout, before the CTA ends: time for the loads and MMAs that its other
+// roles issued last (microseconds each) to end, so that none reaches shared memory
+// or TMEM that has changed hands.
+__device__ __noinline__ void gemm_settle() {
+  const unsigned long long t0 = global_timer_ns();
+  for (int i = 0; i < 1 << 20 && global_timer_ns() - t0 < 2000000ull; ++i) __nanosleep(1000);
+}
+
 // Byte offset of element (row, k) in a K-major no-swizzle tile whose 8-row
 // groups are `sbo` bytes apart (core matrices along K 128 bytes apart).
 __device__ __forceinline__ uint32_t kmajor_off(int row, int k, uint32_t sbo) {
@@ -643,6 +651,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_tile_kernel(const GemmA
     }
   }
 
+  if (*sm.abort_s) gemm_settle();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -853,6 +862,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) qgemm_sk_kernel(const __grid_
   }
 #undef WQ_FOR_EACH_PART
 
+  if (*sm.abort_s) gemm_settle();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

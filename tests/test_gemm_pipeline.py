@@ -135,3 +135,12 @@ def test_the_model_sees_the_missing_wait():
     with pytest.raises(AssertionError, match="another part"):
         for parts, slots, seed in schedules():
             run(parts, slots, False, seed)
+
+
+def test_a_timeout_settles_before_the_cta_ends():
+    """Both kernels: a CTA that met a timeout gives the loads and MMAs of its other roles
+    time to end before it frees its tensor memory and leaves."""
+    text = open(SRC).read()
+    ends = re.findall(r"  if \(\*sm\.abort_s\) gemm_settle\(\);\n  tc_fence_before\(\);\n  __syncthreads\(\);\n  tc_fence_after\(\);"
+                      r"\n  if \(warp == kMmaWarp\) tmem_dealloc\(tmem", text)
+    assert len(ends) == 2 and text.count("tmem_dealloc(tmem") == 2
